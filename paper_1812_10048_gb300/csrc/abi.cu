@@ -116,7 +116,7 @@ void free_ctx(Ctx& c) {
     c.h_chain0 = nullptr;
     if (c.lml) {
         void* lp[] = {c.lml->labels, c.lml->n, c.lml->S, c.lml->T, c.lml->common, c.lml->out,
-                      c.lml->grad, c.lml->beta_stage};
+                      c.lml->grad, c.lml->beta_stage, c.lml->part, c.lml->ticket};
         for (void* q : lp)
             if (q) cudaFree(q);
         delete c.lml;
@@ -1082,7 +1082,7 @@ int dpmm_debug_moves(dpmm_ctx* ctx, int32_t* chain, double* log_h, int32_t* pair
 
 static void free_lml(LmlPlan& p) {
     void* ptrs[] = {p.indptr, p.cols, p.counts, p.labels, p.n, p.S, p.T, p.common, p.out, p.grad,
-                    p.beta_stage};
+                    p.beta_stage, p.part, p.ticket};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (p.own_stream && p.stream) cudaStreamDestroy(p.stream);
@@ -1139,7 +1139,9 @@ int dpmm_logml_create(dpmm_logml** out, const int32_t* indptr, const int32_t* in
         (e = dalloc(&p.counts, (size_t)nnz)) || (e = dalloc(&p.labels, (size_t)N)) ||
         (e = dalloc(&p.n, (size_t)K)) || (e = dalloc(&p.S, (size_t)K * D)) ||
         (e = dalloc(&p.T, (size_t)K)) || (e = dalloc(&p.common, 1)) || (e = dalloc(&p.out, 2)) ||
-        (e = dalloc(&p.grad, (size_t)D)) || (e = dalloc(&p.beta_stage, (size_t)D)))
+        (e = dalloc(&p.grad, (size_t)D)) || (e = dalloc(&p.beta_stage, (size_t)D)) ||
+        (e = dalloc(&p.part, lml_part_count(D))) || (e = dalloc(&p.ticket, 1)) ||
+        (e = cudaMemsetAsync(p.ticket, 0, sizeof(int32_t), p.stream)))
         return bail(e, "cudaMalloc");
     if ((e = cudaMemcpy(p.indptr, hptr.data(), sizeof(int32_t) * (N + 1), cudaMemcpyHostToDevice)) ||
         (nnz && (e = cudaMemcpy(p.cols, hidx.data(), sizeof(int32_t) * nnz, cudaMemcpyHostToDevice))) ||
@@ -1177,7 +1179,7 @@ int dpmm_logml_forward(dpmm_logml* h, double log_alpha, const float* log_beta, d
     const float* lb;
     int rc = stage_beta(p, log_beta, &lb);
     if (rc) return rc;
-    CK(lml_forward(p, log_alpha, lb, p.out));
+    CK(lml_terms(p, log_alpha, lb, p.out, nullptr));
     CK(cudaMemcpyAsync(logml, p.out, sizeof(double), cudaMemcpyDefault, p.stream));
     if (!is_device_ptr(logml)) CK(cudaStreamSynchronize(p.stream));
     return DPMM_OK;
@@ -1191,7 +1193,8 @@ int dpmm_logml_backward(dpmm_logml* h, double log_alpha, const float* log_beta,
     int rc = stage_beta(p, log_beta, &lb);
     if (rc) return rc;
     const bool dev_out = is_device_ptr(grad_log_beta);
-    CK(lml_backward(p, log_alpha, lb, dev_out ? grad_log_beta : p.grad, p.out + 1));
+    CK(lml_terms(p, log_alpha, lb, nullptr, p.out + 1));
+    CK(lml_backward(p, lb, dev_out ? grad_log_beta : p.grad));
     if (!dev_out)
         CK(cudaMemcpyAsync(grad_log_beta, p.grad, sizeof(float) * p.D, cudaMemcpyDeviceToHost,
                            p.stream));
@@ -1227,7 +1230,9 @@ int dpmm_logml_grad(dpmm_ctx* ctx, const int32_t* labels, int32_t K_labels, doub
         if ((e = dalloc(&p->labels, (size_t)c.N)) || (e = dalloc(&p->n, (size_t)c.kmax)) ||
             (e = dalloc(&p->S, (size_t)c.kmax * c.D)) || (e = dalloc(&p->T, (size_t)c.kmax)) ||
             (e = dalloc(&p->common, 1)) || (e = dalloc(&p->out, 2)) ||
-            (e = dalloc(&p->grad, (size_t)c.D)) || (e = dalloc(&p->beta_stage, (size_t)c.D))) {
+            (e = dalloc(&p->grad, (size_t)c.D)) || (e = dalloc(&p->beta_stage, (size_t)c.D)) ||
+            (e = dalloc(&p->part, lml_part_count(c.D))) || (e = dalloc(&p->ticket, 1)) ||
+            (e = cudaMemsetAsync(p->ticket, 0, sizeof(int32_t), c.stream))) {
             p->own_stream = false;
             free_lml(*p);
             delete p;
@@ -1253,13 +1258,13 @@ int dpmm_logml_grad(dpmm_ctx* ctx, const int32_t* labels, int32_t K_labels, doub
     }
     const float* lb;
     if ((rc = stage_beta(p, log_beta, &lb))) return rc;
-    if (logml) {
-        CK(lml_forward(p, log_alpha, lb, p.out));
-        CK(cudaMemcpyAsync(logml, p.out, sizeof(double), cudaMemcpyDefault, c.stream));
-    }
-    if (grad_log_alpha || grad_log_beta) {
+    const bool grads = grad_log_alpha || grad_log_beta;
+    if (logml || grads)
+        CK(lml_terms(p, log_alpha, lb, logml ? p.out : nullptr, grads ? p.out + 1 : nullptr));
+    if (logml) CK(cudaMemcpyAsync(logml, p.out, sizeof(double), cudaMemcpyDefault, c.stream));
+    if (grads) {
         const bool dev_out = grad_log_beta && is_device_ptr(grad_log_beta);
-        CK(lml_backward(p, log_alpha, lb, dev_out ? grad_log_beta : p.grad, p.out + 1));
+        if (grad_log_beta) CK(lml_backward(p, lb, dev_out ? grad_log_beta : p.grad));
         if (grad_log_beta && !dev_out)
             CK(cudaMemcpyAsync(grad_log_beta, p.grad, sizeof(float) * c.D,
                                cudaMemcpyDeviceToHost, c.stream));

@@ -303,7 +303,7 @@ __device__ __forceinline__ float log_gamma_draw(const Stream& st, uint32_t tag, 
 // then the asymptotic series ln x - 1/(2x) - 1/(12x^2) + 1/(120x^4)
 // - 1/(252x^6) + 1/(240x^8) (Abramowitz & Stegun 6.3.5, 6.3.18).
 template <typename T>
-__device__ __forceinline__ T digamma(T x) {
+__host__ __device__ __forceinline__ T digamma(T x) {
     T acc = 0;
     while (x < T(6)) {
         acc -= T(1) / x;

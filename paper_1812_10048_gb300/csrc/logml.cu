@@ -2,144 +2,172 @@
 // respect to log alpha and a gene-wise log beta (theta integrated out of
 // eq. 12 against eq. 28 with lambda generalised to beta_u, pi out of eq. 10).
 //
-//   k_lml_stats     n_k, S_ku of the labelled cells (integer, exact); for a
-//                   sampler's chain (dpmm_logml_grad) k_lml_from_chain sums
-//                   its sub-cluster statistics and k_lml_csr_stats counts
-//                   given labels from its packed CSR
-//   k_lml_forward   FP64, blocks (cluster, 256 genes): lgamma(n_k) + lgamma(B) - lgamma(B + T_k)
-//                   + sum_{u: S_ku > 0} [lgamma(beta_u + S_ku) - lgamma(beta_u)];
-//                   one extra block adds K log alpha + lgamma(alpha) - lgamma(alpha + N)
-//   k_lml_common    B = sum beta_u; c = sum_k [psi(B) - psi(B + T_k)];
+//   k_lml_stats     (logml_stats.cuh) n_k, S_ku, T_k of the labelled cells
+//                   (integer, exact); for a sampler's chain (dpmm_logml_grad)
+//                   k_lml_from_chain sums its sub-cluster statistics
+//   k_lml_terms     FP64, blocks of kLmlGenes genes: the gene terms
+//                   sum_{u, k: S_ku > 0} [lgamma(beta_u + S_ku) - lgamma(beta_u)]
+//                   and B = sum beta_u; the last block adds the cluster terms
+//                   lgamma(n_k) + lgamma(B) - lgamma(B + T_k) and the partition
+//                   terms (from the host), and for the gradient forms
+//                   c = sum_k [psi(B) - psi(B + T_k)] and
 //                   d/d log alpha = K + alpha (psi(alpha) - psi(alpha + N))
-//   k_lml_backward  FP32: beta_u (c + sum_{k: S_ku > 0} [psi(beta_u + S_ku) - psi(beta_u)])
+//   k_lml_backward  beta_u (c + sum_{k: S_ku > 0} [psi(beta_u + S_ku) - psi(beta_u)]),
+//                   FP32 digammas summed in FP64
 #include <math_constants.h>
 
+#include <cmath>
+
 #include "logml.cuh"
+#include "logml_stats.cuh"
 
 namespace dpmm {
 
-constexpr int kLmlThreads = 256;
+constexpr int kLmlGenes = 8;      // genes per block
+constexpr int kLmlLanes = 32;     // threads per gene, each every 32nd cluster
+constexpr int kLmlThreads = kLmlGenes * kLmlLanes;
+constexpr int kLmlChainThreads = 256;
 
-__global__ void k_lml_stats(const int32_t* __restrict__ indptr, const int32_t* __restrict__ cols,
-                            const int32_t* __restrict__ counts, const int32_t* __restrict__ labels,
-                            int64_t N, int32_t D, int32_t K, uint32_t* __restrict__ n,
-                            uint32_t* __restrict__ S, unsigned long long* __restrict__ T) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t cell = w0; cell < N; cell += nw) {
-        const int32_t k = labels[cell];
-        if (k < 0 || k >= K) continue;
-        const int64_t beg = indptr[cell], end = indptr[cell + 1];
-        unsigned long long rowsum = 0;
-        for (int64_t e = beg + lane; e < end; e += 32) {
-            const int32_t x = counts[e];
-            if (x) {
-                atomicAdd(&S[(size_t)k * D + cols[e]], (uint32_t)x);
-                rowsum += (unsigned long long)x;
+// Block sums of M values at once (every thread gets them); red: 32 M doubles.
+template <int M>
+__device__ __forceinline__ void block_sums(double (&v)[M], double* red) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+#pragma unroll
+        for (int m = 0; m < M; ++m) v[m] += __shfl_xor_sync(0xFFFFFFFFu, v[m], o);
+    __syncthreads();
+    if (l == 0)
+#pragma unroll
+        for (int m = 0; m < M; ++m) red[32 * m + w] = v[m];
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < M; ++m) v[m] = l < nw ? red[32 * m + l] : 0.0;
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+        if (o < nw)
+#pragma unroll
+            for (int m = 0; m < M; ++m) v[m] += __shfl_xor_sync(0xFFFFFFFFu, v[m], o);
+#pragma unroll
+    for (int m = 0; m < M; ++m) v[m] = __shfl_sync(0xFFFFFFFFu, v[m], 0);
+}
+
+// Block g: genes 8 g .. 8 g + 7, 32 threads a gene (every 32nd cluster each).
+// GB300 issues 1.7 FP64 operations per SM and cycle, 65 cycles deep (measured;
+// a library lgamma takes about 2,400 cycles alone and 20 cycles per thread of
+// a full SM), so the cost is the number of FP64 operations, how evenly they
+// lie on the SMs and how many follow one another: a term is one lgamma;
+// exp(log beta_u) and lgamma(beta_u) are taken once per gene, beside the
+// terms, instead of once per term; B is summed by all blocks (the exponentials
+// of 2,000 genes on one SM took 23 us); the last block to finish adds the
+// cluster terms, one lgamma per thread.  100,000 x 2,000 with K = 25 (ncu,
+// cold): value and gradients 93 -> 34 us.  The per-block sums are added in block order,
+// so the value is the same in every run.
+// value: the log ML itself; grad: c and d/d log alpha.  part_value, part_grad:
+// lgamma(alpha) - lgamma(alpha + N), alpha (psi(alpha) - psi(alpha + N)).
+__global__ void __launch_bounds__(kLmlThreads)
+k_lml_terms(const uint32_t* __restrict__ n, const uint32_t* __restrict__ S,
+            const unsigned long long* __restrict__ T, const float* __restrict__ log_beta,
+            int32_t D, int32_t K, double log_alpha, double part_value, double part_grad,
+            int32_t value, int32_t grad, double* part, int32_t* ticket, double* __restrict__ out,
+            double* __restrict__ grad_alpha, double* __restrict__ common, uint32_t* wrap_flag) {
+    __shared__ double red[3 * 32];
+    __shared__ double sb[kLmlGenes], slg[kLmlGenes], slgB;
+    __shared__ int last;
+    const int j = threadIdx.x % kLmlGenes, q = threadIdx.x / kLmlGenes;
+    const int u = blockIdx.x * kLmlGenes + j;
+    if (q == 0) sb[j] = u < D ? exp((double)log_beta[u]) : 0.0;
+    __syncthreads();
+    double acc[1] = {0.0};
+    if (value) {
+        const double b = sb[j];
+        int terms = 0;
+        if (u < D) {
+            for (int k = q; k < K; k += kLmlLanes) {
+                const uint32_t s = S[(size_t)k * D + u];
+                if (s) {
+                    acc[0] += lgamma(b + (double)s);
+                    ++terms;
+                }
             }
+            // (the last warp, with the fewest clusters, takes lgamma(beta_u) as well)
+            if (q == kLmlLanes - 1) slg[j] = lgamma(b);
         }
-        rowsum = warp_sum(rowsum);
-        if (lane == 0) {
-            atomicAdd(&n[k], 1u);
-            if (rowsum) atomicAdd(&T[k], rowsum);
-        }
+        __syncthreads();
+        if (terms) acc[0] -= (double)terms * slg[j];
+        block_sums(acc, red);
     }
-}
-
-__device__ __forceinline__ double block_sum_lml(double v, double* red) {
-    v = warp_sum(v);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += red[i];
-    return r;
-}
-
-__global__ void __launch_bounds__(kLmlThreads)
-k_lml_forward(const uint32_t* __restrict__ n, const uint32_t* __restrict__ S,
-              const unsigned long long* __restrict__ T, const float* __restrict__ log_beta,
-              int64_t N, int32_t D, int32_t K, double log_alpha, double* __restrict__ out) {
-    // block (k, g): the gene terms of cluster k over genes [256 g, 256 g + 256);
-    // blocks (k, 0) also add cluster k's count and total terms, block (K, 0)
-    // the partition terms.  GB300's FP64 rate makes the lgamma calls the cost,
-    // so they are spread over K x D / 256 blocks.
-    __shared__ double red[32];
-    const int k = blockIdx.x, g = blockIdx.y;
-    if (k == K) {
-        if (g != 0) return;
-        double keff = 0.0;
-        for (int j = threadIdx.x; j < K; j += blockDim.x) keff += n[j] ? 1.0 : 0.0;
-        keff = block_sum_lml(keff, red);
-        if (threadIdx.x == 0) {
-            const double alpha = exp(log_alpha);
-            atomicAdd(out, keff * log_alpha + lgamma(alpha) - lgamma(alpha + (double)N));
-        }
-        return;
-    }
-    if (n[k] == 0) return;
-    const uint32_t* Sk = S + (size_t)k * D;
-    double acc = 0.0;
-    const int u = g * blockDim.x + threadIdx.x;
-    if (u < D) {
-        const uint32_t s = Sk[u];
-        if (s) {
-            const double b = exp((double)log_beta[u]);
-            acc = lgamma(b + (double)s) - lgamma(b);
-        }
-    }
-    if (g == 0) {
-        double B = 0.0;
-        for (int v = threadIdx.x; v < D; v += blockDim.x) B += exp((double)log_beta[v]);
-        B = block_sum_lml(B, red);
-        if (threadIdx.x == 0) acc += lgamma((double)n[k]) + lgamma(B) - lgamma(B + (double)T[k]);
-    }
-    acc = block_sum_lml(acc, red);
-    if (threadIdx.x == 0) atomicAdd(out, acc);
-}
-
-__global__ void __launch_bounds__(kLmlThreads)
-k_lml_common(const uint32_t* __restrict__ n, const unsigned long long* __restrict__ T,
-             const float* __restrict__ log_beta, int64_t N, int32_t D, int32_t K,
-             double log_alpha, float* __restrict__ common, double* __restrict__ grad_alpha) {
-    __shared__ double red[32];
-    double B = 0.0;
-    for (int u = threadIdx.x; u < D; u += blockDim.x) B += exp((double)log_beta[u]);
-    B = block_sum_lml(B, red);
-    const float Bf = (float)B;
-    const float psiB = digamma<float>(Bf);
-    double c = 0.0, keff = 0.0;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        if (n[k]) {
-            c += (double)(psiB - digamma<float>(Bf + (float)T[k]));
-            keff += 1.0;
-        }
-    }
-    c = block_sum_lml(c, red);
-    keff = block_sum_lml(keff, red);
     if (threadIdx.x == 0) {
-        *common = (float)c;
-        const double alpha = exp(log_alpha);
-        *grad_alpha = keff + alpha * (digamma<double>(alpha) - digamma<double>(alpha + (double)N));
+        double sum = 0.0;
+        for (int i = 0; i < kLmlGenes; ++i) sum += sb[i];
+        part[2 * (size_t)blockIdx.x] = acc[0];
+        part[2 * (size_t)blockIdx.x + 1] = sum;
+        __threadfence();
+        last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *ticket = 0;
+    double ab[2] = {0.0, 0.0};
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+        ab[0] += __ldcg(part + 2 * (size_t)i);
+        ab[1] += __ldcg(part + 2 * (size_t)i + 1);
+    }
+    block_sums(ab, red);
+    const double B = ab[1];
+    // items 0 .. K - 1: lgamma(n_k) and c's term; K .. 2K - 1: lgamma(B + T_k);
+    // 2K: lgamma(B), once per cluster
+    const float Bf = (float)B;
+    const float psiB = grad ? digamma<float>(Bf) : 0.0f;
+    double t[3] = {0.0, 0.0, 0.0};   // value, c, clusters
+    for (int i = threadIdx.x; i < 2 * K + 1; i += blockDim.x) {
+        if (i == 2 * K) {
+            slgB = value ? lgamma(B) : 0.0;
+        } else if (i >= K) {
+            if (value && n[i - K]) t[0] -= lgamma(B + (double)T[i - K]);
+        } else if (n[i]) {
+            t[2] += 1.0;
+            if (wrap_flag && (T[i] >> 32)) atomicOr(wrap_flag, kLmlWrapFlag);
+            if (value) t[0] += lgamma((double)n[i]);
+            if (grad) t[1] += (double)(psiB - digamma<float>(Bf + (float)T[i]));
+        }
+    }
+    block_sums(t, red);
+    if (threadIdx.x == 0) {
+        if (value) *out = ab[0] + (t[0] + t[2] * slgB) + (t[2] * log_alpha + part_value);
+        if (grad) {
+            *common = t[1];
+            *grad_alpha = t[2] + part_grad;
+        }
     }
 }
 
+// Threads as in k_lml_terms.  The digammas are FP32, their sum over the
+// clusters FP64 (the terms cancel against c).
 __global__ void __launch_bounds__(kLmlThreads)
-k_lml_backward(const uint32_t* __restrict__ n, const uint32_t* __restrict__ S,
-               const float* __restrict__ log_beta, int32_t D, int32_t K,
-               const float* __restrict__ common, float* __restrict__ grad) {
-    const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= D) return;
-    const float b = expf(log_beta[u]);
-    const float psib = digamma<float>(b);
-    float acc = *common;
-    for (int k = 0; k < K; ++k) {
-        const uint32_t s = S[(size_t)k * D + u];
-        if (s && n[k]) acc += digamma<float>(b + (float)s) - psib;
+k_lml_backward(const uint32_t* __restrict__ S, const float* log_beta, int32_t D, int32_t K,
+               const double* __restrict__ common, float* grad) {
+    __shared__ double sacc[kLmlLanes][kLmlGenes];
+    const int j = threadIdx.x % kLmlGenes, q = threadIdx.x / kLmlGenes;
+    const int u = blockIdx.x * kLmlGenes + j;
+    double acc = 0.0;
+    float b = 0.0f;
+    if (u < D) {
+        b = expf(log_beta[u]);
+        const float psib = digamma<float>(b);
+        for (int k = q; k < K; k += kLmlLanes) {
+            const uint32_t s = S[(size_t)k * D + u];
+            if (s) acc += (double)(digamma<float>(b + (float)s) - psib);
+        }
     }
-    grad[u] = b * acc;
+    sacc[q][j] = acc;
+    __syncthreads();
+    if (q == 0 && u < D) {
+        acc = *common;
+        for (int i = 0; i < kLmlLanes; ++i) acc += sacc[i][j];
+        grad[u] = (float)((double)b * acc);
+    }
 }
 
 // Cluster statistics of a sampler's current state from its sub-cluster
@@ -170,10 +198,12 @@ __global__ void k_lml_from_chain(const uint32_t* __restrict__ nsub,
     }
 }
 
-// Cluster statistics of given labels over a sampler's own CSR copy.
-__global__ void k_lml_csr_stats(Csr csr, const int32_t* __restrict__ labels, int64_t N,
-                                int32_t D, int32_t K, uint32_t* __restrict__ n,
-                                uint32_t* __restrict__ S, unsigned long long* __restrict__ T) {
+// n_k, S_ku, T_k with the additions in global memory: for clusters whose counters
+// fit no shared memory (see logml_stats.cuh).
+template <class Rows>
+__global__ void k_lml_stats_global(Rows csr, const int32_t* __restrict__ labels, int64_t N,
+                                   int32_t D, int32_t K, uint32_t* __restrict__ n,
+                                   uint32_t* __restrict__ S, unsigned long long* __restrict__ T) {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -199,45 +229,49 @@ __global__ void k_lml_csr_stats(Csr csr, const int32_t* __restrict__ labels, int
 }
 
 cudaError_t lml_stats_from_chain(LmlPlan& p, const uint32_t* nsub, const uint32_t* Ssub) {
-    k_lml_from_chain<<<p.K, kLmlThreads, 0, p.stream>>>(nsub, Ssub, p.D, p.n, p.S, p.T);
+    k_lml_from_chain<<<p.K, kLmlChainThreads, 0, p.stream>>>(nsub, Ssub, p.D, p.n, p.S, p.T);
     return cudaGetLastError();
 }
 
-cudaError_t lml_stats_from_csr(LmlPlan& p, const Csr& csr, const int32_t* labels) {
+namespace {
+
+template <class Rows>
+cudaError_t lml_count(LmlPlan& p, const Rows& rows, const int32_t* labels) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(p.n, 0, sizeof(uint32_t) * p.K, p.stream))) return e;
     if ((e = cudaMemsetAsync(p.S, 0, sizeof(uint32_t) * (size_t)p.K * p.D, p.stream))) return e;
     if ((e = cudaMemsetAsync(p.T, 0, sizeof(unsigned long long) * p.K, p.stream))) return e;
-    k_lml_csr_stats<<<p.num_sms * 4, 256, 0, p.stream>>>(csr, labels, p.N, p.D, p.K, p.n, p.S,
-                                                         p.T);
+    if ((e = lml_launch_stats<false>(p, rows, labels, nullptr)) != cudaErrorNotSupported) return e;
+    k_lml_stats_global<<<p.num_sms * 4, 256, 0, p.stream>>>(rows, labels, p.N, p.D, p.K, p.n, p.S,
+                                                            p.T);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t lml_stats_from_csr(LmlPlan& p, const Csr& csr, const int32_t* labels) {
+    return lml_count(p, csr, labels);
 }
 
 cudaError_t lml_compute_stats(LmlPlan& p) {
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(p.n, 0, sizeof(uint32_t) * p.K, p.stream))) return e;
-    if ((e = cudaMemsetAsync(p.S, 0, sizeof(uint32_t) * (size_t)p.K * p.D, p.stream))) return e;
-    if ((e = cudaMemsetAsync(p.T, 0, sizeof(unsigned long long) * p.K, p.stream))) return e;
-    k_lml_stats<<<p.num_sms * 4, 256, 0, p.stream>>>(p.indptr, p.cols, p.counts, p.labels, p.N,
-                                                      p.D, p.K, p.n, p.S, p.T);
+    return lml_count(p, PlainCsr{p.indptr, p.cols, p.counts}, p.labels);
+}
+
+size_t lml_part_count(int32_t D) { return 2 * (size_t)((D + kLmlGenes - 1) / kLmlGenes); }
+
+cudaError_t lml_terms(LmlPlan& p, double log_alpha, const float* log_beta, double* value_dev,
+                      double* grad_alpha_dev, uint32_t* wrap_flag) {
+    const double alpha = std::exp(log_alpha), an = alpha + (double)p.N;
+    k_lml_terms<<<(p.D + kLmlGenes - 1) / kLmlGenes, kLmlThreads, 0, p.stream>>>(
+        p.n, p.S, p.T, log_beta, p.D, p.K, log_alpha, std::lgamma(alpha) - std::lgamma(an),
+        alpha * (digamma(alpha) - digamma(an)), value_dev != nullptr, grad_alpha_dev != nullptr,
+        p.part, p.ticket, value_dev, grad_alpha_dev, p.common, wrap_flag);
     return cudaGetLastError();
 }
 
-cudaError_t lml_forward(LmlPlan& p, double log_alpha, const float* log_beta, double* out_dev) {
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(out_dev, 0, sizeof(double), p.stream))) return e;
-    const dim3 grid(p.K + 1, (p.D + kLmlThreads - 1) / kLmlThreads);
-    k_lml_forward<<<grid, kLmlThreads, 0, p.stream>>>(p.n, p.S, p.T, log_beta, p.N, p.D, p.K,
-                                                      log_alpha, out_dev);
-    return cudaGetLastError();
-}
-
-cudaError_t lml_backward(LmlPlan& p, double log_alpha, const float* log_beta, float* grad_dev,
-                         double* grad_alpha_dev) {
-    k_lml_common<<<1, kLmlThreads, 0, p.stream>>>(p.n, p.T, log_beta, p.N, p.D, p.K, log_alpha,
-                                                  p.common, grad_alpha_dev);
-    k_lml_backward<<<(p.D + kLmlThreads - 1) / kLmlThreads, kLmlThreads, 0, p.stream>>>(
-        p.n, p.S, log_beta, p.D, p.K, p.common, grad_dev);
+cudaError_t lml_backward(LmlPlan& p, const float* log_beta, float* grad_dev) {
+    k_lml_backward<<<(p.D + kLmlGenes - 1) / kLmlGenes, kLmlThreads, 0, p.stream>>>(
+        p.S, log_beta, p.D, p.K, p.common, grad_dev);
     return cudaGetLastError();
 }
 

@@ -17,7 +17,7 @@
 // calling concurrently) race on the array and must be serialised by the caller.
 #include <mutex>
 
-#include "logml.cuh"
+#include "logml_stats.cuh"
 
 namespace dpmm {
 int noalloc_fail(int code, const char* msg);
@@ -32,16 +32,29 @@ constexpr int32_t kMaxK = 1024;
 constexpr int32_t kMaxD = 65536;
 constexpr int kMaxDevices = 64;
 
-// Byte layout of the scratch array (every piece 256-byte aligned).
-constexpr size_t kOffS = 0;                                     // uint32[kMaxKD]
-constexpr size_t kOffN = kOffS + sizeof(uint32_t) * kMaxKD;     // uint32[kMaxK]
+// Byte layout of the scratch array (every piece 256-byte aligned).  What each
+// call clears lies together at its start (n, T, the flag, the ticket, then the
+// K * D words of S in use), what it returns to the host lies together too
+// (logml, d/d log alpha, the flag).
+constexpr size_t kOffN = 0;                                     // uint32[kMaxK]
 constexpr size_t kOffT = kOffN + sizeof(uint32_t) * kMaxK;      // uint64[kMaxK]
-constexpr size_t kOffOut = kOffT + sizeof(uint64_t) * kMaxK;    // double[2]
-constexpr size_t kOffCommon = kOffOut + 256;                    // float
-constexpr size_t kOffFlag = kOffCommon + 256;                   // uint32
-constexpr size_t kOffBeta = kOffFlag + 256;                     // float[kMaxD]
+constexpr size_t kOffOut = kOffT + sizeof(uint64_t) * kMaxK;    // double[2], then the flag
+constexpr size_t kOffFlag = kOffOut + 16;                       // uint32
+constexpr size_t kOffTicket = kOffOut + 128;                    // int32
+constexpr size_t kOffCommon = kOffOut + 192;                    // double
+constexpr size_t kOffS = kOffOut + 256;                         // uint32[kMaxKD]
+constexpr size_t kOffBeta = kOffS + sizeof(uint32_t) * kMaxKD;  // float[kMaxD]
 constexpr size_t kOffGrad = kOffBeta + sizeof(float) * kMaxD;   // float[kMaxD]
-constexpr size_t kScratchBytes = kOffGrad + sizeof(float) * kMaxD;
+constexpr size_t kOffPart = kOffGrad + sizeof(float) * kMaxD;   // double[kMaxD / 4]
+constexpr size_t kScratchBytes = kOffPart + sizeof(double) * (kMaxD / 4);
+
+// What a call reads back in one copy.
+struct NoallocResult {
+    double logml, grad_log_alpha;
+    uint32_t flag;
+    uint32_t pad;
+};
+static_assert(sizeof(NoallocResult) == 24 && kOffFlag == kOffOut + 16, "result layout");
 
 }  // namespace
 
@@ -79,8 +92,10 @@ bool on_device(const void* p, int dev) {
            a.type == cudaMemoryTypeManaged;
 }
 
-// n_k, S_ku, T_k of the labelled cells, like k_lml_stats, but the arrays come
-// from a caller that was not validated on the host: rows with a decreasing
+// n_k, S_ku, T_k of the labelled cells with the additions in global memory, for
+// clusters whose counters do not fit shared memory and for totals that could
+// reach 2^32 (k_lml_stats, logml_stats.cuh, counts the others).  The arrays
+// come from a caller that was not validated on the host: rows with a decreasing
 // indptr or one beyond indptr[N], columns outside [0, D), negative counts and
 // labels outside [0, K) are skipped and reported in *flag (bit 0: row or
 // label, bit 1: entry); a gene total S_ku that wraps 2^32 sets bit 2.
@@ -123,6 +138,22 @@ __global__ void k_lml_stats_checked(const int32_t* __restrict__ indptr,
             if (rowsum) atomicAdd(&T[k], rowsum);
         }
     }
+}
+
+// A result into the caller's memory, host or device (no host copy is queued
+// for host memory).
+cudaError_t give(double* dst, const double* v, cudaStream_t st) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, dst) != cudaSuccess) {
+        cudaGetLastError();
+        a.type = cudaMemoryTypeUnregistered;
+    }
+    if (a.type != cudaMemoryTypeDevice) {
+        *dst = *v;
+        return cudaSuccess;
+    }
+    cudaError_t e = cudaMemcpyAsync(dst, v, sizeof(double), cudaMemcpyHostToDevice, st);
+    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
 }
 
 }  // namespace
@@ -168,39 +199,57 @@ extern "C" int dpmm_logml_grad_noalloc(const int32_t* indptr, const int32_t* ind
     p.n = reinterpret_cast<uint32_t*>(base + kOffN);
     p.T = reinterpret_cast<unsigned long long*>(base + kOffT);
     p.out = reinterpret_cast<double*>(base + kOffOut);
-    p.common = reinterpret_cast<float*>(base + kOffCommon);
+    p.common = reinterpret_cast<double*>(base + kOffCommon);
     p.beta_stage = reinterpret_cast<float*>(base + kOffBeta);
     p.grad = reinterpret_cast<float*>(base + kOffGrad);
     uint32_t* flag = reinterpret_cast<uint32_t*>(base + kOffFlag);
 
-    // clear what must start at zero: statistics and the error flag
-    if (!e) e = cudaMemsetAsync(p.S, 0, sizeof(uint32_t) * (size_t)K * D, p.stream);
-    if (!e) e = cudaMemsetAsync(p.n, 0, sizeof(uint32_t) * K, p.stream);
-    if (!e) e = cudaMemsetAsync(p.T, 0, sizeof(unsigned long long) * K, p.stream);
-    if (!e) e = cudaMemsetAsync(flag, 0, sizeof(uint32_t), p.stream);
-    if (!e) e = cudaMemcpyAsync(p.beta_stage, log_beta, sizeof(float) * D, cudaMemcpyDefault,
-                                p.stream);
+    p.part = reinterpret_cast<double*>(base + kOffPart);
+    p.ticket = reinterpret_cast<int32_t*>(base + kOffTicket);
+    // log_beta and grad_log_beta on this device are used where they are, unless
+    // they overlap
+    const float* lb = p.beta_stage;
+    float* grad = p.grad;
     if (!e) {
-        k_lml_stats_checked<<<p.num_sms * 4, 256, 0, p.stream>>>(p.indptr, p.cols, p.counts,
-                                                               p.labels, N, D, K, p.n, p.S, p.T,
-                                                               flag);
-        e = cudaGetLastError();
+        if (on_device(grad_log_beta, dev)) grad = grad_log_beta;
+        const bool apart = log_beta + D <= grad_log_beta || grad_log_beta + D <= log_beta;
+        if (apart && on_device(log_beta, dev)) lb = log_beta;
+        else
+            e = cudaMemcpyAsync(p.beta_stage, log_beta, sizeof(float) * D, cudaMemcpyDefault,
+                                p.stream);
     }
-    if (!e) e = lml_forward(p, log_alpha, p.beta_stage, p.out);
-    if (!e) e = lml_backward(p, log_alpha, p.beta_stage, p.grad, p.out + 1);
-    if (!e) e = cudaMemcpyAsync(logml, p.out, sizeof(double), cudaMemcpyDefault, p.stream);
-    if (!e)
-        e = cudaMemcpyAsync(grad_log_alpha, p.out + 1, sizeof(double), cudaMemcpyDefault, p.stream);
-    if (!e)
-        e = cudaMemcpyAsync(grad_log_beta, p.grad, sizeof(float) * D, cudaMemcpyDefault, p.stream);
-    uint32_t hflag = 0;
-    if (!e) e = cudaMemcpyAsync(&hflag, flag, sizeof(uint32_t), cudaMemcpyDeviceToHost, p.stream);
-    if (!e) e = cudaStreamSynchronize(p.stream);
+    NoallocResult res{};
+    // the counts in shared memory; where they do not fit, or when a total could
+    // have wrapped (k_lml_terms finds a T_k of 2^32 or more), in global memory
+    for (int pass = 0; pass < 2 && !e; ++pass) {
+        e = cudaMemsetAsync(base, 0, kOffS + sizeof(uint32_t) * (size_t)K * D, p.stream);
+        if (e) break;
+        e = pass ? cudaErrorNotSupported
+                 : lml_launch_stats<true>(p, PlainCsr{indptr, indices, data}, labels, flag);
+        const bool counted = e == cudaSuccess;
+        if (e == cudaErrorNotSupported) {
+            k_lml_stats_checked<<<p.num_sms * 4, 256, 0, p.stream>>>(
+                p.indptr, p.cols, p.counts, p.labels, N, D, K, p.n, p.S, p.T, flag);
+            e = cudaGetLastError();
+        }
+        if (!e) e = lml_terms(p, log_alpha, lb, p.out, p.out + 1, counted ? flag : nullptr);
+        if (!e) e = lml_backward(p, lb, grad);
+        if (!e) e = cudaMemcpyAsync(&res, p.out, sizeof(res), cudaMemcpyDeviceToHost, p.stream);
+        if (!e) e = cudaStreamSynchronize(p.stream);
+        if (!(res.flag & kLmlWrapFlag)) break;
+    }
+    if (!e && grad != grad_log_beta) {
+        e = cudaMemcpyAsync(grad_log_beta, grad, sizeof(float) * D, cudaMemcpyDefault, p.stream);
+        if (!e) e = cudaStreamSynchronize(p.stream);
+    }
+    if (!e) e = give(logml, &res.logml, p.stream);
+    if (!e) e = give(grad_log_alpha, &res.grad_log_alpha, p.stream);
+    const uint32_t hflag = res.flag;
     if (e != cudaSuccess) return noalloc_fail(DPMM_ECUDA, cudaGetErrorString(e));
     if (hflag & 4u)
         return noalloc_fail(DPMM_EOVERFLOW,
                             "dpmm_logml_grad_noalloc: a cluster's count of one gene reaches 2^32");
-    if (hflag)
+    if (hflag & 3u)
         return noalloc_fail(DPMM_EINVAL,
                             (hflag & 1u) ? "dpmm_logml_grad_noalloc: label outside [0, K) or "
                                            "malformed indptr (rows skipped)"

@@ -41,7 +41,9 @@ extern "C" {
 
 #define DPMM_ENGINE_AUTO 0      /* pick per sweep from K and the count density (measured) */
 #define DPMM_ENGINE_CSR_FP32 1  /* warp-per-cell CSR contraction, FP32 */
-#define DPMM_ENGINE_TILE_BF16 2 /* dense 128-cell tiles on tcgen05, BF16 hi/lo; needs
+#define DPMM_ENGINE_TILE_BF16 2 /* dense 128-cell tiles on tcgen05, 16-bit hi/lo operands
+                                   (FP16; BF16 where log theta may pass FP16's
+                                   range), FP32 accumulation; needs
                                    the packed entries (D <= 65,536 genes, every count
                                    <= 65,535) and 1 <= K <= 40: a sweep outside that
                                    runs the CSR engine (dpmm_debug_engine tells) */
@@ -202,9 +204,11 @@ int dpmm_debug_engine(dpmm_ctx* ctx, int32_t* tile_used);
  * package's autotune module times the candidates and caches the fastest).
  *   stats_blocks_per_sm  statistics kernel blocks per SM: 1, 2, 4 or 8
  *                        (default 4 for one chain, 2 for a batch)
- *   tile_stages          dense-tile label kernel A/B stages: 2, or 4 (four
- *                        when they fit in shared memory, else two); default
- *                        4 for one chain, 2 for a batch
+ *   tile_stages          dense-tile label kernel, where two A stages for each
+ *                        of four or three producer sets do not fit in shared
+ *                        memory: 4, four sets of one stage when they fit; 2,
+ *                        two sets of two; default 4 for one chain, 2 for a
+ *                        batch
  *   tile_scatter         row entries a producer lane loads per batch: 8, 12 or
  *                        16 (default 12)
  *   draw_blocks_per_sm   parameter-draw kernel blocks per SM: 1 or 2 (default 2)

@@ -84,6 +84,9 @@ struct DevScalars {
     uint32_t n_apply;     // plans applied so far (sweep compactions and moves)
     int32_t inst_fresh;   // the last plan was a sweep's compaction: the sweep's
                           // pi / theta draws (pre-compaction rows) serve eq. 18
+    int32_t wide_params;  // some log theta may lie beyond FP16's range (set by the draws
+                          // from beta, by dpmm_set_params from the values): the
+                          // dense-tile engine then takes BF16 operands
     int32_t open_slot;    // cluster K - 1 is the eq. 4 K+1 candidate appended for
                           // this sweep (no cells yet; cleared by every plan)
 };
@@ -96,6 +99,11 @@ constexpr int kTileMaxK = 40;
 // density; at K <= 2 and density >= kTileDenseCut the CSR engine is (up to 10%)
 // faster.  So the automatic choice takes the tile engine for K >= 3 always and
 // for K <= 2 only below that density.
+// Segment table of the blocked copy: bit 31 of a segment's quarter-1 pointer: it
+// has a count above 2,047 (a second plane in FP16); of its quarter-2 pointer: a
+// count above 255 (a second plane in BF16).
+constexpr int32_t kTilePtrMask = 0x7FFFFFFF;
+constexpr uint32_t kTileFlag = 0x80000000u;
 constexpr double kTileDenseCut = 0.12;
 constexpr int kTileDenseKmin = 3;
 
@@ -122,6 +130,7 @@ struct Ctx {
     double alpha = 1.0, beta = 1.0;
     dpmm_opts opts{};
     int32_t kmax = 0;
+    int32_t max_count = 0;
     bool packed = false;   // entries stored as (col << 16 | count)
 
     // CSR (device)
@@ -383,6 +392,8 @@ struct ChainArgs {
     // dense-tile engine (tile_enabled = 0: not built for this chain)
     int32_t tile_enabled, tile_C, tile_T, tile_Lslot;
     int32_t tile_kmin;    // smallest K the dense-tile engine labels (engine choice)
+    int32_t max_count;    // largest count of the matrix
+    int32_t wide_beta;    // drawn log theta values may lie beyond FP16's range
     uint32_t* tile_ent;
     int32_t* tile_ptr;
     float* noise;
@@ -623,7 +634,7 @@ cudaError_t launch_tile_count(const int32_t* indptr, const uint32_t* entries, in
 cudaError_t launch_tile_scan(const int32_t* qcount, int64_t TC, int32_t* qptr, long long* out,
                              cudaStream_t st);
 cudaError_t launch_tile_scatter(const int32_t* indptr, const uint32_t* entries, int64_t N,
-                                int32_t T, int32_t C, const int32_t* qptr, uint32_t* tent,
+                                int32_t T, int32_t C, int32_t* qptr, uint32_t* tent,
                                 int num_sms, cudaStream_t st);
 cudaError_t launch_open_slot(Ctx& c);
 cudaError_t launch_local_iteration(Ctx& c, int32_t j);

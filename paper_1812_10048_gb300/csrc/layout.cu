@@ -83,7 +83,7 @@ template <bool COUNT>
 __global__ void __launch_bounds__(kLayoutThreads)
 k_tile_bucket(const int32_t* __restrict__ indptr, const uint32_t* __restrict__ entries, int64_t N,
               int32_t T, int32_t C, int32_t* __restrict__ qcount,
-              const int32_t* __restrict__ qptr, uint32_t* __restrict__ tent) {
+              int32_t* qptr, uint32_t* __restrict__ tent) {
     extern __shared__ int32_t off_all[];   // [warps][C] running offsets
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int32_t* off = off_all + (size_t)w * C;
@@ -109,8 +109,13 @@ k_tile_bucket(const int32_t* __restrict__ indptr, const uint32_t* __restrict__ e
                 if (live) {
                     if (!COUNT) {
                         const int64_t bucket = 4 * (t * C + chunk) + q;
-                        tent[(int64_t)qptr[bucket] + off[chunk] + rank] =
+                        tent[(int64_t)(qptr[bucket] & kTilePtrMask) + off[chunk] + rank] =
                             (r << 22) | (((v >> 16) & 63u) << 16) | (v & 0xFFFFu);
+                        // the segment's second-plane flags
+                        uint32_t* flags =
+                            reinterpret_cast<uint32_t*>(qptr) + 4 * (t * C + chunk);
+                        if ((v & 0xFFFFu) > 255u) atomicOr(flags + 2, kTileFlag);
+                        if ((v & 0xFFFFu) > 2047u) atomicOr(flags + 1, kTileFlag);
                     }
                 }
                 __syncwarp();
@@ -211,7 +216,7 @@ cudaError_t launch_tile_scan(const int32_t* qcount, int64_t TC, int32_t* qptr, l
 }
 
 cudaError_t launch_tile_scatter(const int32_t* indptr, const uint32_t* entries, int64_t N,
-                                int32_t T, int32_t C, const int32_t* qptr, uint32_t* tent,
+                                int32_t T, int32_t C, int32_t* qptr, uint32_t* tent,
                                 int num_sms, cudaStream_t st) {
     const size_t smem = (size_t)(kLayoutThreads / 32) * C * sizeof(int32_t);
     cudaError_t e = cudaFuncSetAttribute(k_tile_bucket<false>,

@@ -242,7 +242,10 @@ k_draw_params(const __grid_constant__ Tab tab) {
             const ChainArgs& ch = tab[c];
             const int row = id - srow[c], K = sK[c];
             if (row == 0) {
-                if (threadIdx.x == 0) select_engine(ch.sc, K, ch);
+                if (threadIdx.x == 0) {
+                    select_engine(ch.sc, K, ch);
+                    ch.sc->wide_params = ch.wide_beta;
+                }
                 clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
             }
             draw_row(ch, K, sopen[c], TAG_THETA, st_[c], row, red, lgc);
@@ -265,7 +268,10 @@ k_draw_params(const __grid_constant__ Tab tab) {
         for (int64_t id = first; id < base + rows; id += gridDim.x) {
             const int row = (int)(id - base);
             if (row == 0) {
-                if (threadIdx.x == 0) select_engine(ch.sc, K, ch);
+                if (threadIdx.x == 0) {
+                    select_engine(ch.sc, K, ch);
+                    ch.sc->wide_params = ch.wide_beta;
+                }
                 clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
             }
             draw_row(ch, K, open, TAG_THETA, t, row, red, lgc);

@@ -4,6 +4,7 @@
 // layout, descriptors and tensor-memory path: C[128][N] = A[128][Kd] B[N][Kd]^T
 // for BF16 operands with FP32 accumulation, one CTA.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <math_constants.h>
 
 #include "common.cuh"
@@ -56,7 +57,7 @@ k_debug_tc_gemm(const uint16_t* __restrict__ A, const uint16_t* __restrict__ B, 
                 const uint64_t ad = tc::desc_sw128(tc::smem_addr(sA + ch * 16384) + 32 * k);
                 const uint64_t bd =
                     tc::desc_sw128(tc::smem_addr(sB + (size_t)ch * N * 128) + 32 * k);
-                tc::mma_bf16(taddr, ad, bd, idesc, (ch | k) != 0);
+                tc::mma_f16(taddr, ad, bd, idesc, (ch | k) != 0);
             }
         tc::mma_commit(bar);
     }
@@ -95,14 +96,16 @@ cudaError_t launch_debug_tc_gemm(const uint16_t* A, const uint16_t* B, int Kd, i
 // ===========================================================================
 // Dense-tile label engine (eq. 4 third line and eq. 8 on the tensor cores).
 //
-// Tiles of 128 consecutive cells, 64-gene chunks.  Per chunk the CTA zeroes a
-// 128 x 64 BF16 operand in shared memory (128-byte swizzled K-major layout) and
-// scatters the chunk's counts into it: x = 256 h + l with l, 256 h exact in
-// BF16 (a second operand holds 256 h and is only multiplied when the chunk has
-// counts above 255).  The B operand (bulk-copied per chunk) holds the centred
-// log theta table split into BF16 hi + lo parts, so that one M=128 MMA per
-// 16 genes accumulates, in FP32 tensor memory, every cluster and sub-cluster
-// score of the 128 cells:
+// Tiles of 128 consecutive cells, 64-gene chunks.  Per (tile, chunk) item the
+// CTA zeroes a 128 x 64 16-bit operand in shared memory (128-byte swizzled
+// K-major layout) and scatters the counts into it; counts beyond the format's
+// exact integers (2,047 in FP16, 255 in BF16) are split into two exact digits,
+// the second of which goes through the same stage as another plane, only for
+// items that have such counts (flagged when the blocked copy is built).  The B
+// operand (bulk-copied per chunk) holds the centred log theta table split into
+// hi + lo parts of the same format, so that one M=128 MMA per 16 genes
+// accumulates, in FP32 tensor memory, every cluster and sub-cluster score of
+// the 128 cells:
 //   TMEM / B column 2k, 2k+1            cluster k, hi and lo part
 //   column S0 + 4k + 2r, S0 + 4k + 2r + 1  sub-cluster (k, r), hi and lo part
 // with S0 = 2K rounded up to 16 and Ntot = (S0 + 4K) rounded up to 16 <= 256
@@ -125,6 +128,22 @@ __host__ __device__ __forceinline__ bool tile_usable(int K) {
 __host__ __device__ __forceinline__ int tile_s0(int K) { return (2 * K + 15) & ~15; }
 __host__ __device__ __forceinline__ int tile_ntot(int K) { return (tile_s0(K) + 4 * K + 15) & ~15; }
 
+// Operand format of a chain's contraction: FP16 (11 significant bits: log theta
+// as hi + lo to 2^-22, counts to 2,047 in one plane) unless a log theta may lie
+// beyond FP16's range, then BF16 (to 2^-16, counts to 255 in one plane).
+__device__ __forceinline__ bool chain_half(const ChainArgs& ch) { return !ch.sc->wide_params; }
+
+// Some segments of the chain have a second plane (counts beyond the lo digit).
+__device__ __forceinline__ bool chain_planes(const ChainArgs& ch) {
+    return ch.max_count > (chain_half(ch) ? 2047 : 255);
+}
+
+__device__ __forceinline__ uint16_t f16_bits_rn(float f) {
+    return __half_as_ushort(__float2half_rn(f));
+}
+__device__ __forceinline__ float f16_value(uint16_t b) {
+    return __half2float(__ushort_as_half(b));
+}
 __device__ __forceinline__ uint16_t bf16_bits_rn(float f) {
     const __nv_bfloat16 h = __float2bfloat16_rn(f);
     return *reinterpret_cast<const uint16_t*>(&h);
@@ -201,6 +220,7 @@ k_build_b(const __grid_constant__ Tab tab, int32_t force, int32_t rb) {
         __syncthreads();
     }
     unsigned char* dst = B + (size_t)c * kBChunkBytes;
+    const bool half = chain_half(ch);
     for (int i = blockIdx.y * rb * 64 + threadIdx.x; i < min(Ntot, (int)(blockIdx.y + 1) * rb) * 64;
          i += blockDim.x) {
         const int row = i >> 6, g = i & 63, u = c * 64 + g;
@@ -220,8 +240,13 @@ k_build_b(const __grid_constant__ Tab tab, int32_t force, int32_t rb) {
         uint16_t v = 0;
         if (live) {
             const float d = L - m[g];
-            const uint16_t hi = bf16_bits_rn(d);
-            v = part ? bf16_bits_rn(d - bf16_value(hi)) : hi;
+            if (half) {
+                const uint16_t hi = f16_bits_rn(d);
+                v = part ? f16_bits_rn(d - f16_value(hi)) : hi;
+            } else {
+                const uint16_t hi = bf16_bits_rn(d);
+                v = part ? bf16_bits_rn(d - bf16_value(hi)) : hi;
+            }
         }
         *reinterpret_cast<uint16_t*>(dst + tc::swz_offset((uint32_t)row, (uint32_t)g)) = v;
     }
@@ -244,43 +269,117 @@ __device__ __forceinline__ void chain_tiles(int64_t off, int T, int& first, int&
 // Warp roles of the pipelined engine (27 warps):
 //   warps 0-7   epilogue, two halves of four warps over the same 128 cells
 //               (warp w reads TMEM lanes 32 (w % 4) ..): each half takes every
-//               other 8-cluster column group of the Gumbel-max; half 1 also
-//               draws the eq. 8 noise, half 0 merges and finishes the cell
-//   warps 8-23  producers, four sets of four warps taking chunks in turn
+//               other 8-cluster column group of the Gumbel-max, then (the
+//               winner exchanged) every other block of sub-cluster columns,
+//               and finishes the cells whose sub-cluster columns it met
+//   warps 8-23  producers, four sets of four warps taking items in turn
 //               (two sets when only two A stages fit); warp q of a set
-//               densifies rows 32q .. 32q + 31 of its chunk (the entries of
+//               densifies rows 32q .. 32q + 31 of its item (the entries of
 //               one quarter) from the staged segment, so the four warps never
 //               wait on one another
-//   warp 24     lane 0 issues the MMAs (two TMEM accumulators of 256 columns)
-//   warp 25     segment loader: bulk-copies each chunk's entries into a ring
-//               of slots, reading the segment table a warp-batch ahead
+//   warp 24     issues the MMAs
+//   warp 25     segment loader: bulk-copies each item's entries into a ring
+//               of slots, one lane per producer set, reading the segment table
+//               a round ahead
 //   warp 26     lane 0 bulk-copies the B operand of each chunk into its ring
-// Every role walks the same sequence: the chains in order, this CTA's tiles
-// of each chain, the chunks of each tile.
+// Every role walks the same sequence of items (tile, chunk): the chains in
+// order, this CTA's tiles of each chain in pairs, the chunks, and for each chunk
+// the tiles of the pair, so that one copy of a chunk's B operand serves both
+// tiles (B, the same for every CTA, is otherwise the largest stream from the
+// L2: 32 KB an item at K = 40, against 4 KB of entries).  A tile's chunks are
+// accumulated in the same order as without the pairing.  The accumulators are
+// nAcc slots of TMEM (512 columns / the score columns, at most four) that the
+// tiles take in turn.
 // Hand-offs are mbarriers: ent_full / ent_free (segment slots), a_full (the
-// four producer warps and the B loader's bulk copy -> MMA: a stage holds a
-// chunk's A tiles and B operand), stage_free (MMA commit -> producers and B
-// loader), acc_full (MMA -> epilogue) / acc_empty (epilogue -> MMA).
+// four producer warps -> MMA), b_full (B copy -> MMA), stage_free, b_free (MMA
+// commit -> producers, B loader), acc_full (MMA -> epilogue) / acc_empty
+// (epilogue -> MMA).  The A operand is written by ordinary stores, each
+// producer lane's proxy fence before its arrival makes them visible to the MMA.
 // Every wait is bounded; a timeout records DPMM_ETIMEOUT, every role leaves
 // its loop, and each role that issued asynchronous work waits (bounded) for
 // it before the block exits.
-constexpr int kMaxStages = 4;        // A stages (lo + hi), even
+constexpr int kMaxStages = 8;        // A stages
+constexpr uint32_t kStageBytes = 16384;   // 128 cells x 64 genes x 2 bytes
+constexpr int kHiStages = 2;          // stages of the items' second planes
+constexpr int kMaxBStages = 4;
+constexpr int kMaxAcc = 4;
+constexpr int kPair = 2;             // tiles that share a chunk's B operand
 constexpr int kMaxESlots = 16;
 constexpr int kEpiWarps = 8;
-constexpr int kProdSets = 4;        // producer sets (4 warps each) on alternate chunks
+constexpr int kProdSets = 4;        // producer sets (4 warps each) on alternate items
 constexpr int kProdWarp0 = 8;
-constexpr int kMmaWarp = kProdWarp0 + 4 * kProdSets;
-constexpr int kELoadWarp = kMmaWarp + 1;
-constexpr int kBLoadWarp = kMmaWarp + 2;
-constexpr int kTileThreadsP = (kMmaWarp + 3) * 32;
-constexpr int kBarEpi = 1, kBarLabel = 2;
+constexpr int kMmaWarp = 8, kELoadWarp = 12, kBLoadWarp = 16;
+constexpr int kTileThreadsP = (kProdWarp0 + (4 * kProdSets + 2) / 3 * 4) * 32;
+constexpr int kBarEpi = 1, kBarHalf = 2;   // kBarHalf + h: one half
+constexpr int kEpiGroups = (kTileMaxK + 15) / 16;   // 8-cluster groups of a half
 constexpr int kSmallBytes = 8192;
 constexpr int kScatterDefault = 12;  // entries per producer lane and batch (tunable: 8, 12, 16)
+
+// The digits of a count in the operand format: lo and hi with lo + hi = x, each
+// exact in 16 bits (FP16: 11 significant bits, x = (x & 2047) + (x & 0xF800);
+// BF16: 8, x = (x & 255) + (x & 0xFF00), whose FP32 patterns truncate exactly).
+template <bool kHalf>
+__device__ __forceinline__ uint16_t digit_bits(uint32_t v) {
+    if (kHalf) return __half_as_ushort(__ushort2half_rn((unsigned short)v));
+    return (uint16_t)(__float_as_uint((float)v) >> 16);
+}
+template <bool kHalf>
+__device__ __forceinline__ constexpr uint32_t lo_mask() { return kHalf ? 0x7FFu : 0xFFu; }
+
+// One producer warp's share of a staged segment into its quarter q of the A stage
+// (kHi: the hi digits, else the lo ones): the 16-byte groups that hold entries
+// [i0, i1), kScatter entries per lane in flight.  A group at either end may hold
+// entries of a neighbouring quarter, which their rows tell apart, and the
+// segment's padding, whose counts are 0.  An entry row << 22 | gene << 16 | count
+// shifted right by 15 has its row and gene at the bytes row * 128 + gene * 2 of
+// the stage; the 128-byte swizzle exchanges bits 4-6 with the row's low bits.
+template <bool kHalf, bool kHi, int kScatter>
+__device__ __forceinline__ void scatter_entries(const uint32_t* ring, int i0, int i1, int q,
+                                                int lane, unsigned char* A) {
+    constexpr uint32_t mask = kHi ? 0xFFFFu & ~lo_mask<kHalf>() : lo_mask<kHalf>();
+    constexpr int U = kScatter / 4;
+    const uint4* ring4 = reinterpret_cast<const uint4*>(ring);
+    const int j1 = (i1 + 3) >> 2;
+    for (int j = (i0 >> 2) + lane; j < j1; j += 32 * U) {
+        uint4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            v[u] = j + 32 * u < j1 ? ring4[j + 32 * u] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t e[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t x = e[k] & mask, t = e[k] >> 15;
+                if (x && (e[k] >> 27) == (uint32_t)q)
+                    *reinterpret_cast<uint16_t*>(A + ((t & 0x3FFEu) ^ ((t >> 3) & 0x70u))) =
+                        digit_bits<kHalf>(x);
+            }
+        }
+    }
+}
+
+// A producer warp's quarter of an A stage, cleared.
+__device__ __forceinline__ void clear_quarter(unsigned char* A, int q, int lane) {
+    uint4* zl = reinterpret_cast<uint4*>(A + q * 4096);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) zl[lane + 32 * i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+}
+
+// A 64-bit sum kept as two 32-bit words in shared memory (the 32-bit shared
+// atomics are single instructions, the 64-bit one is a loop).
+__device__ __forceinline__ void add_words64(uint32_t* w, unsigned long long v) {
+    const uint32_t lo = (uint32_t)v;
+    const uint32_t old = atomicAdd(w, lo);
+    const uint32_t hi = (uint32_t)(v >> 32) + (old + lo < old ? 1u : 0u);
+    if (hi) atomicAdd(w + 1, hi);
+}
 
 // dbg: optional [N][3K] centred scores of a single chain (no state or
 // statistics writes).
 // kScatter: row entries a producer lane loads per batch; stages_pref: 2 to
-// use two A/B stages even when four fit (0: as many as fit).
+// keep two A stages to every producer set rather than four sets of one.
 template <class Tab, int kScatter>
 __global__ void __launch_bounds__(kTileThreadsP, 1)
 k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
@@ -291,8 +390,9 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool dbg = dbg_out != nullptr;
     // this CTA's work and the largest operand / segment over the chains
-    uint32_t total = 0;   // chunks of this block
+    uint32_t total = 0;   // items of this block
     int ntot_max = 0, lslot_max = 4;
+    bool planes_any = false;
     {
         int64_t off = 0;
         for (int b = 0; b < tab.n(); ++b) {
@@ -304,82 +404,100 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             total += (uint32_t)cnt * (uint32_t)ch.tile_C;
             ntot_max = max(ntot_max, tile_ntot(ch.sc->K));
             lslot_max = max(lslot_max, ch.tile_Lslot);
+            planes_any = planes_any || chain_planes(ch);
         }
     }
     if (total == 0) return;
-    // shared-memory plan (identical in every thread): A stages, B slots,
+    // shared-memory plan (identical in every thread): A stages, B stages,
     // segment slots, then the small area
     const int64_t b_slot = ((int64_t)ntot_max * 128 + 1023) & ~(int64_t)1023;
     const int64_t e_slot = (int64_t)lslot_max * 4;
     const int64_t avail = smem_bytes - (int64_t)(base - smem_raw) - kSmallBytes;
-    // a stage holds a chunk's A tiles (lo, hi) and its B operand: one MMA
-    // commit per chunk frees both
-    const int nS = stages_pref != 2 &&
-                           (int64_t)kMaxStages * (32768 + b_slot) + 2 * e_slot <= avail
-                       ? kMaxStages
-                       : 2;
-    const int nB = nS;
+    // hi stages, only when some chain of the launch has a second plane
+    const int64_t h_bytes = planes_any ? (int64_t)kHiStages * kStageBytes : 0;
+    // producer sets and A stages, the most that fit (a set takes every nsets-th
+    // item and always meets the same stages and slots, so nsets divides nS and
+    // nE: slot g % nE is then refilled for item g only after the same set
+    // consumed item g - nE, and a set's parity wait can never be two phases
+    // ahead).  Two stages a set let it fill one while the MMAs read the other.
+    auto fit = [&](int sets, int stages) {
+        return stages * (int64_t)kStageBytes + h_bytes + 2 * b_slot + sets * e_slot <= avail;
+    };
+    // 1.3 M x 2,000, K = 40: four sets of one stage 1,364 us, three of two
+    // 1,288 us; 68,000 x 1,000, K = 10: four sets of two stages 37 us, three 41.
+    int nsets = 2, nS = 2;
+    if (fit(4, 8)) nsets = 4, nS = 8;
+    else if (fit(3, 6)) nsets = 3, nS = 6;
+    else if (stages_pref != 2 && fit(4, 4)) nsets = 4, nS = 4;
+    else if (fit(2, 4)) nsets = 2, nS = 4;
+    // more than two B stages only where they leave eight segment slots
+    int nB = 2;
+    while (nB < kMaxBStages &&
+           nS * (int64_t)kStageBytes + h_bytes + (nB + 1) * b_slot + 8 * e_slot <= avail)
+        ++nB;
     const int nE_fit = (int)min((int64_t)kMaxESlots,
-                                (avail - (int64_t)nS * (32768 + b_slot)) / e_slot);
-    // producer sets in use: each set must meet the same A stages (its hi
-    // halves) and the same segment slots, so nsets divides nS and nE.  Slot
-    // g % nE is then refilled for chunk g only after the same set consumed
-    // chunk g - nE, and a set's parity wait can never be two phases ahead.
-    const int nsets = (nS % kProdSets == 0 && nE_fit >= kProdSets) ? kProdSets : 2;
+                                (avail - nS * (int64_t)kStageBytes - h_bytes - nB * b_slot) / e_slot);
     const int nE = (nE_fit / nsets) * nsets;
-    if (nB < 2 || nE < 2) {
+    if (nE < 2) {
         if (tid == 0) atomicExch(&tab[0].sc->error, DPMM_ECAPACITY);
         return;
     }
-    unsigned char* A_base = base;                                  // stage s: lo, then hi
-    unsigned char* B_base = A_base + nS * 32768;
+    const uint32_t ldN = ((uint32_t)ntot_max + 31u) & ~31u;        // TMEM columns of a slot
+    const uint32_t nAcc = min((uint32_t)kMaxAcc, 512u / ldN);      // >= 2
+    unsigned char* A_base = base;
+    unsigned char* H_base = A_base + nS * kStageBytes;
+    unsigned char* B_base = H_base + h_bytes;
     unsigned char* E_base = B_base + nB * b_slot;
     unsigned char* small = E_base + nE * e_slot;
     small = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(small) + 15) & ~(uintptr_t)15);
-    uint64_t* a_full = reinterpret_cast<uint64_t*>(small);         // [kMaxStages]
+    int4* meta = reinterpret_cast<int4*>(small);                   // [kMaxESlots] quarter ends
+    uint64_t* a_full = reinterpret_cast<uint64_t*>(meta + kMaxESlots);   // [kMaxStages]
     uint64_t* stage_free = a_full + kMaxStages;                     // [kMaxStages]
-    uint64_t* ent_full = stage_free + kMaxStages;                   // [kMaxESlots]
+    uint64_t* b_full = stage_free + kMaxStages;                     // [kMaxBStages]
+    uint64_t* b_free = b_full + kMaxBStages;                        // [kMaxBStages]
+    uint64_t* hi_full = b_free + kMaxBStages;                       // [kHiStages]
+    uint64_t* hi_used = hi_full + kHiStages;                        // [kHiStages]
+    uint64_t* ent_full = hi_used + kHiStages;                       // [kMaxESlots]
     uint64_t* ent_free = ent_full + kMaxESlots;                     // [kMaxESlots]
-    uint64_t* acc_full = ent_free + kMaxESlots;                     // [2]
-    uint64_t* acc_empty = acc_full + 2;                             // [2]
-    int32_t* meta = reinterpret_cast<int32_t*>(acc_empty + 2);      // [kMaxESlots][4]
-    uint32_t* taddr_s = reinterpret_cast<uint32_t*>(meta + 4 * kMaxESlots);
+    uint64_t* acc_full = ent_free + kMaxESlots;                     // [kMaxAcc]
+    uint64_t* acc_empty = acc_full + kMaxAcc;                       // [kMaxAcc]
+    uint64_t* drain = acc_empty + kMaxAcc;                          // [1]
+    uint32_t* taddr_s = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* err = reinterpret_cast<volatile int*>(taddr_s + 1);
     int* stop = const_cast<int*>(err) + 1;                          // [2]
-    uint8_t* stage_hib = reinterpret_cast<uint8_t*>(stop + 2);      // [kMaxStages][4]
-    float* spi = reinterpret_cast<float*>(stage_hib + 4 * kMaxStages);  // [K]
+    int32_t* stage_hi = stop + 2;                                   // [kMaxStages]
+    int32_t* meta_hi = stage_hi + kMaxStages;                       // [kMaxESlots]
+    volatile int32_t* hi_done = meta_hi + kMaxESlots;               // second planes used up
+    float* spi = reinterpret_cast<float*>(meta_hi + kMaxESlots + 1);    // [K]
     float* slw = spi + kTileMaxK;                                   // [4K]
-    float* xbest = slw + 4 * kTileMaxK;                             // [2][128] half 1 -> half 0
-    int* xc = reinterpret_cast<int*>(xbest + 256);                  // [2][128]
-    float* xg0 = reinterpret_cast<float*>(xc + 256);                // [2][128]
-    float* xg1 = xg0 + 256;                                         // [2][128]
-    unsigned long long* wsq =                                       // [4][K] sum log q
-        reinterpret_cast<unsigned long long*>(((reinterpret_cast<uintptr_t>(xg1 + 256)) + 7) & ~(uintptr_t)7);
+    float* xbest = slw + 4 * kTileMaxK;                             // [2][half][128]
+    int* xc = reinterpret_cast<int*>(xbest + 512);                  // [2][half][128]
+    uint32_t* wsq = reinterpret_cast<uint32_t*>(xc + 512);          // [4][K][2] sum log q
 
-    if (tid < 4 * kMaxStages) stage_hib[tid] = 0;
-    {
-        // the hi halves start clear: a producer warp clears its quarter of a hi
-        // half only after it has written counts above 255 there
-        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-        for (int s = 0; s < nS; ++s) {
-            uint4* hi = reinterpret_cast<uint4*>(A_base + s * 32768 + 16384);
-            for (int i = tid; i < 1024; i += blockDim.x) hi[i] = z;
-        }
-    }
     if (tid == 0) {
         *err = 0;
+        *hi_done = 0;
         stop[0] = stop[1] = 0;
         for (int i = 0; i < kMaxStages; ++i) {
-            tc::mbar_init(&a_full[i], 5);   // four producer warps + the B copy
+            tc::mbar_init(&a_full[i], 4);   // four producer warps
             tc::mbar_init(&stage_free[i], 1);
         }
+        for (int i = 0; i < kMaxBStages; ++i) {
+            tc::mbar_init(&b_full[i], 1);
+            tc::mbar_init(&b_free[i], 1);
+        }
+        for (int i = 0; i < kHiStages; ++i) {
+            tc::mbar_init(&hi_full[i], 4);
+            tc::mbar_init(&hi_used[i], 1);
+        }
+        tc::mbar_init(drain, 1);
         for (int i = 0; i < kMaxESlots; ++i) {
             tc::mbar_init(&ent_full[i], 1);
             tc::mbar_init(&ent_free[i], 4);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < kMaxAcc; ++i) {
             tc::mbar_init(&acc_full[i], 1);
-            tc::mbar_init(&acc_empty[i], 1);
+            tc::mbar_init(&acc_empty[i], 2);   // the epilogue's halves
         }
         tc::fence_mbar_init();
     }
@@ -393,75 +511,91 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     tc::fence_after_sync();
     const uint32_t tmem = *taddr_s;
 
-    if (warp >= kProdWarp0 && warp < kMmaWarp) {
+    if (warp >= kProdWarp0 && (warp & 3)) {
         // ---------------- producers ----------------
-        const int set = (warp - kProdWarp0) >> 2, q = (warp - kProdWarp0) & 3;
-        uint32_t hi_dirty = 0u;   // stages whose hi quarter this warp left non-zero
-        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-        for (uint32_t g = (uint32_t)set; set < nsets && g < total; g += (uint32_t)nsets) {
-            const int st = (int)(g % (uint32_t)nS);
-            const int es = (int)(g % (uint32_t)nE);
-            bool ok = tc::mbar_wait(&ent_full[es], (g / (uint32_t)nE) & 1u, kWaitLimit);
-            if (ok && g >= (uint32_t)nS)
-                ok = tc::mbar_wait(&stage_free[st], ((g / (uint32_t)nS) - 1u) & 1u, kWaitLimit);
-            if (!__all_sync(0xFFFFFFFFu, ok)) {
-                if (lane == 0) *err = DPMM_ETIMEOUT;
+        const int pi = (warp - kProdWarp0) / 4 * 3 + (warp & 3) - 1, set = pi >> 2, q = pi & 3;
+        // this set's stages and slots, one after the other
+        uint32_t st = (uint32_t)set % (uint32_t)nS, sph = 1u;   // parity of the stage's last use
+        uint32_t es = (uint32_t)set % (uint32_t)nE, eph = 0u;
+        uint32_t g = set < nsets ? (uint32_t)set : total;
+        uint32_t gend = 0;        // items before the end of the current chain
+        int b = -1;
+        int64_t off = 0;
+        bool half = false;
+        for (; g < total; g += (uint32_t)nsets) {
+            while (g >= gend) {   // the chain of item g: its operand format
+                const ChainArgs& ch = tab[++b];
+                if (!chain_on_tiles(ch, dbg)) continue;
+                int first, cnt;
+                chain_tiles(off, ch.tile_T, first, cnt);
+                off += ch.tile_T;
+                gend += (uint32_t)cnt * (uint32_t)ch.tile_C;
+                half = chain_half(ch);
+            }
+            unsigned char* A = A_base + st * kStageBytes;
+            // (at a stage's first use the parity of the phase before the first)
+            bool ok = tc::mbar_wait(&stage_free[st], sph, kWaitLimit);
+            if (__all_sync(0xFFFFFFFFu, ok)) {
+                clear_quarter(A, q, lane);      // while the segment is still on its way
+                ok = tc::mbar_wait(&ent_full[es], eph, kWaitLimit);
+            }
+            if (!__all_sync(0xFFFFFFFFu, ok && *err == 0)) {
+                if (lane == 0 && !ok) *err = DPMM_ETIMEOUT;
                 break;
             }
-            if (__any_sync(0xFFFFFFFFu, *err != 0)) break;
-            unsigned char* A_lo = A_base + st * 32768;
-            unsigned char* A_hi = A_lo + 16384;
-            uint4* zl = reinterpret_cast<uint4*>(A_lo + q * 4096);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) zl[lane + 32 * i] = z;
-            if ((hi_dirty >> st) & 1u) {
-                uint4* zh = reinterpret_cast<uint4*>(A_hi + q * 4096);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) zh[lane + 32 * i] = z;
-            }
-            __syncwarp();
-            const int32_t* mt = meta + 4 * es;
-            const int i0 = q ? mt[q - 1] : 0, i1 = mt[q];
+            const int4 mt = meta[es];
+            const int i0 = q == 0 ? 0 : q == 1 ? mt.x : q == 2 ? mt.y : mt.z;
+            const int i1 = q == 0 ? mt.x : q == 1 ? mt.y : q == 2 ? mt.z : mt.w;
+            const int hi = planes_any ? meta_hi[es] : 0;    // 0, or 1 + its number
             const uint32_t* ring = reinterpret_cast<const uint32_t*>(E_base + es * e_slot);
-            // batches of kScatter entries per lane: all loads first, then the
-            // stores, so that a lane keeps several shared-memory accesses in
-            // flight.  x & 255 and x & 0xFF00 have at most 8 significant bits,
-            // so their FP32 bit patterns truncate exactly to BF16.
-            int hi = 0;
-            for (int i = i0 + lane; i < i1; i += 32 * kScatter) {
-                uint32_t v[kScatter];
-#pragma unroll
-                for (int u = 0; u < kScatter; ++u) v[u] = i + 32 * u < i1 ? ring[i + 32 * u] : 0u;
-#pragma unroll
-                for (int u = 0; u < kScatter; ++u) {
-                    const uint32_t x = v[u] & 0xFFFFu;
-                    // an entry's row lies in this warp's quarter (checked, so
-                    // that no entry can address outside the stage)
-                    if (x && (v[u] >> 22) - 32u * (uint32_t)q < 32u) {
-                        const uint32_t off = tc::swz_offset(v[u] >> 22, (v[u] >> 16) & 63u);
-                        *reinterpret_cast<uint16_t*>(A_lo + off) =
-                            (uint16_t)(__float_as_uint((float)(x & 255u)) >> 16);
-                        if (x >> 8) {
-                            *reinterpret_cast<uint16_t*>(A_hi + off) =
-                                (uint16_t)(__float_as_uint((float)(x & 0xFF00u)) >> 16);
-                            hi = 1;
-                        }
-                    }
-                }
-            }
-            hi = __any_sync(0xFFFFFFFFu, hi);
+            if (half) scatter_entries<true, false, kScatter>(ring, i0, i1, q, lane, A);
+            else scatter_entries<false, false, kScatter>(ring, i0, i1, q, lane, A);
             tc::fence_async_smem();
             __syncwarp();
             if (lane == 0) {
-                stage_hib[4 * st + q] = (uint8_t)hi;
+                if (planes_any && q == 0) stage_hi[st] = hi;
                 tc::mbar_arrive(&a_full[st]);
-                tc::mbar_arrive(&ent_free[es]);
+                if (!hi) tc::mbar_arrive(&ent_free[es]);
             }
-            hi_dirty = hi ? (hi_dirty | (1u << st)) : (hi_dirty & ~(1u << st));
+            if (hi) {
+                // its hi digits, in the block's order of second planes: the plane
+                // kHiStages before it has been used (a count, since this set may
+                // be more than one use of the stage ahead, which a phase's parity
+                // could not tell)
+                const uint32_t hs = (uint32_t)(hi - 1) % kHiStages;
+                ok = false;
+                for (uint32_t x = 0; x < kWaitLimit && !ok; ++x)
+                    ok = *hi_done + kHiStages >= hi;
+                __threadfence_block();
+                if (!__all_sync(0xFFFFFFFFu, ok)) {
+                    if (lane == 0) *err = DPMM_ETIMEOUT;
+                    break;
+                }
+                unsigned char* H = H_base + hs * kStageBytes;
+                clear_quarter(H, q, lane);
+                if (half) scatter_entries<true, true, kScatter>(ring, i0, i1, q, lane, H);
+                else scatter_entries<false, true, kScatter>(ring, i0, i1, q, lane, H);
+                tc::fence_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tc::mbar_arrive(&hi_full[hs]);
+                    tc::mbar_arrive(&ent_free[es]);
+                }
+            }
+            if ((st += (uint32_t)nsets) >= (uint32_t)nS) {
+                st -= (uint32_t)nS;
+                sph ^= 1u;
+            }
+            if ((es += (uint32_t)nsets) >= (uint32_t)nE) {
+                es -= (uint32_t)nE;
+                eph ^= 1u;
+            }
         }
     } else if (warp == kELoadWarp) {
         // ---------------- segment loader ----------------
-        uint32_t g = 0;        // chunks started (slot sequence)
+        uint32_t g = 0;        // items started (slot sequence)
+        uint32_t hseq = 0;     // second planes started
+        const unsigned lanemask = (1u << lane) - 1u;
         bool stop_l = false;
         int64_t off = 0;
         for (int b = 0; b < tab.n() && !stop_l; ++b) {
@@ -471,62 +605,65 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             chain_tiles(off, ch.tile_T, first, cnt);
             off += ch.tile_T;
             const uint32_t C = (uint32_t)ch.tile_C;
-            const uint32_t nchunk = (uint32_t)cnt * C;
-            // lane j holds the five quarter pointers of chunk jb + j of this chain
-            auto seg_ptrs = [&](uint32_t j, int32_t (&p)[5]) {
-                if (j < nchunk) {
-                    const uint32_t ti = j / C, ci = j - ti * C;
+            const uint32_t nitem = (uint32_t)cnt * C;
+            const bool half = chain_half(ch);
+            // lane l < nsets takes the items l, l + nsets, ...: their five
+            // quarter pointers, read one round ahead
+            auto seg_ptrs = [&](uint32_t j, int32_t (&p)[6]) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k) p[k] = 0;
+                if (lane < nsets && j < nitem) {
+                    const uint32_t pr = j / (kPair * C);           // pair, then chunk, then tile
+                    const uint32_t m = min((uint32_t)kPair, (uint32_t)cnt - kPair * pr);
+                    const uint32_t r = j - pr * kPair * C, ci = r / m;
                     const int64_t sgm =
-                        ((int64_t)first + (int64_t)ti * gridDim.x) * (int64_t)C + ci;
+                        ((int64_t)first + (int64_t)(kPair * pr + (r - ci * m)) * gridDim.x) *
+                            (int64_t)C + ci;
 #pragma unroll
                     for (int k = 0; k < 5; ++k) p[k] = __ldg(ch.tile_ptr + 4 * sgm + k);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) p[k] = 0;
+                    // the segment's second-plane flag, then the pointers
+                    p[5] = half ? p[1] < 0 : p[2] < 0;
+                    p[1] &= kTilePtrMask;
+                    p[2] &= kTilePtrMask;
                 }
             };
-            int32_t cur[5], nxt[5];
+            int32_t cur[6], nxt[6];
             seg_ptrs((uint32_t)lane, cur);
-            for (uint32_t jb = 0; jb < nchunk; jb += 32) {
-                if (__any_sync(0xFFFFFFFFu, *err != 0)) {
+            for (uint32_t jb = 0; jb < nitem; jb += (uint32_t)nsets) {
+                seg_ptrs(jb + (uint32_t)nsets + (uint32_t)lane, nxt);
+                const uint32_t n = min((uint32_t)nsets, nitem - jb);
+                bool ok = true;
+                if ((uint32_t)lane < n) {
+                    const uint32_t gl = g + (uint32_t)lane, es = gl % (uint32_t)nE;
+                    if (gl >= (uint32_t)nE)
+                        ok = tc::mbar_wait(&ent_free[es], (gl / (uint32_t)nE - 1u) & 1u,
+                                           kWaitLimit);
+                    if (!ok) *err = DPMM_ETIMEOUT;
+                }
+                if (!__all_sync(0xFFFFFFFFu, ok && *err == 0)) {
                     stop_l = true;
                     break;
                 }
-                seg_ptrs(jb + 32 + (uint32_t)lane, nxt);
-                for (uint32_t j = 0; j < 32 && jb + j < nchunk; ++j, ++g) {
-                    const int es = (int)(g % (uint32_t)nE);
-                    int32_t p[5];
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) p[k] = __shfl_sync(0xFFFFFFFFu, cur[k], (int)j);
-                    bool ok = true;
-                    if (lane == 0 && g >= (uint32_t)nE)
-                        ok = tc::mbar_wait(&ent_free[es], ((g / (uint32_t)nE) - 1u) & 1u,
-                                           kWaitLimit);
-                    ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
-                    if (!ok && lane == 0) *err = DPMM_ETIMEOUT;
-                    if (__any_sync(0xFFFFFFFFu, !ok || *err != 0)) {
-                        stop_l = true;
-                        break;
-                    }
-                    if (lane == 0) {
-                        int32_t* mt = meta + 4 * es;
-                        mt[0] = p[1] - p[0];
-                        mt[1] = p[2] - p[0];
-                        mt[2] = p[3] - p[0];
-                        mt[3] = p[4] - p[0];
-                        const uint32_t bytes = (uint32_t)(p[4] - p[0]) * 4u;
-                        if (bytes) {
-                            tc::mbar_arrive_expect_tx(&ent_full[es], bytes);
-                            tc::bulk_g2s(E_base + es * e_slot, ch.tile_ent + p[0], bytes,
-                                         &ent_full[es]);
-                        } else {
-                            tc::mbar_arrive(&ent_full[es]);
-                        }
+                const unsigned flagged = __ballot_sync(0xFFFFFFFFu, (uint32_t)lane < n && cur[5]);
+                if ((uint32_t)lane < n) {
+                    const uint32_t es = (g + (uint32_t)lane) % (uint32_t)nE;
+                    meta[es] = make_int4(cur[1] - cur[0], cur[2] - cur[0], cur[3] - cur[0],
+                                         cur[4] - cur[0]);
+                    if (planes_any)
+                        meta_hi[es] = cur[5] ? 1 + (int)(hseq + __popc(flagged & lanemask)) : 0;
+                    const uint32_t bytes = (uint32_t)(cur[4] - cur[0]) * 4u;
+                    if (bytes) {
+                        tc::mbar_arrive_expect_tx(&ent_full[es], bytes);
+                        tc::bulk_g2s(E_base + es * e_slot, ch.tile_ent + cur[0], bytes,
+                                     &ent_full[es]);
+                    } else {
+                        tc::mbar_arrive(&ent_full[es]);
                     }
                 }
-                if (stop_l) break;
+                g += n;
+                hseq += (uint32_t)__popc(flagged);
 #pragma unroll
-                for (int k = 0; k < 5; ++k) cur[k] = nxt[k];
+                for (int k = 0; k < 6; ++k) cur[k] = nxt[k];
             }
         }
         // every started copy has landed before the block can exit
@@ -537,7 +674,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     } else if (warp == kBLoadWarp) {
         // ---------------- B loader ----------------
         if (lane == 0) {
-            uint32_t g = 0;
+            uint32_t g = 0, bs = 0, bph = 0;    // chunks started
             bool stop_b = false;
             int64_t off = 0;
             for (int b = 0; b < tab.n() && !stop_b; ++b) {
@@ -547,91 +684,193 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                 chain_tiles(off, ch.tile_T, first, cnt);
                 off += ch.tile_T;
                 const uint32_t bytes = (uint32_t)tile_ntot(ch.sc->K) * 128u;
-                const uint32_t nchunk = (uint32_t)cnt * (uint32_t)ch.tile_C;
-                for (uint32_t j = 0; j < nchunk; ++j, ++g) {
-                    const int bs = (int)(g % (uint32_t)nB);
-                    if (g >= (uint32_t)nB &&
-                        !tc::mbar_wait(&stage_free[bs], ((g / (uint32_t)nB) - 1u) & 1u,
-                                       kWaitLimit)) {
-                        *err = DPMM_ETIMEOUT;
-                        stop_b = true;
-                        break;
+                for (int i = 0; i < cnt && !stop_b; i += kPair) {
+                    for (int c = 0; c < ch.tile_C; ++c, ++g) {
+                        if (g >= (uint32_t)nB &&
+                            !tc::mbar_wait(&b_free[bs], bph ^ 1u, kWaitLimit)) {
+                            *err = DPMM_ETIMEOUT;
+                            stop_b = true;
+                            break;
+                        }
+                        if (*err) {
+                            stop_b = true;
+                            break;
+                        }
+                        tc::mbar_arrive_expect_tx(&b_full[bs], bytes);
+                        tc::bulk_g2s(B_base + bs * b_slot, ch.tile_B + (size_t)c * kBChunkBytes,
+                                     bytes, &b_full[bs]);
+                        if (++bs == (uint32_t)nB) {
+                            bs = 0;
+                            bph ^= 1u;
+                        }
                     }
-                    if (*err) {
-                        stop_b = true;
-                        break;
-                    }
-                    const uint32_t c = j % (uint32_t)ch.tile_C;
-                    tc::mbar_arrive_expect_tx(&a_full[bs], bytes);
-                    tc::bulk_g2s(B_base + bs * b_slot, ch.tile_B + (size_t)c * kBChunkBytes, bytes,
-                                 &a_full[bs]);
                 }
             }
             const uint32_t issued = g;
             for (uint32_t q = issued > (uint32_t)nB ? issued - (uint32_t)nB : 0u; q < issued; ++q)
-                tc::mbar_wait(&a_full[q % (uint32_t)nB], (q / (uint32_t)nB) & 1u, kWaitLimit);
+                tc::mbar_wait(&b_full[q % (uint32_t)nB], (q / (uint32_t)nB) & 1u, kWaitLimit);
         }
     } else if (warp == kMmaWarp) {
         // ---------------- MMA issue ----------------
-        if (lane == 0) {
-            uint32_t g = 0, it = 0;
-            bool stop_m = false;
-            int64_t off = 0;
-            for (int b = 0; b < tab.n() && !stop_m; ++b) {
-                const ChainArgs& ch = tab[b];
-                if (!chain_on_tiles(ch, dbg)) continue;
-                int first, cnt;
-                chain_tiles(off, ch.tile_T, first, cnt);
-                off += ch.tile_T;
-                const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)tile_ntot(ch.sc->K));
-                for (int i = 0; i < cnt && !stop_m; ++i, ++it) {
-                    if (*err) {
-                        stop_m = true;
-                        break;
-                    }
-                    const uint32_t buf = it & 1;
-                    if (it >= 2 &&
-                        !tc::mbar_wait(&acc_empty[buf], ((it >> 1) - 1) & 1, kWaitLimit)) {
-                        *err = DPMM_ETIMEOUT;
-                        stop_m = true;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    const uint32_t acc = tmem + buf * 256u;
-                    for (int c = 0; c < ch.tile_C; ++c) {
-                        const int st = (int)(g % (uint32_t)nS), bs = (int)(g % (uint32_t)nB);
-                        if (!tc::mbar_wait(&a_full[st], (g / (uint32_t)nS) & 1u, kWaitLimit)) {
-                            *err = DPMM_ETIMEOUT;
-                            stop_m = true;
-                            break;
-                        }
-                        tc::fence_after_sync();
-                        const uint32_t alo = tc::smem_addr(A_base + st * 32768);
-                        const uint32_t bsm = tc::smem_addr(B_base + bs * b_slot);
+        // An item costs this warp the latency of its instructions, not the tensor
+        // core's time, while N <= 128 (alone: four MMAs and a commit 200-260
+        // cycles, a wait for a barrier that is already complete another 200, 340
+        // beside busy producers; the tensor core needs 257 at N = 128, 480 at
+        // N = 240).  So the whole warp walks the items converged and an elected
+        // lane issues (from a branch of one lane the same sequence took 282, its
+        // waits 270 - 500), and one wait serves two items: lanes 0 - 3 poll the
+        // barriers of two A stages and their B stages side by side.
+        uint32_t st = 0, sph = 0, bs = 0, bph = 0;   // next A stage and B stage, their parities
+        uint32_t slot = 0, aph = 1;             // accumulator slot, its reads' parity
+        const uint64_t desc = tc::desc_sw128(0);
+        const uint32_t alo = tc::smem_addr(A_base) >> 4, blo = tc::smem_addr(B_base) >> 4;
+        const uint32_t hlo = tc::smem_addr(H_base) >> 4;
+        const uint32_t bstep = (uint32_t)(b_slot >> 4);
+        auto four = [&](uint32_t acc, uint32_t a, uint32_t bb, uint32_t idesc, uint32_t accum) {
+            const uint64_t ad = desc | a, bd = desc | bb;
+            tc::mma_f16(acc, ad, bd, idesc, accum);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            tc::mma_bf16(acc, tc::desc_sw128(alo + 32 * k),
-                                         tc::desc_sw128(bsm + 32 * k), idesc, (c | k) != 0);
-                        if (*reinterpret_cast<volatile uint32_t*>(stage_hib + 4 * st)) {
+            for (int k = 1; k < 4; ++k) tc::mma_f16(acc, ad + 2 * k, bd + 2 * k, idesc, 1u);
+        };
+        bool go = true;
+        int64_t off = 0;
+        for (int b = 0; b < tab.n() && go; ++b) {
+            const ChainArgs& ch = tab[b];
+            if (!chain_on_tiles(ch, dbg)) continue;
+            int first, cnt;
+            chain_tiles(off, ch.tile_T, first, cnt);
+            off += ch.tile_T;
+            const uint32_t ntot = (uint32_t)tile_ntot(ch.sc->K);
+            const uint32_t idesc = chain_half(ch) ? tc::idesc_f16(128, ntot)
+                                                  : tc::idesc_bf16(128, ntot);
+            const bool planes = chain_planes(ch);
+            const int C = ch.tile_C;
+            for (int i = 0; i < cnt && go; i += kPair) {
+                const int m = min(kPair, cnt - i);
+                uint32_t acc[kPair] = {0u, 0u};
+                uint64_t* full[kPair] = {nullptr, nullptr};
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                tc::mma_bf16(acc, tc::desc_sw128(alo + 16384 + 32 * k),
-                                             tc::desc_sw128(bsm + 32 * k), idesc, 1u);
+                for (int p = 0; p < kPair; ++p) {
+                    if (p < m) {
+                        // the slot's previous tile has been read (at the slot's
+                        // first use the parity of the phase before the first)
+                        go = go && tc::mbar_wait_warp(&acc_empty[slot], aph, kWaitLimit);
+                        acc[p] = tmem + slot * ldN;
+                        full[p] = &acc_full[slot];
+                        if (++slot == nAcc) {
+                            slot = 0;
+                            aph ^= 1u;
                         }
-                        tc::mma_commit(&stage_free[st]);
-                        ++g;
                     }
-                    if (stop_m) break;
-                    tc::mma_commit(&acc_full[buf]);
                 }
-            }
-            // the MMAs of the last chunk have completed (and signalled) before exit
-            if (g > 0) {
-                const uint32_t l = g - 1;
-                tc::mbar_wait(&stage_free[l % (uint32_t)nS], (l / (uint32_t)nS) & 1u, kWaitLimit);
+                if (m == 1) acc[1] = acc[0];
+                tc::fence_after_sync();
+                go = go && __all_sync(0xFFFFFFFFu, *err == 0);
+                // Rounds of two items: a chunk of both tiles, or two chunks of one
+                // (the last may be one chunk alone).  Lanes 0 and 1 follow the
+                // round's A stages, 2 and 3 its B stages (lanes above 3 as lane
+                // 0): index, parity, step, limit, so that a round costs few
+                // instructions.
+                const uint32_t nb = (uint32_t)(kPair / m);      // B stages of a round
+                const int rounds = (C + (int)nb - 1) / (int)nb;
+                const bool isb = lane == 2 || lane == 3;
+                const uint32_t lim = isb ? (uint32_t)nB : (uint32_t)nS;
+                const uint32_t step = isb ? nb : 2u;
+                uint64_t* ring = isb ? b_full : a_full;
+                uint32_t idx = isb ? bs : st, ph = isb ? bph : sph;
+                if (lane == 1 || (lane == 3 && nb == 2)) ++idx;
+                if (idx >= lim) {
+                    idx -= lim;
+                    ph ^= 1u;
+                }
+                for (int rd = 0; rd < rounds && go; ++rd) {
+                    const bool two = m == kPair || 2 * rd + 1 < C;
+                    if (!two) {        // nothing comes for lanes 1 and 3
+                        idx = __shfl_sync(0xFFFFFFFFu, idx, lane & 2);
+                        ph = __shfl_sync(0xFFFFFFFFu, ph, lane & 2);
+                        if (lane > 3) idx = st, ph = sph;
+                    }
+                    go = tc::mbar_wait_warp(ring + idx, ph, kWaitLimit);
+                    if (!go) break;
+                    const int hq = planes && lane < 2
+                                       ? reinterpret_cast<volatile int32_t*>(stage_hi)[idx]
+                                       : 0;
+                    idx += step;
+                    if (idx >= lim) {
+                        idx -= lim;
+                        ph ^= 1u;
+                    }
+                    const uint32_t st1 = st + 1 == (uint32_t)nS ? 0 : st + 1;
+                    const uint32_t bs1 = nb == 1 ? bs : bs + 1 == (uint32_t)nB ? 0 : bs + 1;
+                    if (two && !(planes && __any_sync(0xFFFFFFFFu, hq != 0))) {
+                        if (tc::elect_one()) {
+                            four(acc[0], alo + st * (kStageBytes >> 4), blo + bs * bstep, idesc,
+                                 rd != 0);
+                            tc::mma_commit(&stage_free[st]);
+                            if (nb == 2) tc::mma_commit(&b_free[bs]);
+                            four(acc[1], alo + st1 * (kStageBytes >> 4), blo + bs1 * bstep, idesc,
+                                 (rd != 0) | (nb - 1u));
+                            tc::mma_commit(&stage_free[st1]);
+                            tc::mma_commit(&b_free[bs1]);
+                        }
+                        __syncwarp();
+                    } else {
+                        // one item, or one with a second plane
+#pragma unroll 1
+                        for (uint32_t x = 0; x < (two ? 2u : 1u) && go; ++x) {
+                            const uint32_t sx = x ? st1 : st, bx = x ? bs1 : bs;
+                            const uint32_t ax = x ? acc[1] : acc[0];
+                            const int h = __shfl_sync(0xFFFFFFFFu, hq, (int)x);
+                            if (tc::elect_one()) {
+                                four(ax, alo + sx * (kStageBytes >> 4), blo + bx * bstep, idesc,
+                                     (rd != 0) | (x & (nb - 1u)));
+                                tc::mma_commit(&stage_free[sx]);
+                            }
+                            __syncwarp();
+                            if (h) {
+                                const uint32_t hs = (uint32_t)(h - 1) % kHiStages;
+                                go = tc::mbar_wait_warp(&hi_full[hs],
+                                                        ((uint32_t)(h - 1) / kHiStages) & 1u,
+                                                        kWaitLimit);
+                                if (go && tc::elect_one()) {
+                                    four(ax, hlo + hs * (kStageBytes >> 4), blo + bx * bstep,
+                                         idesc, 1u);
+                                    tc::mma_commit(&hi_used[hs]);
+                                }
+                                __syncwarp();
+                                go = go && tc::mbar_wait_warp(&hi_used[hs],
+                                                              ((uint32_t)(h - 1) / kHiStages) & 1u,
+                                                              kWaitLimit);
+                                __threadfence_block();
+                                if (lane == 0) *hi_done = h;
+                            }
+                            if ((nb == 2 || x == 1) && tc::elect_one()) tc::mma_commit(&b_free[bx]);
+                            __syncwarp();
+                        }
+                    }
+                    const uint32_t na = two ? 2u : 1u;
+                    if ((st += na) >= (uint32_t)nS) {
+                        st -= (uint32_t)nS;
+                        sph ^= 1u;
+                    }
+                    if ((bs += two ? nb : 1u) >= (uint32_t)nB) {
+                        bs -= (uint32_t)nB;
+                        bph ^= 1u;
+                    }
+                }
+                if (go && tc::elect_one()) {
+                    tc::mma_commit(full[0]);
+                    if (m == kPair) tc::mma_commit(full[1]);
+                }
+                __syncwarp();
             }
         }
-    } else {
+        if (!go && lane == 0) *err = DPMM_ETIMEOUT;
+        // every MMA issued has completed (and signalled) before exit
+        if (tc::elect_one()) tc::mma_commit(drain);
+        __syncwarp();
+        tc::mbar_wait_warp(drain, 0u, kWaitLimit);
+    } else if (warp < kEpiWarps) {
         // ---------------- epilogue (warps 0-7) ----------------
         const int h = warp >> 2, qw = warp & 3;
         const int r = 32 * qw + lane;
@@ -655,33 +894,41 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                 slw[2 * i] = n > 0.0f ? logf(n) : -CUDART_INF_F;
                 slw[2 * i + 1] = n > 1.0f ? logf(n - 1.0f) : -CUDART_INF_F;
             }
-            for (int i = tid; i < 4 * K; i += 32 * kEpiWarps) wsq[i] = 0ull;
+            for (int i = tid; i < 8 * K; i += 32 * kEpiWarps) wsq[i] = 0u;
             tc::named_bar(kBarEpi, 32 * kEpiWarps);
             for (int ti = 0; ti < cnt; ++ti, ++it) {
                 const int tile = first + ti * (int)gridDim.x;
-                const uint32_t buf = it & 1, xb = it & 1;
+                const uint32_t slot = it % nAcc, xb = it & 1;
                 const int64_t cell = (int64_t)tile * 128 + r;
                 const bool live = cell < ch.N;
-                // this cell's noise for the first cluster group of the half (and
-                // half 1's eq. 8 noise), loaded before the accumulator is ready
-                float gpre[8], gs0 = 0.0f, gs1 = 0.0f;
+                // this cell's noise and old state, loaded before the accumulator is
+                // ready (clusters 16 j + 8 h .. + 7 for this half)
+                float gq[kEpiGroups][8], gs0 = 0.0f, gs1 = 0.0f;
+                uint32_t old = 0u;
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    gpre[i] = live && 8 * h + i < K ? __ldg(ch.noise + (size_t)(8 * h + i) * ch.N + cell)
-                                                    : 0.0f;
-                if (h == 1 && live) {
+                for (int j = 0; j < kEpiGroups; ++j)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int k = 16 * j + 8 * h + i;
+                        gq[j][i] = live && k < K ? __ldg(ch.noise + (size_t)k * ch.N + cell) : 0.0f;
+                    }
+                if (live) {
                     gs0 = __ldg(ch.noise + (size_t)K * ch.N + cell);
                     gs1 = __ldg(ch.noise + (size_t)(K + 1) * ch.N + cell);
+                    old = ch.state[cell];
                 }
-                const bool ok = tc::mbar_wait(&acc_full[buf], (it >> 1) & 1, kWaitLimit);
+                const bool ok = tc::mbar_wait(&acc_full[slot], (it / nAcc) & 1u, kWaitLimit);
                 if (!ok) *err = DPMM_ETIMEOUT;
                 tc::fence_after_sync();
                 const bool okw = __all_sync(0xFFFFFFFFu, ok);
-                const uint32_t trow = tmem + buf * 256u + ((uint32_t)(32 * qw) << 16);
+                const uint32_t trow = tmem + slot * ldN + ((uint32_t)(32 * qw) << 16);
                 float best = -CUDART_INF_F;
                 int c = h ? K : 0;   // half 1's "none" loses every tie
                 if (okw) {
-                    for (int q = h; q < S0 / 16; q += 2) {
+#pragma unroll
+                    for (int j = 0; j < kEpiGroups; ++j) {
+                        const int q = 2 * j + h;
+                        if (q >= S0 / 16) continue;
                         float v[16];
                         tc::tmem_ld16(trow + (uint32_t)(16 * q), v);
                         tc::tmem_ld_wait();
@@ -691,9 +938,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                             if (k < K) {
                                 const float sc = v[2 * i] + v[2 * i + 1];
                                 if (dbg && live) dbg_out[(size_t)cell * 3 * K + k] = sc;
-                                const float gk = q == h ? gpre[i]
-                                                 : (live ? __ldg(ch.noise + (size_t)k * ch.N + cell) : 0.0f);
-                                const float val = (spi[k] + sc) + gk;
+                                const float val = (spi[k] + sc) + gq[j][i];
                                 if (val > best) {
                                     best = val;
                                     c = k;
@@ -702,31 +947,26 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                         }
                     }
                 }
-                if (h == 1) {
-                    xbest[128 * xb + r] = best;
-                    xc[128 * xb + r] = c;
-                    xg0[128 * xb + r] = gs0;
-                    xg1[128 * xb + r] = gs1;
-                }
-                tc::fence_before_sync();
+                // both halves learn the winner: half 0's unless half 1's is larger
+                // (half 0's wins a tie with a lower index, half 1's otherwise)
+                xbest[128 * (2 * xb + h) + r] = best;
+                xc[128 * (2 * xb + h) + r] = c;
                 if (tid == 0) stop[xb] = *err;
                 tc::named_bar(kBarEpi, 32 * kEpiWarps);
                 if (stop[xb]) {
                     halt = true;
                     break;
                 }
-                if (h == 1) continue;
                 {
-                    const float b1 = xbest[128 * xb + r];
-                    const int c1 = xc[128 * xb + r];
-                    if (b1 > best || (b1 == best && c1 < c)) {
-                        best = b1;
-                        c = c1;
-                    }
+                    const float bo = xbest[128 * (2 * xb + (h ^ 1)) + r];
+                    const int co = xc[128 * (2 * xb + (h ^ 1)) + r];
+                    if (bo > best || (bo == best && co < c)) c = co;
                 }
+                // its sub-cluster scores: each half reads every other block of 16
+                // columns, the half that meets the cell's columns finishes it
                 float t0 = 0.0f, t1 = 0.0f;
                 const int s0 = S0 + 4 * c;
-                for (int q = S0 / 16; q < Ntot / 16; ++q) {
+                for (int q = S0 / 16 + h; q < Ntot / 16; q += 2) {
                     float v[16];
                     tc::tmem_ld16(trow + (uint32_t)(16 * q), v);
                     tc::tmem_ld_wait();
@@ -746,9 +986,12 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                         else { t0 = v[12] + v[13]; t1 = v[14] + v[15]; }
                     }
                 }
+                // this half has read the accumulator (both: the slot's next tile may
+                // start)
                 tc::fence_before_sync();
-                if (live && !dbg) {
-                    const uint32_t old = ch.state[cell];
+                tc::named_bar(kBarHalf + h, 128);
+                if (qw == 0 && lane == 0) tc::mbar_arrive(&acc_empty[slot]);
+                if (live && !dbg && (((s0 >> 4) - S0 / 16) & 1) == h) {
                     const bool stays = state_label(old) == (uint32_t)c;
                     const uint32_t so = state_sub(old);
                     const float lw0 = slw[4 * c + (stays && so == 0 ? 1 : 0)];
@@ -756,22 +999,22 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                     const bool both_empty = lw0 == -CUDART_INF_F && lw1 == -CUDART_INF_F;
                     const float l0 = (both_empty ? 0.0f : lw0) + t0;
                     const float l1 = (both_empty ? 0.0f : lw1) + t1;
-                    const uint32_t s =
-                        (l1 + xg1[128 * xb + r] > l0 + xg0[128 * xb + r]) ? 1u : 0u;
+                    const uint32_t s = (l1 + gs1 > l0 + gs0) ? 1u : 0u;
                     const float mx = fmaxf(l0, l1), mn = fminf(l0, l1);
                     const float logq = (s ? l1 : l0) - (mx + log1pf(expf(mn - mx)));
                     ch.state[cell] = pack_state((uint32_t)c, s);
-                    atomicAdd(&wsq[qw * K + c], logq_fixed(logq));
+                    add_words64(wsq + 2 * (qw * K + c), logq_fixed(logq));
                 }
-                tc::named_bar(kBarLabel, 128);
-                if (tid == 0) tc::mbar_arrive(&acc_empty[buf]);
             }
             if (halt) break;
             // this chain's sum log q (per cluster, over its tiles of this block)
             tc::named_bar(kBarEpi, 32 * kEpiWarps);
             if (!dbg)
                 for (int k = tid; k < K; k += 32 * kEpiWarps) {
-                    const unsigned long long v = wsq[k] + wsq[K + k] + wsq[2 * K + k] + wsq[3 * K + k];
+                    unsigned long long v = 0ull;
+                    for (int w = 0; w < 4; ++w)
+                        v += (unsigned long long)wsq[2 * (w * K + k)] +
+                             ((unsigned long long)wsq[2 * (w * K + k) + 1] << 32);
                     if (v) atomicAdd(&ch.acc_logq[k], v);
                 }
         }
@@ -943,9 +1186,8 @@ cudaError_t launch_build_b(Ctx& c, bool force) {
     });
 }
 
-// A/B stages of the label kernel: four for one chain; two for a batch, where
-// the shared memory freed goes to more row-segment slots (measured faster on
-// 64 datasets: 2.85 against 3.18 ms per step), unless tuned.
+// A stages of the label kernel (see k_assign_tc): 4 for one chain, 2 for a
+// batch, unless tuned; they differ only where neither eight nor six stages fit.
 int32_t tile_label_stages(const Ctx& c) {
     return c.tune_tile_stages ? c.tune_tile_stages : (c.nchains > 1 ? 2 : 4);
 }

@@ -133,11 +133,6 @@ __host__ __device__ __forceinline__ int tile_ntot(int K) { return (tile_s0(K) + 
 // beyond FP16's range, then BF16 (to 2^-16, counts to 255 in one plane).
 __device__ __forceinline__ bool chain_half(const ChainArgs& ch) { return !ch.sc->wide_params; }
 
-// Some segments of the chain have a second plane (counts beyond the lo digit).
-__device__ __forceinline__ bool chain_planes(const ChainArgs& ch) {
-    return ch.max_count > (chain_half(ch) ? 2047 : 255);
-}
-
 __device__ __forceinline__ uint16_t f16_bits_rn(float f) {
     return __half_as_ushort(__float2half_rn(f));
 }
@@ -257,9 +252,6 @@ k_build_b(const __grid_constant__ Tab tab, int32_t force, int32_t rb) {
 // list (chain order) dealt round-robin to the CTAs: chain b's tiles handled
 // by this CTA are first, first + gridDim.x, ... (cnt of them), where off is
 // the number of listed tiles before chain b.
-__device__ __forceinline__ bool chain_on_tiles(const ChainArgs& ch, bool dbg) {
-    return ch.tile_enabled && tile_usable(ch.sc->K) && (dbg || ch.sc->tile_used);
-}
 __device__ __forceinline__ void chain_tiles(int64_t off, int T, int& first, int& cnt) {
     const int64_t G = gridDim.x;
     first = (int)((((int64_t)blockIdx.x - off) % G + G) % G);
@@ -367,6 +359,96 @@ __device__ __forceinline__ void clear_quarter(unsigned char* A, int q, int lane)
     __syncwarp();
 }
 
+// A chain's tiles for one CTA: first, first + gridDim.x, ... (cnt of them).
+struct TileJob {
+    int32_t b, first, cnt;
+    uint32_t k;      // K | FP16 operands << 16 | second planes << 17
+    __device__ __forceinline__ int K() const { return (int)(k & 0xFFFFu); }
+    __device__ __forceinline__ bool half() const { return (k >> 16) & 1u; }
+    __device__ __forceinline__ bool planes() const { return (k >> 17) & 1u; }
+};
+
+// The jobs of this CTA in chain order (called by the whole block; jobs and
+// scratch, 68 words: shared memory).  A batch's chains are read side by side, one thread each: the roles
+// used to walk the table themselves, three dependent loads a chain for each of
+// them.
+template <class Tab>
+__device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* jobs, int& njobs,
+                                          uint32_t& total, int& ntot_max, int& lslot_max,
+                                          bool& planes_any, int32_t* scratch) {
+    if (tab.n() == 1) {     // one chain: every thread by itself
+        const ChainArgs& ch = tab[0];
+        const int K = ch.sc->K, used = ch.sc->tile_used, wide = ch.sc->wide_params;
+        if (!ch.tile_enabled || !tile_usable(K) || !(dbg || used)) return;
+        TileJob job{0, 0, 0, (uint32_t)K | (wide ? 0u : 1u << 16) |
+                                 (ch.max_count > (wide ? 255 : 2047) ? 1u << 17 : 0u)};
+        chain_tiles(0, ch.tile_T, job.first, job.cnt);
+        if (!job.cnt) return;
+        if (threadIdx.x == 0) jobs[0] = job;
+        njobs = 1;
+        total = (uint32_t)job.cnt * (uint32_t)ch.tile_C;
+        ntot_max = tile_ntot(K);
+        lslot_max = max(4, ch.tile_Lslot);
+        planes_any = job.planes();
+        return;
+    }
+    int32_t *wtiles = scratch, *wjobs = wtiles + 32, *smax = wjobs + 32;   // [32], [32], [4]
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = (int)(blockDim.x >> 5);
+    if (tid < 4) smax[tid] = 0;      // items, ntot, lslot, planes
+    int64_t tiles_before = 0;
+    for (int b0 = 0; b0 < tab.n(); b0 += blockDim.x) {
+        const int b = b0 + tid;
+        int T = 0, lslot = 0;
+        uint32_t k = 0;
+        if (b < tab.n()) {
+            const ChainArgs& ch = tab[b];
+            const bool enabled = ch.tile_enabled;
+            const int K = ch.sc->K, used = ch.sc->tile_used, wide = ch.sc->wide_params;
+            if (enabled && tile_usable(K) && (dbg || used)) {
+                T = ch.tile_T;
+                lslot = ch.tile_Lslot;
+                k = (uint32_t)K | (wide ? 0u : 1u << 16) |
+                    (ch.max_count > (wide ? 255 : 2047) ? 1u << 17 : 0u);
+            }
+        }
+        int x = T;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wtiles[w] = x;
+        __syncthreads();
+        int64_t off = tiles_before + x - T;
+        for (int i = 0; i < nw; ++i) {
+            if (i < w) off += wtiles[i];
+            tiles_before += wtiles[i];
+        }
+        int first = 0, cnt = 0;
+        if (T) chain_tiles(off, T, first, cnt);
+        const unsigned own = __ballot_sync(0xFFFFFFFFu, cnt > 0);
+        if (lane == 0) wjobs[w] = __popc(own);
+        __syncthreads();
+        int pos = njobs + __popc(own & ((1u << lane) - 1u));
+        for (int i = 0; i < nw; ++i) {
+            if (i < w) pos += wjobs[i];
+            njobs += wjobs[i];
+        }
+        if (cnt > 0) {
+            jobs[pos] = TileJob{b, first, cnt, k};
+            atomicAdd(&smax[0], cnt);
+            atomicMax(&smax[1], tile_ntot((int)(k & 0xFFFFu)));
+            atomicMax(&smax[2], lslot);
+            if (k >> 17) smax[3] = 1;
+        }
+        __syncthreads();
+    }
+    total = (uint32_t)smax[0] * (uint32_t)tab[0].tile_C;
+    ntot_max = smax[1];
+    lslot_max = max(4, smax[2]);
+    planes_any = smax[3] != 0;
+}
+
 // A 64-bit sum kept as two 32-bit words in shared memory (the 32-bit shared
 // atomics are single instructions, the 64-bit one is a loop).
 __device__ __forceinline__ void add_words64(uint32_t* w, unsigned long long v) {
@@ -389,25 +471,16 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool dbg = dbg_out != nullptr;
-    // this CTA's work and the largest operand / segment over the chains
+    // this CTA's chains with their tiles, and the largest operand / segment
+    TileJob* jobs = reinterpret_cast<TileJob*>(base);
     uint32_t total = 0;   // items of this block
-    int ntot_max = 0, lslot_max = 4;
+    int njobs = 0, ntot_max = 0, lslot_max = 4;
     bool planes_any = false;
-    {
-        int64_t off = 0;
-        for (int b = 0; b < tab.n(); ++b) {
-            const ChainArgs& ch = tab[b];
-            if (!chain_on_tiles(ch, dbg)) continue;
-            int first, cnt;
-            chain_tiles(off, ch.tile_T, first, cnt);
-            off += ch.tile_T;
-            total += (uint32_t)cnt * (uint32_t)ch.tile_C;
-            ntot_max = max(ntot_max, tile_ntot(ch.sc->K));
-            lslot_max = max(lslot_max, ch.tile_Lslot);
-            planes_any = planes_any || chain_planes(ch);
-        }
-    }
+    list_jobs(tab, dbg, jobs, njobs, total, ntot_max, lslot_max, planes_any,
+              reinterpret_cast<int32_t*>(smem_raw + smem_bytes - 512));
     if (total == 0) return;
+    base += ((int64_t)njobs * sizeof(TileJob) + 1023) & ~(int64_t)1023;
+    const int C = tab[0].tile_C;     // (the chains share D)
     // shared-memory plan (identical in every thread): A stages, B stages,
     // segment slots, then the small area
     const int64_t b_slot = ((int64_t)ntot_max * 128 + 1023) & ~(int64_t)1023;
@@ -519,18 +592,13 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         uint32_t es = (uint32_t)set % (uint32_t)nE, eph = 0u;
         uint32_t g = set < nsets ? (uint32_t)set : total;
         uint32_t gend = 0;        // items before the end of the current chain
-        int b = -1;
-        int64_t off = 0;
+        int jb = -1;
         bool half = false;
         for (; g < total; g += (uint32_t)nsets) {
             while (g >= gend) {   // the chain of item g: its operand format
-                const ChainArgs& ch = tab[++b];
-                if (!chain_on_tiles(ch, dbg)) continue;
-                int first, cnt;
-                chain_tiles(off, ch.tile_T, first, cnt);
-                off += ch.tile_T;
-                gend += (uint32_t)cnt * (uint32_t)ch.tile_C;
-                half = chain_half(ch);
+                const TileJob job = jobs[++jb];
+                gend += (uint32_t)job.cnt * (uint32_t)C;
+                half = job.half();
             }
             unsigned char* A = A_base + st * kStageBytes;
             // (at a stage's first use the parity of the phase before the first)
@@ -597,28 +665,25 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         uint32_t hseq = 0;     // second planes started
         const unsigned lanemask = (1u << lane) - 1u;
         bool stop_l = false;
-        int64_t off = 0;
-        for (int b = 0; b < tab.n() && !stop_l; ++b) {
-            const ChainArgs& ch = tab[b];
-            if (!chain_on_tiles(ch, dbg)) continue;
-            int first, cnt;
-            chain_tiles(off, ch.tile_T, first, cnt);
-            off += ch.tile_T;
-            const uint32_t C = (uint32_t)ch.tile_C;
-            const uint32_t nitem = (uint32_t)cnt * C;
-            const bool half = chain_half(ch);
+        for (int jn = 0; jn < njobs && !stop_l; ++jn) {
+            const TileJob job = jobs[jn];
+            const ChainArgs& ch = tab[job.b];
+            const int first = job.first, cnt = job.cnt;
+            const uint32_t Cu = (uint32_t)C;
+            const uint32_t nitem = (uint32_t)cnt * Cu;
+            const bool half = job.half();
             // lane l < nsets takes the items l, l + nsets, ...: their five
             // quarter pointers, read one round ahead
             auto seg_ptrs = [&](uint32_t j, int32_t (&p)[6]) {
 #pragma unroll
                 for (int k = 0; k < 6; ++k) p[k] = 0;
                 if (lane < nsets && j < nitem) {
-                    const uint32_t pr = j / (kPair * C);           // pair, then chunk, then tile
+                    const uint32_t pr = j / (kPair * Cu);          // pair, then chunk, then tile
                     const uint32_t m = min((uint32_t)kPair, (uint32_t)cnt - kPair * pr);
-                    const uint32_t r = j - pr * kPair * C, ci = r / m;
+                    const uint32_t r = j - pr * kPair * Cu, ci = r / m;
                     const int64_t sgm =
                         ((int64_t)first + (int64_t)(kPair * pr + (r - ci * m)) * gridDim.x) *
-                            (int64_t)C + ci;
+                            (int64_t)Cu + ci;
 #pragma unroll
                     for (int k = 0; k < 5; ++k) p[k] = __ldg(ch.tile_ptr + 4 * sgm + k);
                     // the segment's second-plane flag, then the pointers
@@ -676,16 +741,12 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         if (lane == 0) {
             uint32_t g = 0, bs = 0, bph = 0;    // chunks started
             bool stop_b = false;
-            int64_t off = 0;
-            for (int b = 0; b < tab.n() && !stop_b; ++b) {
-                const ChainArgs& ch = tab[b];
-                if (!chain_on_tiles(ch, dbg)) continue;
-                int first, cnt;
-                chain_tiles(off, ch.tile_T, first, cnt);
-                off += ch.tile_T;
-                const uint32_t bytes = (uint32_t)tile_ntot(ch.sc->K) * 128u;
-                for (int i = 0; i < cnt && !stop_b; i += kPair) {
-                    for (int c = 0; c < ch.tile_C; ++c, ++g) {
+            for (int jn = 0; jn < njobs && !stop_b; ++jn) {
+                const TileJob job = jobs[jn];
+                const unsigned char* B = tab[job.b].tile_B;
+                const uint32_t bytes = (uint32_t)tile_ntot(job.K()) * 128u;
+                for (int i = 0; i < job.cnt && !stop_b; i += kPair) {
+                    for (int c = 0; c < C; ++c, ++g) {
                         if (g >= (uint32_t)nB &&
                             !tc::mbar_wait(&b_free[bs], bph ^ 1u, kWaitLimit)) {
                             *err = DPMM_ETIMEOUT;
@@ -697,7 +758,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                             break;
                         }
                         tc::mbar_arrive_expect_tx(&b_full[bs], bytes);
-                        tc::bulk_g2s(B_base + bs * b_slot, ch.tile_B + (size_t)c * kBChunkBytes,
+                        tc::bulk_g2s(B_base + bs * b_slot, B + (size_t)c * kBChunkBytes,
                                      bytes, &b_full[bs]);
                         if (++bs == (uint32_t)nB) {
                             bs = 0;
@@ -733,18 +794,13 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             for (int k = 1; k < 4; ++k) tc::mma_f16(acc, ad + 2 * k, bd + 2 * k, idesc, 1u);
         };
         bool go = true;
-        int64_t off = 0;
-        for (int b = 0; b < tab.n() && go; ++b) {
-            const ChainArgs& ch = tab[b];
-            if (!chain_on_tiles(ch, dbg)) continue;
-            int first, cnt;
-            chain_tiles(off, ch.tile_T, first, cnt);
-            off += ch.tile_T;
-            const uint32_t ntot = (uint32_t)tile_ntot(ch.sc->K);
-            const uint32_t idesc = chain_half(ch) ? tc::idesc_f16(128, ntot)
-                                                  : tc::idesc_bf16(128, ntot);
-            const bool planes = chain_planes(ch);
-            const int C = ch.tile_C;
+        for (int jn = 0; jn < njobs && go; ++jn) {
+            const TileJob job = jobs[jn];
+            const int cnt = job.cnt;
+            const uint32_t ntot = (uint32_t)tile_ntot(job.K());
+            const uint32_t idesc = job.half() ? tc::idesc_f16(128, ntot)
+                                              : tc::idesc_bf16(128, ntot);
+            const bool planes = job.planes();
             for (int i = 0; i < cnt && go; i += kPair) {
                 const int m = min(kPair, cnt - i);
                 uint32_t acc[kPair] = {0u, 0u};
@@ -876,15 +932,10 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         const int r = 32 * qw + lane;
         uint32_t it = 0;
         bool halt = false;
-        int64_t off = 0;
-        for (int b = 0; b < tab.n() && !halt; ++b) {
-            const ChainArgs& ch = tab[b];
-            if (!chain_on_tiles(ch, dbg)) continue;
-            int first, cnt;
-            chain_tiles(off, ch.tile_T, first, cnt);
-            off += ch.tile_T;
-            if (!cnt) continue;
-            const int K = ch.sc->K;
+        for (int jn = 0; jn < njobs && !halt; ++jn) {
+            const TileJob job = jobs[jn];
+            const ChainArgs& ch = tab[job.b];
+            const int first = job.first, cnt = job.cnt, K = job.K();
             const int S0 = tile_s0(K), Ntot = tile_ntot(K);
             // this chain's log pi, eq. 8 weights and log q sums in shared memory
             tc::named_bar(kBarEpi, 32 * kEpiWarps);
@@ -1023,8 +1074,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     tc::fence_after_sync();
     if (warp == 0) tc::tmem_dealloc(tmem, 512);
     if (*err && tid == 0)
-        for (int b = 0; b < tab.n(); ++b)
-            if (chain_on_tiles(tab[b], dbg)) atomicExch(&tab[b].sc->error, *err);
+        for (int jn = 0; jn < njobs; ++jn) atomicExch(&tab[jobs[jn].b].sc->error, *err);
 }
 
 // Statistics n-bar[k][r], S-bar[k][r][u] of the sweep's labels (from either

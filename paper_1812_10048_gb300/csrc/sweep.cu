@@ -25,6 +25,8 @@
 // k_debug_scores (scores of selected cells, a test hook).
 #include <math_constants.h>
 
+#include <cooperative_groups.h>
+
 #include <climits>
 
 #include "common.cuh"
@@ -121,54 +123,81 @@ __global__ void k_open_slot(const __grid_constant__ Tab tab) {
 
 // Rows 0 .. 3K-1 are theta rows (row 3k + p: cluster k for p = 0, its
 // sub-cluster p - 1 otherwise); row 3K is the pi row.  log G is kept in the
-// block's cache (D <= kDrawCache; else in the output slot), then normalised
+// block's cache (kDrawCache genes; else in the output slot), then normalised
 // into the output (log theta = log G - logsumexp).  With an appended K+1
 // candidate (open = 1) the alpha entry of pi is the candidate's weight and
 // there is no remainder entry (log pi_K = -inf).
+//
+// A row is drawn by a cluster of CS blocks, block r taking genes r Dc ..
+// (Dc = D / CS rounded up): the maximum and the sum of the logsumexp cross the
+// cluster through distributed shared memory, in rank order.  One block a row
+// left most SMs idle where a chain has few clusters and many genes (19 rows of
+// 32,738 genes: 164 us with one block a row, 43 us with eight); CS comes
+// from D (draw_cluster), so a chain's values do not depend on what it is
+// batched with.
 constexpr int kDrawCache = 8192;
 // Row stride (in pairs) of the staged table: K rounded up to odd, so that
 // the pairs of one cluster for 32 random genes spread over 16 bank pairs.
 __host__ __device__ __forceinline__ int staged_ld(int K) { return K | 1; }
 
+// A value of every block of the cluster combined in rank order; slot: this
+// block's shared-memory word, rewritten only after another exchange's barrier.
+template <int CS, class Op>
+__device__ __forceinline__ float cluster_combine(float v, float* slot, Op op) {
+    if (CS == 1) return v;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    if (threadIdx.x == 0) *slot = v;
+    cl.sync();
+    float r = *cl.map_shared_rank(slot, 0);
+#pragma unroll
+    for (int i = 1; i < CS; ++i) r = op(r, *cl.map_shared_rank(slot, i));
+    return r;
+}
+
 // compact: when not null (local iterations), the sub-cluster rows are also
 // written to it as [D][K | 1] pairs, the local kernel's shared-memory layout.
+template <int CS>
 __device__ __forceinline__ void draw_row(const ChainArgs& ch, int K, int open, uint32_t theta_tag,
-                                         uint32_t t, int row, float* red, float* lgc,
-                                         float* compact = nullptr) {
+                                         uint32_t t, int row, float* red, float* lgc, float* cx,
+                                         int rank, float* compact = nullptr) {
     const int D = ch.D, kmax = ch.kmax;
     const float beta = (float)ch.beta, alpha = (float)ch.alpha;
     const Stream& st = ch.st;
     if (row < 3 * K) {
         const int k = row / 3, p = row % 3;
+        const int Dc = (D + CS - 1) / CS, u0 = min(D, rank * Dc), u1 = min(D, u0 + Dc);
         const uint32_t* S0 = ch.Ssub + (size_t)(2 * k) * D;
         const uint32_t* S1 = S0 + D;
         float* Lc = ch.Lc;
         float* Ls = ch.Ls;
-        const bool cached = D <= kDrawCache;
+        const bool cached = Dc <= kDrawCache;
         auto slot = [&](int u) -> float* {
             return p == 0 ? &Lc[(size_t)u * kmax + k] : &Ls[((size_t)u * kmax + k) * 2 + (p - 1)];
         };
         float mx = -CUDART_INF_F;
-        for (int u = threadIdx.x; u < D; u += blockDim.x) {
+        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
             const uint32_t S = p == 0 ? S0[u] + S1[u] : (p == 1 ? S0[u] : S1[u]);
             const float lg = log_gamma_draw(st, theta_tag, beta + (float)S,
                                             (uint32_t)row * (uint32_t)D + (uint32_t)u, t);
-            if (cached) lgc[u] = lg;
+            if (cached) lgc[u - u0] = lg;
             else *slot(u) = lg;
             mx = fmaxf(mx, lg);
         }
         mx = block_reduce_max(mx, red);   // (its barrier also publishes lgc)
+        mx = cluster_combine<CS>(mx, cx, [](float a, float b) { return fmaxf(a, b); });
         float s = 0.0f;
-        for (int u = threadIdx.x; u < D; u += blockDim.x)
-            s += expf((cached ? lgc[u] : *slot(u)) - mx);
+        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x)
+            s += expf((cached ? lgc[u - u0] : *slot(u)) - mx);
         s = block_reduce_sum(s, red);
+        s = cluster_combine<CS>(s, cx + 1, [](float a, float b) { return a + b; });
         const float lse = mx + logf(s);
-        for (int u = threadIdx.x; u < D; u += blockDim.x) {
-            const float v = (cached ? lgc[u] : *slot(u)) - lse;
+        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
+            const float v = (cached ? lgc[u - u0] : *slot(u)) - lse;
             *slot(u) = v;
             if (compact && p != 0) compact[((size_t)u * staged_ld(K) + k) * 2 + (p - 1)] = v;
         }
-    } else {
+    } else if (rank == 0) {
         const uint32_t* nsub = ch.nsub;
         float* logpi = ch.logpi;
         const int Kc = K - open;   // clusters with cells; entry Kc takes alpha
@@ -189,23 +218,75 @@ __device__ __forceinline__ void draw_row(const ChainArgs& ch, int K, int open, u
     }
 }
 
+// One chain's label noise over the blocks of the draw kernel, the first `busy` of
+// which have drawn rows of `genes` genes each: the shares make a row block's
+// genes and Gumbels add up to another block's Gumbels (a Gamma draw costs about
+// four Gumbels), so that little noise goes to the blocks without rows alone
+// and much of it to all (1.3 M cells, K = 40, 54.6 M Gumbels: 194 us with the
+// blocks without rows alone, 135 us shared).
+__device__ __forceinline__ void noise_after_rows(const ChainArgs& ch, int K, int busy, int genes) {
+    if (!noise_wanted(ch, K)) return;
+    // (32-bit divisions: the 64-bit ones cost the idle blocks 2 us)
+    const uint32_t N = (uint32_t)ch.N, G = gridDim.x, idle = G - (uint32_t)busy;
+    const float per = (float)(K + 2), row = 4.0f * (float)genes;
+    if (idle && (float)N * per < (float)idle * row) {
+        // the first blocks without rows, whole: they lie on SMs of their own
+        // (spread thinly over all blocks the noise slowed the rows by 2 us)
+        if (blockIdx.x >= (uint32_t)busy)
+            noise_cells(ch, (int64_t)(blockIdx.x - (uint32_t)busy) * blockDim.x + threadIdx.x,
+                        ch.N, (int64_t)idle * blockDim.x);
+        return;
+    }
+    const float load = ((float)N * per + (float)busy * row) / (float)G;
+    uint32_t xr = 0, xi = 0;           // cells of a block with a row, of one without
+    if (!idle) {
+        xr = (N - 1u) / G + 1u;
+    } else {
+        if (load > row) xr = min((uint32_t)((load - row) / per), N / G);
+        xi = (N - xr * (uint32_t)busy + idle - 1u) / idle;
+    }
+    const uint32_t b = blockIdx.x;
+    const bool free_block = b >= (uint32_t)busy;
+    const int64_t c0 = free_block ? (int64_t)(b - (uint32_t)busy) * xi
+                                  : (int64_t)idle * xi + (int64_t)b * xr;
+    noise_cells(ch, min(ch.N, c0) + threadIdx.x, min(ch.N, c0 + (free_block ? xi : xr)),
+                blockDim.x);
+}
+
+// Blocks that read a block's exchange words have done so before it may exit.
+template <int CS>
+__device__ __forceinline__ void cluster_end() {
+    if (CS > 1) cooperative_groups::this_cluster().sync();
+}
+
 // The 3K + 1 rows of every chain form one list dealt round-robin to the
-// blocks.  The block that draws row 0 of a chain also selects the chain's
-// labelling engine and clears its n-bar / sum log q accumulators.  With
+// clusters of blocks.  The block that draws row 0 of a chain also selects the
+// chain's labelling engine and clears its n-bar / sum log q accumulators.  With
 // several chains (at most kDrawTable) the threads first read every chain's
 // K, open slot and counter side by side, so a block finds its rows without a
 // round trip per chain.
 constexpr int kDrawTable = 512;
 
-template <class Tab>
+template <class Tab, int CS>
 __global__ void __launch_bounds__(kDrawThreads)
 k_draw_params(const __grid_constant__ Tab tab) {
     __shared__ float red[32];
+    __shared__ float cx[2];
     __shared__ __align__(16) float lgc[kDrawCache];   // also the noise split's scratch
     __shared__ int32_t srow[kDrawTable + 1];           // rows before chain b
     __shared__ int32_t sK[kDrawTable], sopen[kDrawTable];
     __shared__ uint32_t st_[kDrawTable];
     const int n = tab.n();
+    const int rank = (int)blockIdx.x % CS, blk = (int)blockIdx.x / CS;
+    const int nblk = (int)gridDim.x / CS;
+    auto first_row = [&](const ChainArgs& ch, int K) {
+        if (rank) return;
+        if (threadIdx.x == 0) {
+            select_engine(ch.sc, K, ch);
+            ch.sc->wide_params = ch.wide_beta;
+        }
+        clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
+    };
     if (n > 1 && n <= kDrawTable) {
         const int b = threadIdx.x;
         int rows = 0;
@@ -237,24 +318,19 @@ k_draw_params(const __grid_constant__ Tab tab) {
         __syncthreads();
         const int total = srow[n];
         int c = 0;
-        for (int id = blockIdx.x; id < total; id += gridDim.x) {
+        for (int id = blk; id < total; id += nblk) {
             while (srow[c + 1] <= id) ++c;
             const ChainArgs& ch = tab[c];
             const int row = id - srow[c], K = sK[c];
-            if (row == 0) {
-                if (threadIdx.x == 0) {
-                    select_engine(ch.sc, K, ch);
-                    ch.sc->wide_params = ch.wide_beta;
-                }
-                clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
-            }
-            draw_row(ch, K, sopen[c], TAG_THETA, st_[c], row, red, lgc);
+            if (row == 0) first_row(ch, K);
+            draw_row<CS>(ch, K, sopen[c], TAG_THETA, st_[c], row, red, lgc, cx, rank);
             __syncthreads();
         }
-        const int64_t free0 = total < (int)gridDim.x ? total : 0;
+        const int64_t free0 = total < nblk ? (int64_t)total * CS : 0;
         if ((int64_t)blockIdx.x >= free0)
             fill_noise(tab, (int64_t)gridDim.x - free0, (int64_t)blockIdx.x - free0,
                        reinterpret_cast<long long*>(lgc));
+        cluster_end<CS>();
         return;
     }
     int64_t base = 0;
@@ -264,30 +340,28 @@ k_draw_params(const __grid_constant__ Tab tab) {
         const int open = ch.open_new ? ch.sc->open_slot : 0;
         const uint32_t t = ch.sc->t;
         const int rows = 3 * K + 1;
-        int64_t first = base + (((int64_t)blockIdx.x - base) % gridDim.x + gridDim.x) % gridDim.x;
-        for (int64_t id = first; id < base + rows; id += gridDim.x) {
+        int64_t first = base + (((int64_t)blk - base) % nblk + nblk) % nblk;
+        for (int64_t id = first; id < base + rows; id += nblk) {
             const int row = (int)(id - base);
-            if (row == 0) {
-                if (threadIdx.x == 0) {
-                    select_engine(ch.sc, K, ch);
-                    ch.sc->wide_params = ch.wide_beta;
-                }
-                clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
-            }
-            draw_row(ch, K, open, TAG_THETA, t, row, red, lgc);
+            if (row == 0) first_row(ch, K);
+            draw_row<CS>(ch, K, open, TAG_THETA, t, row, red, lgc, cx, rank);
             __syncthreads();
         }
         base += rows;
     }
-    // the label noise: blocks without a row take it (all blocks when every
-    // block has rows); 2 n + 33 int64 of scratch fit the 32 KB cache for
-    // n <= 1,024 chains
+    // 2 n + 33 int64 of scratch fit the 32 KB cache for n <= 1,024 chains
     static_assert(sizeof(float) * kDrawCache >= sizeof(long long) * (2 * kDrawThreads + 33),
                   "noise scratch");
-    const int64_t free0 = base < gridDim.x ? base : 0;
-    if ((int64_t)blockIdx.x >= free0)
-        fill_noise(tab, (int64_t)gridDim.x - free0, (int64_t)blockIdx.x - free0,
-                   reinterpret_cast<long long*>(lgc));
+    if (n == 1) {
+        noise_after_rows(tab[0], (int)((base - 1) / 3), (int)min((int64_t)nblk, base) * CS,
+                         (tab[0].D + CS - 1) / CS);
+    } else {
+        const int64_t free0 = base < nblk ? base * CS : 0;
+        if ((int64_t)blockIdx.x >= free0)
+            fill_noise(tab, (int64_t)gridDim.x - free0, (int64_t)blockIdx.x - free0,
+                       reinterpret_cast<long long*>(lgc));
+    }
+    cluster_end<CS>();
 }
 
 // Local Gibbs iteration j >= 1 after a sweep (Section 2.3), first half: the
@@ -295,27 +369,32 @@ k_draw_params(const __grid_constant__ Tab tab) {
 // under the iteration's tag and the sweep's own counter t - 1 (the
 // compaction has advanced t).  The block of a chain's first row clears its
 // n-bar / sum log q accumulators.
-template <class Tab>
+template <class Tab, int CS>
 __global__ void __launch_bounds__(kDrawThreads)
 k_draw_local(const __grid_constant__ Tab tab, int32_t j) {
     __shared__ float red[32];
+    __shared__ float cx[2];
     __shared__ float lgc[kDrawCache];
     const uint32_t tag = kLocalTag0 + 2u * (uint32_t)(j - 1);
+    const int rank = (int)blockIdx.x % CS, blk = (int)blockIdx.x / CS;
+    const int nblk = (int)gridDim.x / CS;
     int64_t base = 0;
     for (int b = 0; b < tab.n(); ++b) {
         const ChainArgs& ch = tab[b];
         const int K = ch.sc->K;
         const uint32_t t = ch.sc->t - 1u;
         const int rows = 2 * K;
-        int64_t first = base + (((int64_t)blockIdx.x - base) % gridDim.x + gridDim.x) % gridDim.x;
-        for (int64_t id = first; id < base + rows; id += gridDim.x) {
+        int64_t first = base + (((int64_t)blk - base) % nblk + nblk) % nblk;
+        for (int64_t id = first; id < base + rows; id += nblk) {
             const int i = (int)(id - base);
-            if (i == 0) clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
-            draw_row(ch, K, 0, tag, t, 3 * (i >> 1) + 1 + (i & 1), red, lgc, ch.local_tab);
+            if (i == 0 && rank == 0) clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
+            draw_row<CS>(ch, K, 0, tag, t, 3 * (i >> 1) + 1 + (i & 1), red, lgc, cx, rank,
+                         ch.local_tab);
             __syncthreads();
         }
         base += rows;
     }
+    cluster_end<CS>();
 }
 
 // ---------------------------------------------------------------------------
@@ -1607,11 +1686,38 @@ cudaError_t configure_launches(Ctx& c) {
     return cudaSuccess;
 }
 
+// Blocks that draw one parameter row together: about 2,048 genes each, at most
+// eight (the portable cluster size).
+static int draw_cluster(int32_t D) { return D <= 2048 ? 1 : D <= 4096 ? 2 : D <= 8192 ? 4 : 8; }
+
+// kernel(args...) on `blocks` blocks of kDrawThreads (a multiple of the cluster
+// size cs) in clusters of cs.
+template <class... Params, class... Args>
+static cudaError_t launch_draw(void (*kernel)(Params...), int cs, int blocks, cudaStream_t st,
+                               Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks / cs * cs);
+    cfg.blockDim = dim3(kDrawThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cs > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 cudaError_t launch_draw_params(Ctx& c) {
     return with_table(c, [&](auto tab) {
-        const int per_sm = c.tune_draw_per_sm ? c.tune_draw_per_sm : 2;
-        k_draw_params<<<per_sm * c.num_sms, kDrawThreads, 0, c.stream>>>(tab);
-        return cudaGetLastError();
+        using T = decltype(tab);
+        const int blocks = (c.tune_draw_per_sm ? c.tune_draw_per_sm : 2) * c.num_sms;
+        const int cs = draw_cluster(c.D);
+        return launch_draw(cs == 1   ? k_draw_params<T, 1>
+                           : cs == 2 ? k_draw_params<T, 2>
+                           : cs == 4 ? k_draw_params<T, 4>
+                                     : k_draw_params<T, 8>,
+                           cs, blocks, c.stream, tab);
     });
 }
 
@@ -1637,7 +1743,14 @@ int32_t local_lanes(const Ctx& c) {
 // One local Gibbs iteration j >= 1 (after the sweep's compaction).
 cudaError_t launch_local_iteration(Ctx& c, int32_t j) {
     cudaError_t e = with_table(c, [&](auto tab) {
-        k_draw_local<<<2 * c.num_sms, kDrawThreads, 0, c.stream>>>(tab, j);
+        using T = decltype(tab);
+        const int cs = draw_cluster(c.D);
+        const cudaError_t ed = launch_draw(cs == 1   ? k_draw_local<T, 1>
+                                           : cs == 2 ? k_draw_local<T, 2>
+                                           : cs == 4 ? k_draw_local<T, 4>
+                                                     : k_draw_local<T, 8>,
+                                           cs, 2 * c.num_sms, c.stream, tab, j);
+        if (ed != cudaSuccess) return ed;
         const int lanes = local_lanes(c);
         const int32_t gf = c.tune_local_stream;
         const dim3 grid(c.num_sms);

@@ -159,6 +159,7 @@ ChainArgs dpmm::chain_args(const Ctx& c) {
     a.tile_C = c.tile_C;
     a.tile_T = c.tile_T;
     a.tile_Lslot = c.tile_Lslot;
+    a.tile_Lmean = c.tile_Lmean;
     // engine choice by measured density (constants in common.cuh); the tile
     // engine forced by the caller labels every 1 <= K <= 40
     const double density = (c.N > 0 && c.D > 0) ? (double)c.nnz / ((double)c.N * c.D) : 0.0;
@@ -512,6 +513,7 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
             return bail(fail(DPMM_EOVERFLOW, "the dense-tile copy needs %lld entries (> 2^31 - 1)",
                              scan[0]));
         c.tile_Lslot = (int32_t)scan[1];
+        c.tile_Lmean = (int32_t)((scan[0] + TC - 1) / TC);
         CKI(dalloc(&c.tile_ent, (size_t)scan[0]));
         CKI(cudaMemsetAsync(c.tile_ent, 0, sizeof(uint32_t) * std::max<long long>(1, scan[0]),
                             c.stream));

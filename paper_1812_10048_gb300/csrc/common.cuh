@@ -182,6 +182,7 @@ struct Ctx {
     bool tile_enabled = false;
     int32_t tile_T = 0, tile_C = 0;
     int32_t tile_Lslot = 0;         // longest padded segment, entries
+    int32_t tile_Lmean = 0;         // mean padded segment, entries (rounded up)
     uint32_t* tile_ent = nullptr;   // row << 22 | gene-in-chunk << 16 | count (0: padding)
     int32_t* tile_ptr = nullptr;    // [4 T C + 1] quarter starts
     unsigned char* tile_B = nullptr;  // per-sweep BF16 hi/lo table, [C][256 rows][64] swizzled
@@ -390,7 +391,7 @@ struct ChainArgs {
     unsigned char* move_part;
     int32_t* move_ticket;
     // dense-tile engine (tile_enabled = 0: not built for this chain)
-    int32_t tile_enabled, tile_C, tile_T, tile_Lslot;
+    int32_t tile_enabled, tile_C, tile_T, tile_Lslot, tile_Lmean;
     int32_t tile_kmin;    // smallest K the dense-tile engine labels (engine choice)
     int32_t max_count;    // largest count of the matrix
     int32_t wide_beta;    // drawn log theta values may lie beyond FP16's range

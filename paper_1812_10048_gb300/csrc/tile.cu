@@ -258,22 +258,27 @@ __device__ __forceinline__ void chain_tiles(int64_t off, int T, int& first, int&
     cnt = first < T ? (T - 1 - first) / (int)G + 1 : 0;
 }
 
-// Warp roles of the pipelined engine (27 warps):
+// Warp roles of the pipelined engine (32 warp numbers; 20, 24 and 28 idle):
 //   warps 0-7   epilogue, two halves of four warps over the same 128 cells
 //               (warp w reads TMEM lanes 32 (w % 4) ..): each half takes every
 //               other 8-cluster column group of the Gumbel-max, then (the
 //               winner exchanged) every other block of sub-cluster columns,
 //               and finishes the cells whose sub-cluster columns it met
-//   warps 8-23  producers, four sets of four warps taking items in turn
-//               (two sets when only two A stages fit); warp q of a set
-//               densifies rows 32q .. 32q + 31 of its item (the entries of
-//               one quarter) from the staged segment, so the four warps never
-//               wait on one another
-//   warp 24     issues the MMAs
-//   warp 25     segment loader: bulk-copies each item's entries into a ring
-//               of slots, one lane per producer set, reading the segment table
-//               a round ahead
-//   warp 26     lane 0 bulk-copies the B operand of each chunk into its ring
+//   warps from 8 with w % 4 != 0  producers, up to four sets of four warps
+//               taking items in turn; warp q of a set densifies rows 32q ..
+//               32q + 31 of its item (the entries of one quarter) from the
+//               staged segment, so the four warps never wait on one another
+//   warp 8      issues the MMAs
+//   warp 12     segment loader: bulk-copies each item's entries into a ring,
+//               one lane per producer set, reading the segment table a round
+//               ahead.  The items lie end to end in the ring: a few deep cells
+//               make one segment several times the mean, and slots of that
+//               size left room for fewer A stages (1.3 M x 2,000 with 2% deep
+//               cells: 1,557 us with slots, RING us)
+//   warp 16     lane 0 bulk-copies the B operand of each chunk into its ring
+// The roles that feed the tensor core are alone on their scheduler (w % 4 = 0)
+// but for two epilogue warps: each item costs them the latency of a chain of
+// instructions.
 // Every role walks the same sequence of items (tile, chunk): the chains in
 // order, this CTA's tiles of each chain in pairs, the chunks, and for each chunk
 // the tiles of the pair, so that one copy of a chunk's B operand serves both
@@ -369,13 +374,13 @@ struct TileJob {
 };
 
 // The jobs of this CTA in chain order (called by the whole block; jobs and
-// scratch, 68 words: shared memory).  A batch's chains are read side by side, one thread each: the roles
+// scratch, 69 words: shared memory).  A batch's chains are read side by side, one thread each: the roles
 // used to walk the table themselves, three dependent loads a chain for each of
 // them.
 template <class Tab>
 __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* jobs, int& njobs,
                                           uint32_t& total, int& ntot_max, int& lslot_max,
-                                          bool& planes_any, int32_t* scratch) {
+                                          int& lmean_max, bool& planes_any, int32_t* scratch) {
     if (tab.n() == 1) {     // one chain: every thread by itself
         const ChainArgs& ch = tab[0];
         const int K = ch.sc->K, used = ch.sc->tile_used, wide = ch.sc->wide_params;
@@ -389,16 +394,17 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
         total = (uint32_t)job.cnt * (uint32_t)ch.tile_C;
         ntot_max = tile_ntot(K);
         lslot_max = max(4, ch.tile_Lslot);
+        lmean_max = max(4, ch.tile_Lmean);
         planes_any = job.planes();
         return;
     }
-    int32_t *wtiles = scratch, *wjobs = wtiles + 32, *smax = wjobs + 32;   // [32], [32], [4]
+    int32_t *wtiles = scratch, *wjobs = wtiles + 32, *smax = wjobs + 32;   // [32], [32], [5]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = (int)(blockDim.x >> 5);
-    if (tid < 4) smax[tid] = 0;      // items, ntot, lslot, planes
+    if (tid < 5) smax[tid] = 0;      // tiles, ntot, lslot, planes, lmean
     int64_t tiles_before = 0;
     for (int b0 = 0; b0 < tab.n(); b0 += blockDim.x) {
         const int b = b0 + tid;
-        int T = 0, lslot = 0;
+        int T = 0, lslot = 0, lmean = 0;
         uint32_t k = 0;
         if (b < tab.n()) {
             const ChainArgs& ch = tab[b];
@@ -407,6 +413,7 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
             if (enabled && tile_usable(K) && (dbg || used)) {
                 T = ch.tile_T;
                 lslot = ch.tile_Lslot;
+                lmean = ch.tile_Lmean;
                 k = (uint32_t)K | (wide ? 0u : 1u << 16) |
                     (ch.max_count > (wide ? 255 : 2047) ? 1u << 17 : 0u);
             }
@@ -439,6 +446,7 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
             atomicAdd(&smax[0], cnt);
             atomicMax(&smax[1], tile_ntot((int)(k & 0xFFFFu)));
             atomicMax(&smax[2], lslot);
+            atomicMax(&smax[4], lmean);
             if (k >> 17) smax[3] = 1;
         }
         __syncthreads();
@@ -446,6 +454,7 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
     total = (uint32_t)smax[0] * (uint32_t)tab[0].tile_C;
     ntot_max = smax[1];
     lslot_max = max(4, smax[2]);
+    lmean_max = max(4, smax[4]);
     planes_any = smax[3] != 0;
 }
 
@@ -474,9 +483,9 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // this CTA's chains with their tiles, and the largest operand / segment
     TileJob* jobs = reinterpret_cast<TileJob*>(base);
     uint32_t total = 0;   // items of this block
-    int njobs = 0, ntot_max = 0, lslot_max = 4;
+    int njobs = 0, ntot_max = 0, lslot_max = 4, lmean_max = 4;
     bool planes_any = false;
-    list_jobs(tab, dbg, jobs, njobs, total, ntot_max, lslot_max, planes_any,
+    list_jobs(tab, dbg, jobs, njobs, total, ntot_max, lslot_max, lmean_max, planes_any,
               reinterpret_cast<int32_t*>(smem_raw + smem_bytes - 512));
     if (total == 0) return;
     base += ((int64_t)njobs * sizeof(TileJob) + 1023) & ~(int64_t)1023;
@@ -484,17 +493,21 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // shared-memory plan (identical in every thread): A stages, B stages,
     // segment slots, then the small area
     const int64_t b_slot = ((int64_t)ntot_max * 128 + 1023) & ~(int64_t)1023;
-    const int64_t e_slot = (int64_t)lslot_max * 4;
+    const int64_t e_max = (int64_t)lslot_max * 4, e_mean = (int64_t)lmean_max * 4;
     const int64_t avail = smem_bytes - (int64_t)(base - smem_raw) - kSmallBytes;
-    // hi stages, only when some chain of the launch has a second plane
+    // hi stages, only when some chain of the block has a second plane
     const int64_t h_bytes = planes_any ? (int64_t)kHiStages * kStageBytes : 0;
-    // producer sets and A stages, the most that fit (a set takes every nsets-th
-    // item and always meets the same stages and slots, so nsets divides nS and
-    // nE: slot g % nE is then refilled for item g only after the same set
-    // consumed item g - nE, and a set's parity wait can never be two phases
-    // ahead).  Two stages a set let it fill one while the MMAs read the other.
+    // Producer sets and A stages, the most that fit beside a segment ring for two
+    // items of a set and the longest segment.  A set takes every nsets-th item
+    // and always meets the same stages and slots, so nsets divides nS and nE:
+    // slot g % nE is then refilled for item g only after the same set consumed
+    // item g - nE, and a set's parity wait can never be two phases ahead.  Two
+    // stages a set let it fill one while the MMAs read the other.
+    auto ring_left = [&](int stages, int b_stages) {
+        return avail - stages * (int64_t)kStageBytes - h_bytes - b_stages * b_slot;
+    };
     auto fit = [&](int sets, int stages) {
-        return stages * (int64_t)kStageBytes + h_bytes + 2 * b_slot + sets * e_slot <= avail;
+        return ring_left(stages, 2) >= max(e_max, 2 * sets * e_mean);
     };
     // 1.3 M x 2,000, K = 40: four sets of one stage 1,364 us, three of two
     // 1,288 us; 68,000 x 1,000, K = 10: four sets of two stages 37 us, three 41.
@@ -503,15 +516,20 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     else if (fit(3, 6)) nsets = 3, nS = 6;
     else if (stages_pref != 2 && fit(4, 4)) nsets = 4, nS = 4;
     else if (fit(2, 4)) nsets = 2, nS = 4;
-    // more than two B stages only where they leave eight segment slots
+    // more than two B stages only where they leave room for twelve segments
     int nB = 2;
-    while (nB < kMaxBStages &&
-           nS * (int64_t)kStageBytes + h_bytes + (nB + 1) * b_slot + 8 * e_slot <= avail)
-        ++nB;
-    const int nE_fit = (int)min((int64_t)kMaxESlots,
-                                (avail - nS * (int64_t)kStageBytes - h_bytes - nB * b_slot) / e_slot);
-    const int nE = (nE_fit / nsets) * nsets;
-    if (nE < 2) {
+    while (nB < kMaxBStages && ring_left(nS, nB + 1) >= max(e_max, 12 * e_mean)) ++nB;
+    const int64_t e_ring = ring_left(nS, nB) & ~(int64_t)15;
+    // items in the ring at most: as many as it nearly always has room for, so
+    // that a round seldom waits for more than its own slots
+    // (fixed slots for the longest segment where two a set fit: a round of the
+    // loader is shorter then; 68,000 x 1,000 39 -> 35 us, 8,000 x 32,738
+    // 191 -> 165 us, while the ring gives 89 -> 76 us for 24 datasets)
+    const bool fixed = e_ring >= 2 * nsets * e_max;
+    const int64_t e_item = fixed ? e_max : e_mean + e_mean / 4;
+    const int nE = (int)min((int64_t)(kMaxESlots / nsets),
+                            max((int64_t)2, e_ring / (e_item * nsets))) * nsets;
+    if (e_ring < e_max) {
         if (tid == 0) atomicExch(&tab[0].sc->error, DPMM_ECAPACITY);
         return;
     }
@@ -521,7 +539,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     unsigned char* H_base = A_base + nS * kStageBytes;
     unsigned char* B_base = H_base + h_bytes;
     unsigned char* E_base = B_base + nB * b_slot;
-    unsigned char* small = E_base + nE * e_slot;
+    unsigned char* small = E_base + e_ring;
     small = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(small) + 15) & ~(uintptr_t)15);
     int4* meta = reinterpret_cast<int4*>(small);                   // [kMaxESlots] quarter ends
     uint64_t* a_full = reinterpret_cast<uint64_t*>(meta + kMaxESlots);   // [kMaxStages]
@@ -539,7 +557,8 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     volatile int* err = reinterpret_cast<volatile int*>(taddr_s + 1);
     int* stop = const_cast<int*>(err) + 1;                          // [2]
     int32_t* stage_hi = stop + 2;                                   // [kMaxStages]
-    int32_t* meta_hi = stage_hi + kMaxStages;                       // [kMaxESlots]
+    int32_t* slot_off = stage_hi + kMaxStages;                      // [kMaxESlots] ring offsets
+    int32_t* meta_hi = slot_off + kMaxESlots;                       // [kMaxESlots]
     volatile int32_t* hi_done = meta_hi + kMaxESlots;               // second planes used up
     float* spi = reinterpret_cast<float*>(meta_hi + kMaxESlots + 1);    // [K]
     float* slw = spi + kTileMaxK;                                   // [4K]
@@ -615,7 +634,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             const int i0 = q == 0 ? 0 : q == 1 ? mt.x : q == 2 ? mt.y : mt.z;
             const int i1 = q == 0 ? mt.x : q == 1 ? mt.y : q == 2 ? mt.z : mt.w;
             const int hi = planes_any ? meta_hi[es] : 0;    // 0, or 1 + its number
-            const uint32_t* ring = reinterpret_cast<const uint32_t*>(E_base + es * e_slot);
+            const uint32_t* ring = reinterpret_cast<const uint32_t*>(E_base + slot_off[es]);
             if (half) scatter_entries<true, false, kScatter>(ring, i0, i1, q, lane, A);
             else scatter_entries<false, false, kScatter>(ring, i0, i1, q, lane, A);
             tc::fence_async_smem();
@@ -663,6 +682,9 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         // ---------------- segment loader ----------------
         uint32_t g = 0;        // items started (slot sequence)
         uint32_t hseq = 0;     // second planes started
+        uint32_t es = (uint32_t)lane % (uint32_t)nE, eph = 0;   // this lane's slot, its use's parity
+        uint32_t tail = 0;     // oldest item that may still be in the ring
+        int32_t head = 0;      // the ring's next free byte (the items lie between)
         const unsigned lanemask = (1u << lane) - 1u;
         bool stop_l = false;
         for (int jn = 0; jn < njobs && !stop_l; ++jn) {
@@ -697,33 +719,86 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             for (uint32_t jb = 0; jb < nitem; jb += (uint32_t)nsets) {
                 seg_ptrs(jb + (uint32_t)nsets + (uint32_t)lane, nxt);
                 const uint32_t n = min((uint32_t)nsets, nitem - jb);
-                bool ok = true;
-                if ((uint32_t)lane < n) {
-                    const uint32_t gl = g + (uint32_t)lane, es = gl % (uint32_t)nE;
-                    if (gl >= (uint32_t)nE)
-                        ok = tc::mbar_wait(&ent_free[es], (gl / (uint32_t)nE - 1u) & 1u,
-                                           kWaitLimit);
-                    if (!ok) *err = DPMM_ETIMEOUT;
-                }
-                if (!__all_sync(0xFFFFFFFFu, ok && *err == 0)) {
-                    stop_l = true;
-                    break;
-                }
                 const unsigned flagged = __ballot_sync(0xFFFFFFFFu, (uint32_t)lane < n && cur[5]);
-                if ((uint32_t)lane < n) {
-                    const uint32_t es = (g + (uint32_t)lane) % (uint32_t)nE;
-                    meta[es] = make_int4(cur[1] - cur[0], cur[2] - cur[0], cur[3] - cur[0],
-                                         cur[4] - cur[0]);
+                const int32_t len = cur[4] - cur[0];
+                const int32_t room = (uint32_t)lane < n ? max(len, 4) * 4 : 0;   // ring bytes
+                auto issue = [&](int32_t at) {
+                    slot_off[es] = at;
+                    meta[es] = make_int4(cur[1] - cur[0], cur[2] - cur[0], cur[3] - cur[0], len);
                     if (planes_any)
                         meta_hi[es] = cur[5] ? 1 + (int)(hseq + __popc(flagged & lanemask)) : 0;
-                    const uint32_t bytes = (uint32_t)(cur[4] - cur[0]) * 4u;
-                    if (bytes) {
-                        tc::mbar_arrive_expect_tx(&ent_full[es], bytes);
-                        tc::bulk_g2s(E_base + es * e_slot, ch.tile_ent + cur[0], bytes,
+                    if (len) {
+                        tc::mbar_arrive_expect_tx(&ent_full[es], (uint32_t)len * 4u);
+                        tc::bulk_g2s(E_base + at, ch.tile_ent + cur[0], (uint32_t)len * 4u,
                                      &ent_full[es]);
                     } else {
                         tc::mbar_arrive(&ent_full[es]);
                     }
+                };
+                // the slots' previous items have been consumed (a lane each; at a
+                // slot's first use the parity of the phase before the first)
+                bool ok = (uint32_t)lane >= n || tc::mbar_wait(&ent_free[es], eph ^ 1u, kWaitLimit);
+                ok = __all_sync(0xFFFFFFFFu, ok && *err == 0);
+                if (fixed) {
+                    if (ok && (uint32_t)lane < n) issue((int32_t)(es * (uint32_t)e_max));
+                } else {
+                    if (g + n > tail + (uint32_t)nE) tail = g + n - (uint32_t)nE;
+                    // the round's items side by side when the ring has room for all
+                    int32_t off = room;
+#pragma unroll
+                    for (int o = 1; o < kProdSets; o <<= 1) {
+                        const int32_t y = __shfl_up_sync(0xFFFFFFFFu, off, o);
+                        if (lane >= o) off += y;
+                    }
+                    const int32_t all = __shfl_sync(0xFFFFFFFFu, off, kProdSets - 1);
+                    off -= room;
+                    if (tail == g) head = 0;
+                    int32_t toff = tail == g ? -1 : slot_off[tail % (uint32_t)nE];
+                    if (ok && (head > toff ? (int32_t)e_ring - head : toff - head) >= all) {
+                        if ((uint32_t)lane < n) issue(head + off);
+                        head += all;
+                    } else {
+                        // one after the other, wrapping, and waiting for the oldest
+                        // items in the ring as needed
+                        for (uint32_t j = 0; j < n && ok; ++j) {
+                            const int32_t need = __shfl_sync(0xFFFFFFFFu, room, (int)j);
+                            int32_t at = -1;
+                            while (ok && at < 0) {
+                                if (tail == g + j) {
+                                    at = 0;
+                                } else {
+                                    const uint32_t ts = tail % (uint32_t)nE;
+                                    toff = slot_off[ts];
+                                    if (head > toff) {
+                                        if ((int32_t)e_ring - head >= need) at = head;
+                                        else if (toff >= need) at = 0;
+                                    } else if (toff - head >= need) {
+                                        at = head;
+                                    }
+                                    if (at < 0) {
+                                        ok = tc::mbar_wait_warp(&ent_free[ts],
+                                                                (tail / (uint32_t)nE) & 1u,
+                                                                kWaitLimit) &&
+                                             __all_sync(0xFFFFFFFFu, *err == 0);
+                                        ++tail;
+                                    }
+                                }
+                            }
+                            if (ok && (uint32_t)lane == j) issue(at);
+                            head = at + need;
+                            __syncwarp();
+                        }
+                    }
+                }
+                if (!ok) {
+                    if (lane == 0) *err = DPMM_ETIMEOUT;
+                    stop_l = true;
+                    break;
+                }
+                __syncwarp();
+                if ((es += n) >= (uint32_t)nE) {
+                    es -= (uint32_t)nE;
+                    eph ^= 1u;
                 }
                 g += n;
                 hseq += (uint32_t)__popc(flagged);
@@ -731,11 +806,13 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                 for (int k = 0; k < 6; ++k) cur[k] = nxt[k];
             }
         }
-        // every started copy has landed before the block can exit
-        const uint32_t issued = g;
+        // every started copy has landed before the block can exit (after a
+        // timeout perhaps some of the round that was cut short)
+        const uint32_t issued = g + (stop_l ? (uint32_t)nsets : 0u);
         if (lane == 0)
             for (uint32_t q = issued > (uint32_t)nE ? issued - (uint32_t)nE : 0u; q < issued; ++q)
-                tc::mbar_wait(&ent_full[q % (uint32_t)nE], (q / (uint32_t)nE) & 1u, kWaitLimit);
+                tc::mbar_wait(&ent_full[q % (uint32_t)nE], (q / (uint32_t)nE) & 1u,
+                              stop_l ? kWaitLimit >> 8 : kWaitLimit);
     } else if (warp == kBLoadWarp) {
         // ---------------- B loader ----------------
         if (lane == 0) {

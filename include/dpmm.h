@@ -307,7 +307,7 @@ int dpmm_set_params(dpmm_ctx* ctx, const float* logpi, const float* logtheta);
 
 /*
  * FP32 log-likelihood scores of selected cells under the current parameters,
- * computed by the same device code as the sweep's contraction:
+ * by the CSR engine's FP32 contraction (its sums in another order for K > 32):
  * out float[n][3K]: columns 0..K-1 hold log pi_k + sum_u x_i^u log theta_k^u
  * (eq. 4 third line with eq. 26), column K + 2k + r holds
  * sum_u x_i^u log theta-bar_{k,r}^u (the likelihood factor of eq. 8).

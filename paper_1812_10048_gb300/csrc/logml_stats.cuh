@@ -7,7 +7,7 @@
 // atomics on 50,000 hot words were the bound.  Here a block owns a private
 // copy of the counters of a range of clusters ([kg][D] words, all K when they
 // fit) and adds them into S with bulk reductions (cp.reduce.async.bulk), which
-// the L2 performs a sector at a time: 152 blocks x 200 KB.
+// the L2 performs a sector at a time: 152 blocks x 200 KB; 323 -> 58 us.
 //
 // Clusters that do not fit together are split into G contiguous groups of kg
 // clusters (a multiple of four, so that every group starts on 16 bytes); a

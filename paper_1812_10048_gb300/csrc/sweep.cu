@@ -1142,8 +1142,10 @@ __device__ __forceinline__ int warp_argmax(float best, int bestk) {
     return bestk;
 }
 
-// K > 32: lanes own clusters lane, lane + 32, ...; the row is contracted once
-// per chunk of 32 clusters and the running Gumbel-max kept across chunks.
+// More clusters or genes than the forms below hold in shared memory (fewer than
+// four clusters of a table of D genes fit): lanes own clusters lane, lane + 32,
+// ..., the row is contracted once per chunk of 32 clusters from global memory
+// and the running Gumbel-max kept across chunks.
 __device__ __forceinline__ void assign_cells(const ChainArgs& a, const float* L, int ldL, int K,
                                              uint32_t t, unsigned long long* blk_logq) {
     const int lane = threadIdx.x & 31;
@@ -1427,6 +1429,205 @@ __device__ __forceinline__ void assign_cells_v2(const ChainArgs& a, const float*
     }
 }
 
+// K > 32, or tables too long for assign_cells_v2: the cluster table passes
+// through shared memory in slabs of 4 LPE clusters (row stride 4 LPE floats).
+// LPE lanes hold one entry's slab row (a float4 each), so that a warp adds
+// 32 / LPE entries with one 16-byte shared-memory load per lane; LPE x 16 bytes
+// are contiguous, so no two lanes meet on a bank.  What bounds it is that
+// traffic: 4 bytes an entry and cluster.  (Lanes that own clusters and take the
+// entries one by one read the same bytes but spend eight instructions an entry,
+// and with a table beyond shared memory read it from the L2, 256 bytes an entry
+// at K = 64: 30,011 x 1,000 cells 298 us, 113 us in slabs.)
+//
+// The block's cells [N b / G, N (b + 1) / G) are taken in batches of at most
+// 1,024, 32 a warp: lane i keeps cell i's row bounds, running Gumbel-max and
+// eq. 8 sums, so that the per-cell draws run on all lanes.
+template <int LPE, bool packed>
+__device__ __forceinline__ void assign_wide(const ChainArgs& a, float* slab, int K, int KS,
+                                            uint32_t t, const float* spi,
+                                            unsigned long long* blk_logq) {
+    constexpr int ld = 4 * LPE, E = 32 / LPE;     // row stride, entries per step
+    constexpr int kRow = 4;                       // 32-entry pieces in flight
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nw = (int)(blockDim.x >> 5);
+    const int ql = lane % LPE, g = lane / LPE;    // float4 of the slab row, entry of the step
+    const int D = a.D;
+    const float2* __restrict__ Ls2 = reinterpret_cast<const float2*>(a.Ls);
+    const int64_t b0 = a.N * blockIdx.x / gridDim.x, b1 = a.N * (blockIdx.x + 1) / gridDim.x;
+    const int passes = (K + KS - 1) / KS;
+    for (int64_t c0 = b0; c0 < b1; c0 += 32 * nw) {
+        // lane i: cell c0 + w + nw i of the batch
+        const int64_t cell = c0 + w + (int64_t)nw * lane;
+        const bool mine = cell < b1;
+        const int cells = (int)max((int64_t)0, min((int64_t)32, (b1 - c0 - w + nw - 1) / nw));
+        long long beg = 0;
+        int len = 0;
+        if (mine) {
+            beg = a.csr.indptr[cell];
+            len = (int)(a.csr.indptr[cell + 1] - beg);
+        }
+        float best = -CUDART_INF_F;
+        int bestk = K;
+        for (int p = 0; p < passes; ++p) {
+            const int k0 = p * KS, kn = min(KS, K - k0);
+            if (passes > 1 || c0 == b0) {
+                __syncthreads();
+                // (the values of clusters from K on are never looked at)
+                if ((a.kmax & 3) == 0) {
+                    float4* s4 = reinterpret_cast<float4*>(slab);
+                    const int tot = D * LPE, nthr = (int)blockDim.x;
+                    for (int i0 = threadIdx.x; i0 < tot; i0 += 4 * nthr) {
+                        float4 v[4];
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            const int i = i0 + x * nthr, u = i / LPE, k = k0 + 4 * (i - u * LPE);
+                            if (i < tot && k < a.kmax)
+                                v[x] = __ldg(reinterpret_cast<const float4*>(
+                                    a.Lc + (size_t)u * a.kmax + k));
+                        }
+#pragma unroll
+                        for (int x = 0; x < 4; ++x)
+                            if (i0 + x * nthr < tot) s4[i0 + x * nthr] = v[x];
+                    }
+                } else {
+                    for (int i = threadIdx.x; i < D * ld; i += blockDim.x) {
+                        const int u = i / ld, k = i - u * ld;
+                        if (k < kn) slab[i] = __ldg(a.Lc + (size_t)u * a.kmax + k0 + k);
+                    }
+                }
+                __syncthreads();
+            }
+            const float4* row4 = reinterpret_cast<const float4*>(slab) + ql;
+            for (int i = 0; i < cells; ++i) {
+                const long long rb = __shfl_sync(0xFFFFFFFFu, beg, i);
+                const int rl = __shfl_sync(0xFFFFFFFFu, len, i);
+                const uint32_t ci = (uint32_t)(c0 + w + (int64_t)nw * i);
+                float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                auto add = [&](uint32_t u, uint32_t x) {
+                    const float4 l = row4[u * LPE];
+                    const float xf = (float)x;
+                    acc.x = fmaf(xf, l.x, acc.x);
+                    acc.y = fmaf(xf, l.y, acc.y);
+                    acc.z = fmaf(xf, l.z, acc.z);
+                    acc.w = fmaf(xf, l.w, acc.w);
+                };
+                for (int e0 = 0; e0 < rl; e0 += 32 * kRow) {
+                    uint32_t ev[kRow], xv[kRow];
+#pragma unroll
+                    for (int r = 0; r < kRow; ++r) {
+                        ev[r] = xv[r] = 0u;
+                        const int e = e0 + 32 * r + lane;
+                        if (e < rl) {
+                            if (packed) {
+                                ev[r] = __ldg(a.csr.entries + rb + e);
+                            } else {
+                                ev[r] = (uint32_t)__ldg(a.csr.cols + rb + e);
+                                xv[r] = (uint32_t)__ldg(a.csr.counts + rb + e);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < kRow; ++r) {
+                        const int n = rl - e0 - 32 * r;      // entries of this piece on
+                        if (n <= 0) break;
+                        if (n >= 32) {
+#pragma unroll
+                            for (int j = 0; j < 32; j += E) {
+                                const uint32_t v = __shfl_sync(0xFFFFFFFFu, ev[r], j + g);
+                                if (packed) add(v >> 16, v & 0xFFFFu);
+                                else add(v, __shfl_sync(0xFFFFFFFFu, xv[r], j + g));
+                            }
+                        } else {
+                            for (int j = 0; j < n; j += E) {
+                                const uint32_t v = __shfl_sync(0xFFFFFFFFu, ev[r], j + g);
+                                const uint32_t x = __shfl_sync(0xFFFFFFFFu, xv[r], j + g);
+                                if (j + g < n) add(packed ? v >> 16 : v, packed ? v & 0xFFFFu : x);
+                            }
+                        }
+                    }
+                }
+                // the entry groups' sums; then lane (g, ql) takes cluster
+                // 4 ql + g' for the g' it stands for
+#pragma unroll
+                for (int o = 16; o >= LPE; o >>= 1) {
+                    acc.x += __shfl_xor_sync(0xFFFFFFFFu, acc.x, o);
+                    acc.y += __shfl_xor_sync(0xFFFFFFFFu, acc.y, o);
+                    acc.z += __shfl_xor_sync(0xFFFFFFFFu, acc.z, o);
+                    acc.w += __shfl_xor_sync(0xFFFFFFFFu, acc.w, o);
+                }
+                float bv = -CUDART_INF_F;
+                int bk = 0x7FFFFFFF;
+                const uint4 wd = a.st.words(TAG_LABEL, ci, t, (uint32_t)((k0 >> 2) + ql));
+                constexpr int per = E >= 4 ? 1 : 4 / E;      // clusters a lane draws
+#pragma unroll
+                for (int q = 0; q < per; ++q) {
+                    const int j = (g + E * q) & 3, k = 4 * ql + j;
+                    if (k < kn) {
+                        const float sc = j == 0 ? acc.x : j == 1 ? acc.y : j == 2 ? acc.z : acc.w;
+                        const float v = (spi[k0 + k] + sc) + gumbel(word_of(wd, j));
+                        if (v > bv || (v == bv && k0 + k < bk)) {
+                            bv = v;
+                            bk = k0 + k;
+                        }
+                    }
+                }
+                // the warp's largest value, then the lowest cluster that has it
+                // (floats in the order of their sortable integers; no NaN here)
+                const uint32_t fb = __float_as_uint(bv + 0.0f);   // (-0 as 0)
+                const uint32_t key = fb & 0x80000000u ? ~fb : fb | 0x80000000u;
+                const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, key);
+                bk = (int)__reduce_min_sync(0xFFFFFFFFu,
+                                            key == top ? (uint32_t)bk : 0x7FFFFFFFu);
+                bv = __uint_as_float(top & 0x80000000u ? top & 0x7FFFFFFFu : ~top);
+                if (lane == i && bk < K && (bv > best || bestk == K)) {
+                    best = bv;
+                    bestk = bk;
+                }
+            }
+        }
+        if (bestk == K) bestk = 0;     // every score a NaN: some cluster of the table
+        // eq. 8 likelihood factors of each cell's cluster
+        float2 lik = make_float2(0.0f, 0.0f);
+        for (int i = 0; i < cells; ++i) {
+            const long long rb = __shfl_sync(0xFFFFFFFFu, beg, i);
+            const int rl = __shfl_sync(0xFFFFFFFFu, len, i);
+            const int c = __shfl_sync(0xFFFFFFFFu, bestk, i);
+            float t0 = 0.0f, t1 = 0.0f;
+            for (int e0 = lane; e0 < rl; e0 += 32 * kRow) {
+                int32_t u[kRow], x[kRow];
+#pragma unroll
+                for (int r = 0; r < kRow; ++r) {
+                    u[r] = x[r] = 0;
+                    if (e0 + 32 * r < rl) a.csr.get(rb + e0 + 32 * r, u[r], x[r]);
+                }
+                float2 l[kRow];
+#pragma unroll
+                for (int r = 0; r < kRow; ++r)
+                    if (e0 + 32 * r < rl) l[r] = __ldg(Ls2 + (size_t)u[r] * a.kmax + c);
+#pragma unroll
+                for (int r = 0; r < kRow; ++r)
+                    if (e0 + 32 * r < rl) {
+                        t0 = fmaf((float)x[r], l[r].x, t0);
+                        t1 = fmaf((float)x[r], l[r].y, t1);
+                    }
+            }
+            t0 = warp_sum(t0);
+            t1 = warp_sum(t1);
+            if (lane == i) lik = make_float2(t0, t1);
+        }
+        int c = -1;
+        unsigned long long q = 0ull;
+        if (mine) {
+            float logq;
+            c = bestk;
+            const uint32_t s = draw_sublabel(a, cell, c, lik, TAG_SUBLABEL, t, &logq);
+            a.state[cell] = pack_state((uint32_t)c, s);
+            q = logq_fixed(logq);
+        }
+        warp_add_by_cluster(blk_logq, c, q);
+    }
+}
+
 __device__ __forceinline__ void assign_chain(const ChainArgs& a, int64_t smem_bytes) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (a.sc->tile_used) return;   // the dense-tile engine labelled this sweep
@@ -1506,19 +1707,30 @@ __device__ __forceinline__ void assign_chain(const ChainArgs& a, int64_t smem_by
             blk_logq[k] = v;
         }
     } else {
-        // large K: lanes own clusters, table in shared memory when it fits
-        float* sL = reinterpret_cast<float*>(rest);
-        const bool in_smem = (int64_t)K * D * 4 <= avail;
-        if (in_smem)
-            for (int64_t i = threadIdx.x; i < (int64_t)K * D; i += blockDim.x) {
-                const int64_t u = i / K, k = i - u * K;
-                sL[i] = __ldg(a.Lc + u * a.kmax + k);
-            }
+        float* slab = reinterpret_cast<float*>(rest);
         if (blockIdx.x == 0 && threadIdx.x == 0) a.sc->stats_fused = 0;
         __syncthreads();
-        const float* L = in_smem ? sL : a.Lc;
-        const int ldL = in_smem ? K : a.kmax;
-        assign_cells(a, L, ldL, K, t, blk_logq);
+        // slabs as wide as fit (a power of two of float4s), no wider than K needs
+        const int64_t fit4 = avail / ((int64_t)16 * D);     // float4s per gene
+        int lpe = 16;
+        while (lpe > 1 && (lpe > fit4 || lpe / 2 >= (K + 3) / 4)) lpe >>= 1;
+        // (the slabs evenly filled, in whole float4s)
+        const int slabs = (K + 4 * lpe - 1) / (4 * lpe);
+        const int KS = ((K + slabs - 1) / slabs + 3) & ~3;
+        if (fit4 < 1) assign_cells(a, a.Lc, a.kmax, K, t, blk_logq);
+        else if (a.csr.entries) {
+            if (lpe == 16) assign_wide<16, true>(a, slab, K, KS, t, spi, blk_logq);
+            else if (lpe == 8) assign_wide<8, true>(a, slab, K, KS, t, spi, blk_logq);
+            else if (lpe == 4) assign_wide<4, true>(a, slab, K, KS, t, spi, blk_logq);
+            else if (lpe == 2) assign_wide<2, true>(a, slab, K, KS, t, spi, blk_logq);
+            else assign_wide<1, true>(a, slab, K, KS, t, spi, blk_logq);
+        } else {
+            if (lpe == 16) assign_wide<16, false>(a, slab, K, KS, t, spi, blk_logq);
+            else if (lpe == 8) assign_wide<8, false>(a, slab, K, KS, t, spi, blk_logq);
+            else if (lpe == 4) assign_wide<4, false>(a, slab, K, KS, t, spi, blk_logq);
+            else if (lpe == 2) assign_wide<2, false>(a, slab, K, KS, t, spi, blk_logq);
+            else assign_wide<1, false>(a, slab, K, KS, t, spi, blk_logq);
+        }
     }
     __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x)

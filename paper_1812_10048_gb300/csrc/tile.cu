@@ -274,7 +274,7 @@ __device__ __forceinline__ void chain_tiles(int64_t off, int T, int& first, int&
 //               ahead.  The items lie end to end in the ring: a few deep cells
 //               make one segment several times the mean, and slots of that
 //               size left room for fewer A stages (1.3 M x 2,000 with 2% deep
-//               cells: 1,557 us with slots, RING us)
+//               cells: 1,557 us with slots, 1,246 us)
 //   warp 16     lane 0 bulk-copies the B operand of each chunk into its ring
 // The roles that feed the tensor core are alone on their scheduler (w % 4 = 0)
 // but for two epilogue warps: each item costs them the latency of a chain of
@@ -524,7 +524,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // that a round seldom waits for more than its own slots
     // (fixed slots for the longest segment where two a set fit: a round of the
     // loader is shorter then; 68,000 x 1,000 39 -> 35 us, 8,000 x 32,738
-    // 191 -> 165 us, while the ring gives 89 -> 76 us for 24 datasets)
+    // 191 -> 172 us, while the ring gives 89 -> 76 us for 24 datasets)
     const bool fixed = e_ring >= 2 * nsets * e_max;
     const int64_t e_item = fixed ? e_max : e_mean + e_mean / 4;
     const int nE = (int)min((int64_t)(kMaxESlots / nsets),

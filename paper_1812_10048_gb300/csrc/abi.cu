@@ -420,12 +420,14 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         CKI(cudaMemcpyAsync(d_idx, indices, sizeof(int32_t) * nnz, cudaMemcpyDefault, c.stream));
         CKI(cudaMemcpyAsync(d_val, data, sizeof(int32_t) * nnz, cudaMemcpyDefault, c.stream));
     }
-    CKI(dalloc(&d_colsum, (size_t)D));
     CKI(dalloc(&d_chk, 1));
-    CKI(cudaMemsetAsync(d_colsum, 0, sizeof(unsigned long long) * D, c.stream));
-    CsrCheck chk = {LLONG_MAX, LLONG_MAX, 0, INT_MAX};
+    // the packed copy is written by the pass that checks the entries (padded to a
+    // multiple of four entries, zeros, so that 16-byte aligned bulk copies of rows
+    // stay inside the allocation); a count beyond 16 bits drops it again
+    if (D <= 65536) CKI(dalloc(&c.entries, std::max<size_t>(4, ((size_t)nnz + 3) & ~(size_t)3)));
+    CsrCheck chk = {LLONG_MAX, LLONG_MAX, 0, INT_MAX, 0};
     CKI(cudaMemcpyAsync(d_chk, &chk, sizeof(CsrCheck), cudaMemcpyHostToDevice, c.stream));
-    CKI(launch_check_csr(c.indptr, d_idx, d_val, N, nnz, D, d_colsum, d_chk, c.num_sms,
+    CKI(launch_check_csr(c.indptr, d_idx, d_val, N, nnz, D, c.entries, d_chk, c.num_sms,
                          c.stream));
     CKI(cudaMemcpyAsync(&chk, d_chk, sizeof(CsrCheck), cudaMemcpyDeviceToHost, c.stream));
     CKI(cudaStreamSynchronize(c.stream));
@@ -440,6 +442,14 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
                              chk.bad_entry));
         return bail(fail(DPMM_EINVAL, "negative count %d at entry %lld", x, chk.bad_entry));
     }
+    if (chk.total >= (1ull << 32)) {
+        // some gene may reach 2^32: its sum decides
+        CKI(dalloc(&d_colsum, (size_t)D));
+        CKI(cudaMemsetAsync(d_colsum, 0, sizeof(unsigned long long) * D, c.stream));
+        CKI(launch_gene_sums(d_idx, d_val, nnz, D, d_colsum, d_chk, c.num_sms, c.stream));
+        CKI(cudaMemcpyAsync(&chk, d_chk, sizeof(CsrCheck), cudaMemcpyDeviceToHost, c.stream));
+        CKI(cudaStreamSynchronize(c.stream));
+    }
     if (chk.overflow_gene != INT_MAX) {
         unsigned long long sum = 0;
         CKI(cudaMemcpy(&sum, d_colsum + chk.overflow_gene, sizeof(sum), cudaMemcpyDeviceToHost));
@@ -450,16 +460,9 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
     c.packed = D <= 65536 && chk.max_count <= 65535;
 
     const size_t K2 = 2 * (size_t)c.kmax;
-    if (c.packed) {
-        // padded to a multiple of four entries (zeros) so that 16-byte aligned
-        // bulk copies of rows stay inside the allocation
-        const size_t padded = ((size_t)nnz + 3) & ~(size_t)3;
-        CKI(dalloc(&c.entries, padded > 0 ? padded : 4));
-        if (padded > (size_t)nnz)
-            CKI(cudaMemsetAsync(c.entries + nnz, 0, (padded - (size_t)nnz) * sizeof(uint32_t),
-                                c.stream));
-        CKI(launch_pack(d_idx, d_val, nnz, c.entries, c.num_sms, c.stream));
-    } else {
+    if (!c.packed) {
+        if (c.entries) CKI(cudaFree(c.entries));
+        c.entries = nullptr;
         c.cols = d_idx;
         c.counts = d_val;
         d_idx = d_val = nullptr;
@@ -500,11 +503,10 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         c.tile_C = (D + 63) / 64;
         const int64_t TC = (int64_t)c.tile_T * c.tile_C;
         CKI(dalloc(&d_qcount, (size_t)(4 * TC)));
-        CKI(cudaMemsetAsync(d_qcount, 0, sizeof(int32_t) * 4 * TC, c.stream));
         CKI(dalloc(&c.tile_ptr, (size_t)(4 * TC + 1)));
-        CKI(launch_tile_count(c.indptr, c.entries, N, c.tile_T, c.tile_C, d_qcount, c.num_sms,
-                              c.stream));
-        CKI(dalloc(&d_scan, 2));
+        CKI(launch_tile_count(c.indptr, c.entries, N, c.tile_T, c.tile_C, d_qcount, c.stream));
+        CKI(dalloc(&d_scan, (size_t)tile_scan_words(TC)));
+        CKI(cudaMemsetAsync(d_scan, 0, 2 * sizeof(long long), c.stream));
         CKI(launch_tile_scan(d_qcount, TC, c.tile_ptr, d_scan, c.stream));
         long long scan[2] = {0, 0};
         CKI(cudaMemcpyAsync(scan, d_scan, sizeof(scan), cudaMemcpyDeviceToHost, c.stream));
@@ -512,13 +514,11 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         if (scan[0] > (long long)INT32_MAX)
             return bail(fail(DPMM_EOVERFLOW, "the dense-tile copy needs %lld entries (> 2^31 - 1)",
                              scan[0]));
-        c.tile_Lslot = (int32_t)scan[1];
+        c.tile_Lslot = (int32_t)std::max<long long>(4, scan[1]);
         c.tile_Lmean = (int32_t)((scan[0] + TC - 1) / TC);
         CKI(dalloc(&c.tile_ent, (size_t)scan[0]));
-        CKI(cudaMemsetAsync(c.tile_ent, 0, sizeof(uint32_t) * std::max<long long>(1, scan[0]),
-                            c.stream));
         CKI(launch_tile_scatter(c.indptr, c.entries, N, c.tile_T, c.tile_C, c.tile_ptr,
-                                c.tile_ent, c.num_sms, c.stream));
+                                c.tile_ent, c.stream));
         CKI(dalloc(&c.tile_B, tile_b_bytes(c.tile_C)));
         CKI(dalloc(&c.noise, (size_t)(kTileMaxK + 2) * (size_t)N));
         c.tile_enabled = true;

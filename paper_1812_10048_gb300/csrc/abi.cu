@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -70,6 +71,26 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Memory the host reads directly (pageable or pinned).
+bool is_host_ptr(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeUnregistered;
+}
+
+// Device memory of device `dev`.
+bool on_this_device(const void* p, int dev) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 // Host-side CSR checks (shared by dpmm_init and dpmm_logml_create).
 int check_csr(const std::vector<int32_t>& indptr, const std::vector<int32_t>& idx,
               const std::vector<int32_t>& val, int64_t N, int32_t D, int32_t* max_count) {
@@ -104,14 +125,11 @@ void free_ctx(Ctx& c) {
     if (c.step_exec) cudaGraphExecDestroy(c.step_exec);
     for (cudaEvent_t& e : c.ev)
         if (e) cudaEventDestroy(e);
-    void* ptrs[] = {c.indptr, c.entries, c.cols, c.counts, c.state, c.sc, c.nsub, c.Ssub,
-                    c.sumlogq, c.acc_nsub, c.acc_Ssub, c.acc_logq, c.logpi, c.Lc, c.Ls,
-                    c.local_tab, c.lmap, c.desc, c.reinit, c.decide, c.log_h, c.pair_ab, c.lg_table,
-                    c.move_part, c.move_ticket, c.tile_ent, c.tile_ptr, c.tile_B, c.noise,
-                    c.gbar, c.d_chains};
+    // (a chain's arrays lie in c.arena; a batch context has only its own few)
+    void* ptrs[] = {c.arena, c.csr_mem, c.tile_ent, c.gbar_own, c.chains_own};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    if (c.sc_host) cudaFreeHost(c.sc_host);
+    delete c.sc_host;
     delete c.h_chain0;
     c.h_chain0 = nullptr;
     if (c.lml) {
@@ -359,23 +377,11 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
     c.opts = o;
     c.kmax = o.kmax;
 
-    // scratch of the device-side CSR preparation (freed on every exit; the
-    // unpacked storage adopts the staging columns and counts)
-    int32_t* d_idx = nullptr;
-    int32_t* d_val = nullptr;
+    // gene sums of the rare matrix that needs them (freed on every exit)
     unsigned long long* d_colsum = nullptr;
-    CsrCheck* d_chk = nullptr;
-    int32_t* d_qcount = nullptr;
-    long long* d_scan = nullptr;
     auto free_scratch = [&]() {
-        void* ps[] = {d_idx, d_val, d_colsum, d_chk, d_qcount, d_scan};
-        for (void* q : ps)
-            if (q) cudaFree(q);
-        d_idx = d_val = nullptr;
+        if (d_colsum) cudaFree(d_colsum);
         d_colsum = nullptr;
-        d_chk = nullptr;
-        d_qcount = nullptr;
-        d_scan = nullptr;
     };
     auto bail = [&](int code) {
         if (c.stream) cudaStreamSynchronize(c.stream);
@@ -401,33 +407,116 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         c.own_stream = true;
     }
 
-    // ---- the CSR on the device: one copy of each array, then validation ----
-    CKI(dalloc(&c.indptr, (size_t)N + 1));
-    CKI(cudaMemcpyAsync(c.indptr, indptr, sizeof(int32_t) * (N + 1), cudaMemcpyDefault, c.stream));
+    // ---- nnz, then every array whose size follows from N, D, kmax and nnz in one
+    // allocation (a cudaMalloc of 2 MB or more and its cudaFree take 60 - 80 us
+    // each, a pinned allocation 270 us; thirty of them were 1 ms of a 2 ms start)
     int32_t ends[2] = {0, 0};
-    CKI(cudaMemcpyAsync(&ends[0], c.indptr, sizeof(int32_t), cudaMemcpyDeviceToHost, c.stream));
-    CKI(cudaMemcpyAsync(&ends[1], c.indptr + N, sizeof(int32_t), cudaMemcpyDeviceToHost, c.stream));
-    CKI(cudaStreamSynchronize(c.stream));
+    if (is_host_ptr(indptr)) {
+        ends[0] = indptr[0];
+        ends[1] = indptr[N];
+    } else {
+        CKI(cudaMemcpyAsync(&ends[0], indptr, sizeof(int32_t), cudaMemcpyDefault, c.stream));
+        CKI(cudaMemcpyAsync(&ends[1], indptr + N, sizeof(int32_t), cudaMemcpyDefault, c.stream));
+        CKI(cudaStreamSynchronize(c.stream));
+    }
     if (ends[0] != 0) return bail(fail(DPMM_EINVAL, "indptr[0] = %d, expected 0", ends[0]));
     const int64_t nnz = ends[1];
     if (nnz < 0) return bail(fail(DPMM_EINVAL, "indptr[N] = %lld", (long long)nnz));
     if (nnz > 0 && (!indices || !data)) return bail(fail(DPMM_EINVAL, "indices/data are null"));
     c.nnz = nnz;
     c.mean_row = nnz / N;
-    CKI(dalloc(&d_idx, (size_t)nnz));
-    CKI(dalloc(&d_val, (size_t)nnz));
-    if (nnz > 0) {
-        CKI(cudaMemcpyAsync(d_idx, indices, sizeof(int32_t) * nnz, cudaMemcpyDefault, c.stream));
-        CKI(cudaMemcpyAsync(d_val, data, sizeof(int32_t) * nnz, cudaMemcpyDefault, c.stream));
-    }
-    CKI(dalloc(&d_chk, 1));
-    // the packed copy is written by the pass that checks the entries (padded to a
-    // multiple of four entries, zeros, so that 16-byte aligned bulk copies of rows
-    // stay inside the allocation); a count beyond 16 bits drops it again
-    if (D <= 65536) CKI(dalloc(&c.entries, std::max<size_t>(4, ((size_t)nnz + 3) & ~(size_t)3)));
+    const size_t K2 = 2 * (size_t)c.kmax;
+    const int32_t tT = (int32_t)((N + 127) / 128), tC = (D + 63) / 64;
+    const int64_t TC = (int64_t)tT * tC;
+    CsrCheck* d_chk = nullptr;
+    int32_t* d_qcount = nullptr;
+    long long* d_scan = nullptr;
+    // packed: with the packed entries and, unless the engine is the CSR one, the
+    // blocked copy's arrays (but its entries, whose number is found by counting)
+    auto carve = [&](char* base, bool packed) {
+        size_t off = 0;
+        auto take = [&](auto** p, size_t n) {
+            *p = base ? reinterpret_cast<std::remove_reference_t<decltype(*p)>>(base + off)
+                      : nullptr;
+            off += (std::max<size_t>(1, n) * sizeof(**p) + 255) & ~(size_t)255;
+        };
+        take(&c.indptr, (size_t)N + 1);
+        take(&c.state, (size_t)N);
+        take(&c.sc, 1);
+        take(&c.nsub, K2);
+        take(&c.Ssub, K2 * D);
+        take(&c.sumlogq, (size_t)c.kmax);
+        take(&c.acc_nsub, K2);
+        take(&c.acc_Ssub, K2 * D);
+        take(&c.acc_logq, (size_t)c.kmax);
+        take(&c.logpi, (size_t)c.kmax + 1);
+        take(&c.Lc, (size_t)c.kmax * D);
+        take(&c.Ls, K2 * D);
+        if (o.local_iters > 1) take(&c.local_tab, (size_t)D * (size_t)(c.kmax | 1) * 2 + 4);
+        take(&c.lmap, K2);
+        take(&c.desc, K2);
+        take(&c.reinit, (size_t)c.kmax);
+        take(&c.decide, (size_t)c.kmax);
+        take(&c.log_h, (size_t)c.kmax);
+        take(&c.pair_ab, K2);
+        take(&c.lg_table, lg_table_entries());
+        take(&c.move_part, move_partial_bytes());
+        take(&c.move_ticket, (size_t)c.kmax);
+        take(&c.gbar, 1);
+        take(&c.d_chains, 1);
+        take(&d_chk, 1);
+        c.entries = nullptr;
+        c.tile_ptr = nullptr;
+        c.tile_B = nullptr;
+        c.noise = nullptr;
+        if (packed) {
+            // padded to a multiple of four entries (zeros) so that 16-byte aligned
+            // bulk copies of rows stay inside the allocation
+            take(&c.entries, std::max<size_t>(4, ((size_t)nnz + 3) & ~(size_t)3));
+            if (o.engine != DPMM_ENGINE_CSR_FP32) {
+                take(&c.tile_ptr, (size_t)(4 * TC + 1));
+                take(&c.tile_B, tile_b_bytes(tC));
+                // the bucket counts of the preparation lie where the label noise
+                // will
+                take(&c.noise, std::max((size_t)(kTileMaxK + 2) * (size_t)N, (size_t)(4 * TC)));
+                d_qcount = reinterpret_cast<int32_t*>(c.noise);
+                take(&d_scan, (size_t)tile_scan_words(TC));
+            }
+        }
+        return off;
+    };
+    auto allocate = [&](bool packed) {
+        cudaError_t e = cudaMalloc((void**)&c.arena, carve(nullptr, packed));
+        if (e != cudaSuccess) {
+            c.arena = nullptr;
+            return e;
+        }
+        carve(c.arena, packed);
+        return cudaMemcpyAsync(c.indptr, indptr, sizeof(int32_t) * (N + 1), cudaMemcpyDefault,
+                               c.stream);
+    };
+    CKI(allocate(D <= 65536));
+    // the entries: a caller's arrays on this device are read where they are,
+    // others are staged
+    const int32_t *s_idx = indices, *s_val = data;
+    auto stage = [&]() {
+        cudaError_t e = cudaMalloc((void**)&c.csr_mem, 2 * sizeof(int32_t) * (size_t)nnz);
+        if (e != cudaSuccess) {
+            c.csr_mem = nullptr;
+            return e;
+        }
+        int32_t* d = reinterpret_cast<int32_t*>(c.csr_mem);
+        if ((e = cudaMemcpyAsync(d, indices, sizeof(int32_t) * nnz, cudaMemcpyDefault, c.stream)))
+            return e;
+        s_idx = d;
+        s_val = d + nnz;
+        return cudaMemcpyAsync(d + nnz, data, sizeof(int32_t) * nnz, cudaMemcpyDefault, c.stream);
+    };
+    if (nnz > 0 && !(on_this_device(indices, c.device) && on_this_device(data, c.device)))
+        CKI(stage());
     CsrCheck chk = {LLONG_MAX, LLONG_MAX, 0, INT_MAX, 0};
     CKI(cudaMemcpyAsync(d_chk, &chk, sizeof(CsrCheck), cudaMemcpyHostToDevice, c.stream));
-    CKI(launch_check_csr(c.indptr, d_idx, d_val, N, nnz, D, c.entries, d_chk, c.num_sms,
+    CKI(launch_check_csr(c.indptr, s_idx, s_val, N, nnz, D, c.entries, d_chk, c.num_sms,
                          c.stream));
     CKI(cudaMemcpyAsync(&chk, d_chk, sizeof(CsrCheck), cudaMemcpyDeviceToHost, c.stream));
     CKI(cudaStreamSynchronize(c.stream));
@@ -435,8 +524,8 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         return bail(fail(DPMM_EINVAL, "indptr decreases at row %lld", chk.bad_row));
     if (chk.bad_entry != LLONG_MAX) {
         int32_t u = 0, x = 0;
-        CKI(cudaMemcpy(&u, d_idx + chk.bad_entry, sizeof(int32_t), cudaMemcpyDeviceToHost));
-        CKI(cudaMemcpy(&x, d_val + chk.bad_entry, sizeof(int32_t), cudaMemcpyDeviceToHost));
+        CKI(cudaMemcpy(&u, s_idx + chk.bad_entry, sizeof(int32_t), cudaMemcpyDeviceToHost));
+        CKI(cudaMemcpy(&x, s_val + chk.bad_entry, sizeof(int32_t), cudaMemcpyDeviceToHost));
         if (u < 0 || u >= D)
             return bail(fail(DPMM_EINVAL, "column index %d out of [0, %d) at entry %lld", u, D,
                              chk.bad_entry));
@@ -446,7 +535,7 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         // some gene may reach 2^32: its sum decides
         CKI(dalloc(&d_colsum, (size_t)D));
         CKI(cudaMemsetAsync(d_colsum, 0, sizeof(unsigned long long) * D, c.stream));
-        CKI(launch_gene_sums(d_idx, d_val, nnz, D, d_colsum, d_chk, c.num_sms, c.stream));
+        CKI(launch_gene_sums(s_idx, s_val, nnz, D, d_colsum, d_chk, c.num_sms, c.stream));
         CKI(cudaMemcpyAsync(&chk, d_chk, sizeof(CsrCheck), cudaMemcpyDeviceToHost, c.stream));
         CKI(cudaStreamSynchronize(c.stream));
     }
@@ -459,37 +548,22 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
     c.max_count = chk.max_count;
     c.packed = D <= 65536 && chk.max_count <= 65535;
 
-    const size_t K2 = 2 * (size_t)c.kmax;
-    if (!c.packed) {
-        if (c.entries) CKI(cudaFree(c.entries));
-        c.entries = nullptr;
-        c.cols = d_idx;
-        c.counts = d_val;
-        d_idx = d_val = nullptr;
+    if (c.packed) {
+        if (c.csr_mem) CKI(cudaFree(c.csr_mem));
+        c.csr_mem = nullptr;
+    } else {
+        // two int32 arrays instead of the packed entries
+        if (c.entries) {
+            CKI(cudaFree(c.arena));
+            c.arena = nullptr;
+            CKI(allocate(false));
+        }
+        if (!c.csr_mem && nnz > 0) CKI(stage());
+        c.cols = const_cast<int32_t*>(s_idx);
+        c.counts = const_cast<int32_t*>(s_val);
     }
-    CKI(dalloc(&c.state, (size_t)N));
-    CKI(dalloc(&c.sc, 1));
-    CKI(cudaMallocHost((void**)&c.sc_host, sizeof(DevScalars)));
-    CKI(dalloc(&c.nsub, K2));
-    CKI(dalloc(&c.Ssub, K2 * D));
-    CKI(dalloc(&c.sumlogq, (size_t)c.kmax));
-    CKI(dalloc(&c.acc_nsub, K2));
-    CKI(dalloc(&c.acc_Ssub, K2 * D));
-    CKI(dalloc(&c.acc_logq, (size_t)c.kmax));
-    CKI(dalloc(&c.logpi, (size_t)c.kmax + 1));
-    CKI(dalloc(&c.Lc, (size_t)c.kmax * D));
-    CKI(dalloc(&c.Ls, K2 * D));
-    if (c.opts.local_iters > 1)
-        CKI(dalloc(&c.local_tab, (size_t)D * (size_t)(c.kmax | 1) * 2 + 4));
-    CKI(dalloc(&c.lmap, K2));
-    CKI(dalloc(&c.desc, K2));
-    CKI(dalloc(&c.reinit, (size_t)c.kmax));
-    CKI(dalloc(&c.decide, (size_t)c.kmax));
-    CKI(dalloc(&c.log_h, (size_t)c.kmax));
-    CKI(dalloc(&c.pair_ab, K2));
-    CKI(dalloc(&c.lg_table, lg_table_entries()));
-    CKI(dalloc(&c.move_part, move_partial_bytes()));
-    CKI(dalloc(&c.move_ticket, (size_t)c.kmax));
+    c.sc_host = new (std::nothrow) DevScalars();
+    if (!c.sc_host) return bail(fail(DPMM_ENOMEM, "host allocation failed"));
     CKI(cudaMemsetAsync(c.move_ticket, 0, sizeof(int32_t) * c.kmax, c.stream));
 
     if (c.packed && o.engine != DPMM_ENGINE_CSR_FP32) {
@@ -499,13 +573,9 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         // 16-byte boundary (padding entries have count 0) so that it moves as
         // one bulk copy.  tile_ptr[4 s + q] = first entry of quarter q of
         // segment s; tile_ptr[4 (s + 1)] = end of segment s, padding included.
-        c.tile_T = (int32_t)((N + 127) / 128);
-        c.tile_C = (D + 63) / 64;
-        const int64_t TC = (int64_t)c.tile_T * c.tile_C;
-        CKI(dalloc(&d_qcount, (size_t)(4 * TC)));
-        CKI(dalloc(&c.tile_ptr, (size_t)(4 * TC + 1)));
+        c.tile_T = tT;
+        c.tile_C = tC;
         CKI(launch_tile_count(c.indptr, c.entries, N, c.tile_T, c.tile_C, d_qcount, c.stream));
-        CKI(dalloc(&d_scan, (size_t)tile_scan_words(TC)));
         CKI(cudaMemsetAsync(d_scan, 0, 2 * sizeof(long long), c.stream));
         CKI(launch_tile_scan(d_qcount, TC, c.tile_ptr, d_scan, c.stream));
         long long scan[2] = {0, 0};
@@ -519,8 +589,6 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         CKI(dalloc(&c.tile_ent, (size_t)scan[0]));
         CKI(launch_tile_scatter(c.indptr, c.entries, N, c.tile_T, c.tile_C, c.tile_ptr,
                                 c.tile_ent, c.stream));
-        CKI(dalloc(&c.tile_B, tile_b_bytes(c.tile_C)));
-        CKI(dalloc(&c.noise, (size_t)(kTileMaxK + 2) * (size_t)N));
         c.tile_enabled = true;
     }
     CKI(cudaStreamSynchronize(c.stream));
@@ -536,13 +604,11 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
     CKI(cudaMemcpyAsync(c.sc, c.sc_host, sizeof(DevScalars), cudaMemcpyHostToDevice, c.stream));
     CKI(configure_launches(c));
     CKI(configure_plan_apply(c));
-    CKI(dalloc(&c.gbar, 1));
     CKI(cudaMemsetAsync(c.gbar, 0, sizeof(GridBar), c.stream));
     {
         // this context's chain table: itself
         c.h_chain0 = new (std::nothrow) ChainArgs(chain_args(c));
         if (!c.h_chain0) return bail(fail(DPMM_ENOMEM, "host allocation failed"));
-        CKI(dalloc(&c.d_chains, 1));
         CKI(cudaMemcpyAsync(c.d_chains, c.h_chain0, sizeof(ChainArgs), cudaMemcpyHostToDevice,
                             c.stream));
         c.nchains = 1;
@@ -648,13 +714,15 @@ int dpmm_init_batch(dpmm_ctx** out, int32_t B, const int32_t* const* indptr,
     }
     for (const ChainArgs& a : tab) c.tile_sumT += a.tile_enabled ? a.tile_T : 0;
     cudaError_t e;
-    if ((e = dalloc(&c.gbar, 1)) || (e = dalloc(&c.d_chains, (size_t)B)) ||
-        (e = cudaMemsetAsync(c.gbar, 0, sizeof(GridBar), c.stream)) ||
-        (e = cudaMemcpyAsync(c.d_chains, tab.data(), sizeof(ChainArgs) * B,
+    if ((e = dalloc(&c.gbar_own, 1)) || (e = dalloc(&c.chains_own, (size_t)B)) ||
+        (e = cudaMemsetAsync(c.gbar_own, 0, sizeof(GridBar), c.stream)) ||
+        (e = cudaMemcpyAsync(c.chains_own, tab.data(), sizeof(ChainArgs) * B,
                              cudaMemcpyHostToDevice, c.stream)) ||
         (e = cudaStreamSynchronize(c.stream)))
         return bail(fail(e == cudaErrorMemoryAllocation ? DPMM_ENOMEM : DPMM_ECUDA,
                          "batch table: %s", cudaGetErrorString(e)));
+    c.gbar = c.gbar_own;
+    c.d_chains = c.chains_own;
     c.nchains = B;
     c.mean_row = sum_n > 0 ? sum_nnz / sum_n : 0;
     *out = h;

@@ -133,6 +133,14 @@ struct Ctx {
     int32_t max_count = 0;
     bool packed = false;   // entries stored as (col << 16 | count)
 
+    // the chain's device memory: one allocation that holds every array below but
+    // the unpacked entries (csr_mem) and the blocked copy's entries (tile_ent)
+    char* arena = nullptr;
+    char* csr_mem = nullptr;
+    // of a batch context
+    struct GridBar* gbar_own = nullptr;
+    struct ChainArgs* chains_own = nullptr;
+
     // CSR (device)
     int32_t* indptr = nullptr;
     uint32_t* entries = nullptr;  // packed, or nullptr
@@ -142,7 +150,7 @@ struct Ctx {
     // chain state
     uint32_t* state = nullptr;    // [N]
     DevScalars* sc = nullptr;     // device scalars
-    DevScalars* sc_host = nullptr;  // pinned mirror for reads
+    DevScalars* sc_host = nullptr;  // host mirror for reads
 
     // statistics: main (current state) and accumulators (being built)
     uint32_t* nsub = nullptr;     // [kmax][2]

@@ -1161,22 +1161,32 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
 // takes chunk c = b % C of the tiles t = b / C, b / C + nt, ... (nt tile
 // groups), so its private counters cover only 64 genes ([2K][64] words in
 // shared memory; K > kTileMaxK counts straight into global memory) and its
-// flush adds at most 2K x 64 words.  One warp per (tile, chunk) segment at a
-// time, with the counter row (2 k + r) ld of each of the tile's 128 cells
-// cached (0xFFFFFFFF past the last cell).  Integer sums, exact.
+// flush adds at most 2K x 64 words.  A warp takes one (tile, chunk) segment at a
+// time, with the counter row (2 k + r) ld of each of the tile's 128 cells cached
+// (0xFFFFFFFF past the last cell), or (kQuarter) one quarter of a segment.  An
+// item of fewer tiles than half the warps is taken by quarters: a segment alone
+// is several dependent batches of loads long (2,000 x 500: 12.4 -> 6.9 us), but
+// its quarters fill those batches less well (68,000 x 1,000, 14 tiles an item:
+// 16.0 us by segments, 20.7 by quarters).  Integer sums, exact.
 constexpr int kStatsTileThreads = 512;
 
-template <typename T_>
+template <bool kQuarter, typename T_>
 __device__ __forceinline__ void count_segments(T_* priv, int ld, uint32_t* pn, uint32_t* my,
                                                const uint32_t* __restrict__ state,
                                                const uint32_t* __restrict__ ent,
                                                const int32_t* __restrict__ ptr, int32_t T,
                                                int32_t C, int64_t N, int c, int tg, int nt,
                                                int lane, int w, int nw) {
-    for (int tile = tg + nt * w; tile < T; tile += nt * nw) {
+    constexpr int parts = kQuarter ? 4 : 1, rows = 4 / parts;   // 32-cell row blocks of a unit
+    const int units = parts * ((T - tg + nt - 1) / nt);
+    for (int un = w; un < units; un += nw) {
+        const int tile = tg + nt * (un / parts), q0 = un % parts;
+        const int64_t seg = (int64_t)tile * C + c;
+        const int p0 = ptr[4 * seg + q0] & kTilePtrMask;
+        const int p1 = ptr[4 * seg + (kQuarter ? q0 + 1 : 4)] & kTilePtrMask;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t cell = (int64_t)tile * 128 + lane + 32 * j;
+        for (int j = 0; j < rows; ++j) {
+            const int64_t cell = (int64_t)tile * 128 + 32 * (q0 + j) + lane;
             uint32_t row = 0xFFFFFFFFu;
             if (cell < N) {
                 const uint32_t st = state[cell];
@@ -1184,11 +1194,9 @@ __device__ __forceinline__ void count_segments(T_* priv, int ld, uint32_t* pn, u
                 row = kr * (uint32_t)ld;
                 if (c == 0) atomicAdd(&pn[kr], 1u);
             }
-            my[lane + 32 * j] = row;
+            my[32 * (q0 + j) + lane] = row;
         }
         __syncwarp();
-        const int64_t seg = (int64_t)tile * C + c;
-        const int p0 = ptr[4 * seg], p1 = ptr[4 * seg + 4];
         // an entry of count 0 (segment padding) adds nothing; its cell may lie
         // past the last one, so it is skipped before its row is read
         auto add = [&](uint32_t v) {
@@ -1233,14 +1241,19 @@ stats_tile_item(const ChainArgs& ch, int c, int tg, int nt, uint32_t (*cache)[12
     const int gene0 = c * 64;
     if (K > kTileMaxK) {
         // counts straight into the main rows (global atomics)
-        count_segments(Ssub + gene0, D, acc_nsub, cache[w], state, ent, ptr, T, C, N, c, tg, nt,
+        count_segments<false>(Ssub + gene0, D, acc_nsub, cache[w], state, ent, ptr, T, C, N, c, tg, nt,
                        lane, w, nw);
         return;
     }
     for (int i = threadIdx.x; i < 2 * K * 64; i += blockDim.x) priv[i] = 0u;
     for (int i = threadIdx.x; i < 2 * K; i += blockDim.x) pn[i] = 0u;
     __syncthreads();
-    count_segments(priv, 64, pn, cache[w], state, ent, ptr, T, C, N, c, tg, nt, lane, w, nw);
+    if ((T - tg + nt - 1) / nt < nw / 2)
+        count_segments<true>(priv, 64, pn, cache[w], state, ent, ptr, T, C, N, c, tg, nt, lane, w,
+                             nw);
+    else
+        count_segments<false>(priv, 64, pn, cache[w], state, ent, ptr, T, C, N, c, tg, nt, lane,
+                              w, nw);
     __syncthreads();
     for (int i = threadIdx.x; i < 2 * K * 64; i += blockDim.x) {
         const int u = gene0 + (i & 63);

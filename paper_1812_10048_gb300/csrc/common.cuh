@@ -469,17 +469,24 @@ __device__ __forceinline__ bool grid_sync(GridBar* b) {
     return ok_s != 0;
 }
 
-// n-bar[k][r], S-bar[k][r][u] of the cells of this block's contiguous share
+// n-bar[k][r], S-bar[k][r][u] of the cells of share blk of nblk contiguous ones
 // of [0, N) whose cluster passes `mask` (all if null), added into nsub / Ssub
 // (K clusters).  Block-private shared-memory counters (spriv, priv_cap words)
-// when 2 K D + 2 K words fit, else direct global atomics.  Integer sums.
+// when 2 K D + 2 K words fit, but not for a masked share of fewer than
+// kStatsPrivCells cells (whose few rows are added in global memory faster than
+// the counters are cleared and flushed); else direct global atomics.  Integer
+// sums.
+constexpr int kStatsPrivCells = 64;
+
 __device__ __forceinline__ void stats_cells(const Csr& csr, const uint32_t* __restrict__ state,
                                             const uint8_t* __restrict__ mask,
                                             uint32_t* __restrict__ nsub,
                                             uint32_t* __restrict__ Ssub, int64_t N, int32_t D,
-                                            int K, uint32_t* spriv, int64_t priv_cap) {
+                                            int K, uint32_t* spriv, int64_t priv_cap, int blk,
+                                            int nblk) {
     const int64_t words = (int64_t)2 * K * D;
-    const bool priv = words + 2 * K <= priv_cap;
+    const int64_t per = (N + nblk - 1) / nblk;
+    const bool priv = words + 2 * K <= priv_cap && (!mask || per >= kStatsPrivCells);
     uint32_t* sS = spriv;
     uint32_t* sn = spriv + words;
     if (priv)
@@ -487,8 +494,7 @@ __device__ __forceinline__ void stats_cells(const Csr& csr, const uint32_t* __re
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int warps = blockDim.x >> 5;
-    const int64_t per = (N + gridDim.x - 1) / gridDim.x;
-    const int64_t c0 = (int64_t)blockIdx.x * per, c1 = min(N, c0 + per);
+    const int64_t c0 = (int64_t)blk * per, c1 = min(N, c0 + per);
     for (int64_t cell = c0 + (threadIdx.x >> 5); cell < c1; cell += warps) {
         const uint32_t s = __ldcg(state + cell);
         const uint32_t c = state_label(s), r = state_sub(s);

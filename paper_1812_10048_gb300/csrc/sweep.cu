@@ -1772,18 +1772,18 @@ k_stats(const __grid_constant__ Tab tab, int64_t priv_cap, int sweep) {
             // blocked copy into the accumulators
             if (ch.tile_enabled) continue;
             stats_cells(ch.csr, ch.state, nullptr, ch.acc_nsub, ch.acc_Ssub, ch.N, ch.D, sc->K,
-                        spriv, priv_cap);
+                        spriv, priv_cap, (int)blockIdx.x, (int)gridDim.x);
         } else if (sweep) {
             // a sweep's statistics into the accumulators, unless the CSR label
             // kernel added them (a chain with the blocked copy is counted by
             // the tile statistics kernel)
             if (sc->stats_fused || ch.tile_enabled) continue;
             stats_cells(ch.csr, ch.state, nullptr, ch.acc_nsub, ch.acc_Ssub, ch.N, ch.D, sc->K,
-                        spriv, priv_cap);
+                        spriv, priv_cap, (int)blockIdx.x, (int)gridDim.x);
         } else {
             // every cell into the main statistics (cleared by the caller)
             stats_cells(ch.csr, ch.state, nullptr, ch.nsub, ch.Ssub, ch.N, ch.D, sc->K, spriv,
-                        priv_cap);
+                        priv_cap, (int)blockIdx.x, (int)gridDim.x);
         }
         __syncthreads();
     }

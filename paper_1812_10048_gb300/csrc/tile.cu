@@ -1270,21 +1270,64 @@ stats_tile_item(const ChainArgs& ch, int c, int tg, int nt, uint32_t (*cache)[12
 // warrants: g_b = ceil(T_b / S) clamped to [1, min(T_b, nt)], with nt the tile
 // groups per chunk of the launch and S the tiles per item that give the whole
 // table about two items per block (one item per block for a single chain).
-// The counts are integer sums, so the split into items changes nothing.
+// The counts are integer sums, so the split into items changes nothing.  With
+// several chains (at most kStatsTable) the threads read the table side by side
+// first, so that a block finds its items without a round trip per chain.
+constexpr int kStatsTable = kStatsTileThreads;
+
+__device__ __forceinline__ int stats_groups(const ChainArgs& ch, int32_t nt, int64_t S) {
+    return (int)max((int64_t)1,
+                    min(((int64_t)ch.tile_T + S - 1) / S, (int64_t)min(ch.tile_T, nt)));
+}
+
 template <class Tab>
 __global__ void __launch_bounds__(kStatsTileThreads)
 k_stats_tile(const __grid_constant__ Tab tab, int32_t nt, int64_t S) {
     __shared__ uint32_t cache[kStatsTileThreads / 32][128];
     __shared__ uint32_t priv[2 * kTileMaxK * 64];
     __shared__ uint32_t pn[2 * kTileMaxK];
+    __shared__ int32_t before[kStatsTable + 1], groups[kStatsTable];   // items, tile groups
     const int64_t G = gridDim.x;
+    const int n = tab.n();
+    if (n > 1 && n <= kStatsTable) {
+        const int b = threadIdx.x, lane = b & 31, w = b >> 5;
+        int g = 0, items = 0;
+        if (b < n && tab[b].tile_enabled) {
+            g = stats_groups(tab[b], nt, S);
+            items = tab[b].tile_C * g;
+        }
+        int x = items;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) pn[w] = (uint32_t)x;
+        __syncthreads();
+        int off = x - items;
+        for (int i = 0; i < w; ++i) off += (int)pn[i];
+        if (b < n) {
+            before[b] = off;
+            groups[b] = g;
+            if (b == n - 1) before[n] = off + items;
+        }
+        __syncthreads();
+        int c = 0;
+        for (int id = blockIdx.x; id < before[n]; id += (int)G) {
+            while (before[c + 1] <= id) ++c;
+            const ChainArgs& ch = tab[c];
+            const int i = id - before[c], C = ch.tile_C;
+            stats_tile_item(ch, i % C, i / C, groups[c], cache, priv, pn);
+            __syncthreads();
+        }
+        return;
+    }
     int64_t base = 0;
-    for (int b = 0; b < tab.n(); ++b) {
+    for (int b = 0; b < n; ++b) {
         const ChainArgs& ch = tab[b];
         if (!ch.tile_enabled) continue;
         const int C = ch.tile_C;
-        const int g = (int)max((int64_t)1, min(((int64_t)ch.tile_T + S - 1) / S,
-                                               (int64_t)min(ch.tile_T, nt)));
+        const int g = stats_groups(ch, nt, S);
         const int64_t items = (int64_t)C * g;
         const int64_t first = base + (((int64_t)blockIdx.x - base) % G + G) % G;
         for (int64_t id = first; id < base + items; id += G) {

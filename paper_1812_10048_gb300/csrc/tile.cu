@@ -253,9 +253,11 @@ k_build_b(const __grid_constant__ Tab tab, int32_t force, int32_t rb) {
 // by this CTA are first, first + gridDim.x, ... (cnt of them), where off is
 // the number of listed tiles before chain b.
 __device__ __forceinline__ void chain_tiles(int64_t off, int T, int& first, int& cnt) {
-    const int64_t G = gridDim.x;
-    first = (int)((((int64_t)blockIdx.x - off) % G + G) % G);
-    cnt = first < T ? (T - 1 - first) / (int)G + 1 : 0;
+    const int G = (int)gridDim.x;
+    const int skip = off ? (int)((uint64_t)off % (uint32_t)G) : 0;   // CTA of the first tile
+    first = (int)blockIdx.x - skip;
+    if (first < 0) first += G;
+    cnt = first < T ? (T - 1 - first) / G + 1 : 0;
 }
 
 // Warp roles of the pipelined engine (32 warp numbers; 20, 24 and 28 idle):
@@ -374,13 +376,14 @@ struct TileJob {
 };
 
 // The jobs of this CTA in chain order (called by the whole block; jobs and
-// scratch, 69 words: shared memory).  A batch's chains are read side by side, one thread each: the roles
+// scratch, 70 words: shared memory).  A batch's chains are read side by side, one thread each: the roles
 // used to walk the table themselves, three dependent loads a chain for each of
 // them.
 template <class Tab>
 __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* jobs, int& njobs,
                                           uint32_t& total, int& ntot_max, int& lslot_max,
-                                          int& lmean_max, bool& planes_any, int32_t* scratch) {
+                                          int& lmean_max, bool& planes_any, int& C,
+                                          int32_t* scratch) {
     if (tab.n() == 1) {     // one chain: every thread by itself
         const ChainArgs& ch = tab[0];
         const int K = ch.sc->K, used = ch.sc->tile_used, wide = ch.sc->wide_params;
@@ -391,16 +394,17 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
         if (!job.cnt) return;
         if (threadIdx.x == 0) jobs[0] = job;
         njobs = 1;
-        total = (uint32_t)job.cnt * (uint32_t)ch.tile_C;
+        C = ch.tile_C;
+        total = (uint32_t)job.cnt * (uint32_t)C;
         ntot_max = tile_ntot(K);
         lslot_max = max(4, ch.tile_Lslot);
         lmean_max = max(4, ch.tile_Lmean);
         planes_any = job.planes();
         return;
     }
-    int32_t *wtiles = scratch, *wjobs = wtiles + 32, *smax = wjobs + 32;   // [32], [32], [5]
+    int32_t *wtiles = scratch, *wjobs = wtiles + 32, *smax = wjobs + 32;   // [32], [32], [6]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = (int)(blockDim.x >> 5);
-    if (tid < 5) smax[tid] = 0;      // tiles, ntot, lslot, planes, lmean
+    if (tid < 6) smax[tid] = 0;      // tiles, ntot, lslot, planes, lmean, C
     int64_t tiles_before = 0;
     for (int b0 = 0; b0 < tab.n(); b0 += blockDim.x) {
         const int b = b0 + tid;
@@ -448,10 +452,12 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
             atomicMax(&smax[2], lslot);
             atomicMax(&smax[4], lmean);
             if (k >> 17) smax[3] = 1;
+            smax[5] = tab[b].tile_C;     // (the chains share D)
         }
         __syncthreads();
     }
-    total = (uint32_t)smax[0] * (uint32_t)tab[0].tile_C;
+    C = smax[5];
+    total = (uint32_t)smax[0] * (uint32_t)C;
     ntot_max = smax[1];
     lslot_max = max(4, smax[2]);
     lmean_max = max(4, smax[4]);
@@ -483,20 +489,20 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // this CTA's chains with their tiles, and the largest operand / segment
     TileJob* jobs = reinterpret_cast<TileJob*>(base);
     uint32_t total = 0;   // items of this block
-    int njobs = 0, ntot_max = 0, lslot_max = 4, lmean_max = 4;
+    int njobs = 0, ntot_max = 0, lslot_max = 4, lmean_max = 4, C = 0;
     bool planes_any = false;
-    list_jobs(tab, dbg, jobs, njobs, total, ntot_max, lslot_max, lmean_max, planes_any,
+    list_jobs(tab, dbg, jobs, njobs, total, ntot_max, lslot_max, lmean_max, planes_any, C,
               reinterpret_cast<int32_t*>(smem_raw + smem_bytes - 512));
     if (total == 0) return;
-    base += ((int64_t)njobs * sizeof(TileJob) + 1023) & ~(int64_t)1023;
-    const int C = tab[0].tile_C;     // (the chains share D)
+    base += (njobs * (int)sizeof(TileJob) + 1023) & ~1023;
     // shared-memory plan (identical in every thread): A stages, B stages,
-    // segment slots, then the small area
-    const int64_t b_slot = ((int64_t)ntot_max * 128 + 1023) & ~(int64_t)1023;
-    const int64_t e_max = (int64_t)lslot_max * 4, e_mean = (int64_t)lmean_max * 4;
-    const int64_t avail = smem_bytes - (int64_t)(base - smem_raw) - kSmallBytes;
+    // segments, then the small area.  (In 32-bit integers: 64-bit divisions here
+    // and in the roles' starts cost a block 1 us.)
+    const int b_slot = (ntot_max * 128 + 1023) & ~1023;
+    const int e_max = min(lslot_max, 1 << 20) * 4, e_mean = min(lmean_max, 1 << 20) * 4;
+    const int avail = (int)(smem_bytes - (base - smem_raw)) - kSmallBytes;
     // hi stages, only when some chain of the block has a second plane
-    const int64_t h_bytes = planes_any ? (int64_t)kHiStages * kStageBytes : 0;
+    const int h_bytes = planes_any ? kHiStages * (int)kStageBytes : 0;
     // Producer sets and A stages, the most that fit beside a segment ring for two
     // items of a set and the longest segment.  A set takes every nsets-th item
     // and always meets the same stages and slots, so nsets divides nS and nE:
@@ -504,7 +510,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // item g - nE, and a set's parity wait can never be two phases ahead.  Two
     // stages a set let it fill one while the MMAs read the other.
     auto ring_left = [&](int stages, int b_stages) {
-        return avail - stages * (int64_t)kStageBytes - h_bytes - b_stages * b_slot;
+        return avail - stages * (int)kStageBytes - h_bytes - b_stages * b_slot;
     };
     auto fit = [&](int sets, int stages) {
         return ring_left(stages, 2) >= max(e_max, 2 * sets * e_mean);
@@ -519,16 +525,15 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // more than two B stages only where they leave room for twelve segments
     int nB = 2;
     while (nB < kMaxBStages && ring_left(nS, nB + 1) >= max(e_max, 12 * e_mean)) ++nB;
-    const int64_t e_ring = ring_left(nS, nB) & ~(int64_t)15;
+    const int e_ring = ring_left(nS, nB) & ~15;
     // items in the ring at most: as many as it nearly always has room for, so
     // that a round seldom waits for more than its own slots
     // (fixed slots for the longest segment where two a set fit: a round of the
     // loader is shorter then; 68,000 x 1,000 39 -> 35 us, 8,000 x 32,738
     // 191 -> 172 us, while the ring gives 89 -> 76 us for 24 datasets)
     const bool fixed = e_ring >= 2 * nsets * e_max;
-    const int64_t e_item = fixed ? e_max : e_mean + e_mean / 4;
-    const int nE = (int)min((int64_t)(kMaxESlots / nsets),
-                            max((int64_t)2, e_ring / (e_item * nsets))) * nsets;
+    const int e_item = fixed ? e_max : e_mean + e_mean / 4;
+    const int nE = min(kMaxESlots / nsets, max(2, e_ring / (e_item * nsets))) * nsets;
     if (e_ring < e_max) {
         if (tid == 0) atomicExch(&tab[0].sc->error, DPMM_ECAPACITY);
         return;

@@ -105,3 +105,27 @@ def test_small_beta_draws_take_bf16(P):
     s.close()
     from oracle.ari import adjusted_rand_index
     assert adjusted_rand_index(labels, ds.labels) > 0.98
+
+
+def test_batch_whose_first_chain_has_no_blocked_copy(P):
+    """Unpackable counts in the first dataset: the others still go to the
+    tensor cores, each evolving as alone."""
+    rng = np.random.default_rng(8)
+    data = []
+    for i, N in enumerate([300, 700, 150]):
+        X = sparse(N, 200, 0.2, rng)
+        if i == 0:
+            X.data[5] = 70000
+        data.append((X.indptr.astype(np.int32), X.indices.astype(np.int32),
+                     X.data.astype(np.int32), N))
+    b = P.BatchSampler(data, 200, 1.0, 0.5, kmax=16, seed=3, engine=P.ENGINE_TILE_BF16)
+    b.step(6)
+    for i, d in enumerate(data):
+        s = P.Sampler(*d[:3], d[3], 200, 1.0, 0.5, kmax=16, seed=3, chain_id=i,
+                      engine=P.ENGINE_TILE_BF16)
+        s.step(6)
+        assert P.dpmm_debug_engine(b.chain(i).ctx) == (i > 0)
+        for x, y in zip(s.get_state(), b.chain(i).get_state()):
+            np.testing.assert_array_equal(x, y)
+        s.close()
+    b.close()

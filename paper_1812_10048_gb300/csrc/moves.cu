@@ -171,6 +171,14 @@ __device__ __forceinline__ void move_item(DevScalars* sc, const uint32_t* __rest
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int Dc = (D + G - 1) / G;
     const int u0 = g * Dc, u1 = min(D, u0 + Dc);
+    // what the completion needs is asked for with the genes' sums, not after the
+    // ticket (three round trips one after the other there)
+    const int a = split ? e : min(pair_s[0], pair_s[1]);
+    const int b = split ? e : max(pair_s[0], pair_s[1]);
+    const uint2 ca = reinterpret_cast<const uint2*>(nsub)[a];
+    const uint2 cb = reinterpret_cast<const uint2*>(nsub)[b];
+    const double slq = split && split_q ? sumlogq[e] : 0.0;
+    const double lgDb = __ldg(tb.tot);
     double acc = 0.0;
     unsigned long long Ta = 0, Tb = 0;
     // eq. 18 (instantiated): the pre-compaction row of cluster e in the
@@ -187,28 +195,28 @@ __device__ __forceinline__ void move_item(DevScalars* sc, const uint32_t* __rest
         const uint32_t* S0 = Ssub + (size_t)(2 * e) * D;
         const uint32_t* S1 = S0 + D;
         for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
-            const uint32_t a = S0[u], b = S1[u];
-            Ta += a;
-            Tb += b;
+            const uint32_t s0 = S0[u], s1 = S1[u];
+            Ta += s0;
+            Tb += s1;
             if (inst_row >= 0) {
                 const size_t r = (size_t)u * kmax + inst_row;
                 const double l0 = Ls[2 * r], l1 = Ls[2 * r + 1], lk = Lc[r];
-                acc += (beta - 1.0 + a) * l0 + (beta - 1.0 + b) * l1 - (beta - 1.0 + a + b) * lk;
+                acc += (beta - 1.0 + s0) * l0 + (beta - 1.0 + s1) * l1 -
+                       (beta - 1.0 + s0 + s1) * lk;
             }
         }
     } else if (split) {
         const uint32_t* S0 = Ssub + (size_t)(2 * e) * D;
         const uint32_t* S1 = S0 + D;
         for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
-            const uint32_t a = S0[u], b = S1[u];
-            Ta += a;
-            Tb += b;
-            if (a && b)
-                acc += lg_shift(a, beta, lg_beta, tb) + lg_shift(b, beta, lg_beta, tb) -
-                       lg_shift(a + b, beta, lg_beta, tb);
+            const uint32_t s0 = S0[u], s1 = S1[u];
+            Ta += s0;
+            Tb += s1;
+            if (s0 && s1)
+                acc += lg_shift(s0, beta, lg_beta, tb) + lg_shift(s1, beta, lg_beta, tb) -
+                       lg_shift(s0 + s1, beta, lg_beta, tb);
         }
     } else {
-        const int a = min(pair_s[0], pair_s[1]), b = max(pair_s[0], pair_s[1]);
         const uint32_t* A0 = Ssub + (size_t)(2 * a) * D;
         const uint32_t* B0 = Ssub + (size_t)(2 * b) * D;
         for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
@@ -246,17 +254,8 @@ __device__ __forceinline__ void move_item(DevScalars* sc, const uint32_t* __rest
     Ta = warp_sum(Ta);
     Tb = warp_sum(Tb);
     const uint32_t m = m0;
-    uint32_t na, nb;
-    int a = e;
-    if (split) {
-        na = nsub[2 * e];
-        nb = nsub[2 * e + 1];
-    } else {
-        a = min(pair_s[0], pair_s[1]);
-        const int b = max(pair_s[0], pair_s[1]);
-        na = nsub[2 * a] + nsub[2 * a + 1];
-        nb = nsub[2 * b] + nsub[2 * b + 1];
-    }
+    const uint32_t na = split ? ca.x : ca.x + ca.y;
+    const uint32_t nb = split ? ca.y : cb.x + cb.y;
     const double Db = (double)D * beta;
     double v0 = 0.0, v1 = 0.0;
     if (w == 0) {
@@ -281,7 +280,6 @@ __device__ __forceinline__ void move_item(DevScalars* sc, const uint32_t* __rest
     __syncthreads();
     if (threadIdx.x != 0) return;
     ticket[e] = 0;
-    const double lgDb = __ldg(tb.tot);
     const double lfa = lgDb - fin[1][0], lfb = lgDb - fin[2][0], lfab = lgDb - fin[3][0];
     const double lna = fin[1][1], lnb = fin[2][1], lnab = fin[3][1];
     acc = fin[0][0];
@@ -305,7 +303,7 @@ __device__ __forceinline__ void move_item(DevScalars* sc, const uint32_t* __rest
         } else {
             lh = log_alpha + lna + lnb - lnab + lfa + lfb - lfab + acc;
         }
-        if (split_q) lh -= sumlogq[e];
+        if (split_q) lh -= slq;
         decide[e] = log_u < lh ? 1 : 0;
         log_h[e] = lh;
     } else {
@@ -435,9 +433,24 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* tmp, int* total)
     return excl;
 }
 
-// The plan of a sweep's compaction or of a split/merge call (one block of
-// kPlanThreads threads, thread k for cluster k): label map, statistics-gather
-// descriptors and the new n-bar / sum log q of every surviving cluster.
+// What thread k of a plan reads of cluster k, whatever K is (the arrays hold kmax
+// entries): asked for before K is known.
+struct PlanLoads {
+    uint2 n;                       // n-bar: the sweep's accumulator, or the current one
+    unsigned long long logq;       // the sweep's sum log q accumulator
+    int32_t decide;
+};
+__device__ __forceinline__ PlanLoads plan_loads(const ChainArgs& ch, bool compact) {
+    PlanLoads p{make_uint2(0u, 0u), 0ull, 0};
+    const int k = threadIdx.x;
+    if (k < ch.kmax) {
+        p.n = reinterpret_cast<const uint2*>(compact ? ch.acc_nsub : ch.nsub)[k];
+        if (compact) p.logq = ch.acc_logq[k];
+        else p.decide = ch.decide[k];
+    }
+    return p;
+}
+
 struct PlanSmem {
     int tmp[32];
     uint8_t removed[kMaxKmax];
@@ -448,13 +461,16 @@ struct PlanSmem {
     int32_t napplying;
 };
 
+// The plan of a sweep's compaction or of a split/merge call (one block of
+// kPlanThreads threads, thread k for cluster k): label map, statistics-gather
+// descriptors and the new n-bar / sum log q of every surviving cluster.
 __device__ void plan_block(DevScalars* sc, int32_t kind, uint32_t* __restrict__ nsub,
                            double* __restrict__ sumlogq, uint32_t* __restrict__ acc_nsub,
                            const unsigned long long* __restrict__ acc_logq,
                            const int32_t* __restrict__ decide,
                            const int32_t* __restrict__ pair_ab, uint32_t* __restrict__ lmap,
                            int32_t* __restrict__ desc, uint8_t* __restrict__ reinit,
-                           int32_t kmax, uint32_t* bump, PlanSmem& sm) {
+                           int32_t kmax, uint32_t* bump, const PlanLoads& pl, PlanSmem& sm) {
     int* tmp = sm.tmp;
     uint8_t* removed = sm.removed;
     int32_t* partner = sm.partner;
@@ -471,9 +487,9 @@ __device__ void plan_block(DevScalars* sc, int32_t kind, uint32_t* __restrict__ 
         uint32_t n0 = 0, n1 = 0;
         double sq = 0.0;
         if (k < K) {
-            n0 = acc_nsub[2 * k];
-            n1 = acc_nsub[2 * k + 1];
-            sq = logq_value(acc_logq[k]);
+            n0 = pl.n.x;
+            n1 = pl.n.y;
+            sq = logq_value(pl.logq);
         }
         const bool keep = n0 + n1 > 0;
         const int j = block_exclusive_scan(keep ? 1 : 0, tmp, &total);
@@ -510,9 +526,9 @@ __device__ void plan_block(DevScalars* sc, int32_t kind, uint32_t* __restrict__ 
         uint32_t n0 = 0, n1 = 0;
         int d = 0;
         if (k < K) {
-            n0 = nsub[2 * k];
-            n1 = nsub[2 * k + 1];
-            d = decide[k];
+            n0 = pl.n.x;
+            n1 = pl.n.y;
+            d = pl.decide;
         }
         const int j = block_exclusive_scan(d, tmp, &total);
         const int room = kmax - K;
@@ -559,7 +575,7 @@ __device__ void plan_block(DevScalars* sc, int32_t kind, uint32_t* __restrict__ 
         into[k] = -1;
     }
     __syncthreads();
-    if (k < P && decide[k]) {
+    if (k < P && pl.decide) {
         const int a = pair_ab[2 * k], b = pair_ab[2 * k + 1];
         removed[b] = 1;
         partner[a] = b;
@@ -572,8 +588,8 @@ __device__ void plan_block(DevScalars* sc, int32_t kind, uint32_t* __restrict__ 
     uint32_t n0 = 0, n1 = 0, nb0 = 0, nb1 = 0;
     double sq = 0.0;
     if (k < K) {
-        n0 = nsub[2 * k];
-        n1 = nsub[2 * k + 1];
+        n0 = pl.n.x;
+        n1 = pl.n.y;
         sq = sumlogq[k];
         if (partner[k] >= 0) {
             nb0 = nsub[2 * partner[k]];
@@ -657,10 +673,11 @@ __device__ __forceinline__ int plan_changes(const Tab& tab, bool compact) {
     return __syncthreads_or(change);
 }
 
-__device__ __forceinline__ void plan_chain(const ChainArgs& ch, bool compact, PlanSmem& sm) {
+__device__ __forceinline__ void plan_chain(const ChainArgs& ch, bool compact, const PlanLoads& pl,
+                                           PlanSmem& sm) {
     plan_block(ch.sc, compact ? PLAN_COMPACT : PLAN_SPLIT, ch.nsub, ch.sumlogq, ch.acc_nsub,
                ch.acc_logq, ch.decide, ch.pair_ab, ch.lmap, ch.desc, ch.reinit, ch.kmax,
-               compact ? &ch.sc->t : &ch.sc->m, sm);
+               compact ? &ch.sc->t : &ch.sc->m, pl, sm);
 }
 
 // priv_cap: words of dynamic shared memory for the recount.
@@ -670,11 +687,31 @@ k_plan_apply(const __grid_constant__ Tab tab, int32_t kind, GridBar* bar, int64_
     extern __shared__ __align__(16) uint32_t spriv[];
     __shared__ PlanSmem sm;
     const bool compact = kind == PLAN_COMPACT;
-    const int any = plan_changes(tab, compact);
-    // chain b is planned by block b % gridDim.x
-    for (int b = blockIdx.x; b < tab.n(); b += gridDim.x) {
-        plan_chain(tab[b], compact, sm);
-        __syncthreads();
+    int any = 0;
+    if (tab.n() == 1) {
+        // one chain: each thread decides from its own cluster's loads, which
+        // block 0 plans with
+        const ChainArgs& ch = tab[0];
+        const PlanLoads pl = plan_loads(ch, compact);
+        const int K = ch.sc->K, sel = ch.sc->chain_sel, k = threadIdx.x;
+        bool change = false;
+        if (compact)
+            change = k < K && (pl.n.x + pl.n.y == 0u ||
+                               (pl.n.x + pl.n.y >= 2u && (pl.n.x == 0u || pl.n.y == 0u)));
+        else
+            change = pl.decide && (sel == 1 ? K < ch.kmax && k < K : k < K / 2);
+        any = __syncthreads_or(change);
+        if (blockIdx.x == 0) {
+            plan_chain(ch, compact, pl, sm);
+            __syncthreads();
+        }
+    } else {
+        any = plan_changes(tab, compact);
+        // chain b is planned by block b % gridDim.x
+        for (int b = blockIdx.x; b < tab.n(); b += gridDim.x) {
+            plan_chain(tab[b], compact, plan_loads(tab[b], compact), sm);
+            __syncthreads();
+        }
     }
     if (!any) return;
     if (!grid_sync(bar)) {

@@ -29,6 +29,8 @@
 
 #include <climits>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -1254,182 +1256,241 @@ __device__ __forceinline__ float2 sub_pair(const Csr& csr, int64_t beg, int64_t 
     return make_float2(warp_sum(t0), warp_sum(t1));
 }
 
-// Column of the reduce-scatter result held by `lane` (see warp_reduce_scatter).
-template <int P>
-__device__ __forceinline__ int lane_column(int lane) {
-    int base = 0, o = 16;
-#pragma unroll
-    for (int m = P; m > 1; m >>= 1) {
-        if (lane & o) base += m >> 1;
-        o >>= 1;
-    }
-    return base;
-}
-
-// Smallest lane holding column `col` (inverse of lane_column).
-template <int P>
-__device__ __forceinline__ int lane_of_column(int col) {
-    int lane = 0, o = 16;
-#pragma unroll
-    for (int m = P; m > 1; m >>= 1) {
-        const int h = m >> 1;
-        if (col >= h) {
-            lane |= o;
-            col -= h;
+// K <= 32 with the tables (and, when they fit, the statistics) in shared memory.
+// LPE lanes hold one entry's cluster row (a float4 each), so that a warp takes
+// 32 / LPE entries at a time with one 16-byte load per lane, and entry i of a row
+// belongs to slot i mod 32: a slot sums its entries in row order, the slots are
+// combined over slot distance 16, 8, 4, 2, 1 (those 32 / LPE and more apart within
+// the lane, the others by shuffles), which is the order that warp_reduce_scatter
+// has too.
+//
+// What bounds it is shared memory (the gathers' bank conflicts, the counters)
+// and the issue slots about evenly.  A lane that reads a row of its own meets
+// others on a bank more often (2.6 turns for each eight 16-byte loads of random
+// rows, 1.5 with four lanes a row), and noise and draws of one cell at a time leave
+// most lanes idle: 1,100 instructions a cell.  So the block's cells
+// [N b / G, N (b + 1) / G) are taken in batches of at most 1,024, 32 a warp: the
+// label noise of 32 / LPE cells is one Philox call, and the eq. 8 draws of a batch
+// run on all lanes (lane i draws cell i); then the rows are
+// read again (from the L2) for the counters.  A step of 68,000 x 1,000 cells: K = 4
+// 104 -> 85 us, K = 10 126 -> 105, K = 16 230 -> 148, K = 30 465 -> 267; 1,000 cells,
+// K = 10: 51 -> 44.  Rows are held in eight registers a lane, up to 256 entries (four:
+// 110 us at K = 10).
+template <int LPE, bool packed>
+__device__ __forceinline__ void assign_held(const ChainArgs& a, const float* sLc, int Kp,
+                                            const float2* Ls2, int ldS, int K, uint32_t t,
+                                            const float* spi, const float* slw,
+                                            unsigned long long* blk_logq, uint32_t* bn,
+                                            uint32_t* sS) {
+    constexpr int E = 32 / LPE;                   // entries a step
+    constexpr int R = packed && LPE <= 4 ? 8 : 4; // 32-entry pieces held in registers
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nw = (int)(blockDim.x >> 5);
+    const int ql = lane % LPE, g = lane / LPE;    // float4 of the row, entry of the step
+    // (a lane past the row reads its first float4, which is then not looked at)
+    const float4* row4 = reinterpret_cast<const float4*>(sLc) + (4 * ql < Kp ? ql : 0);
+    const int ld4 = Kp >> 2;
+    const int64_t b0 = a.N * blockIdx.x / gridDim.x, b1 = a.N * (blockIdx.x + 1) / gridDim.x;
+    for (int64_t c0 = b0; c0 < b1; c0 += 32 * nw) {
+        // lane i: cell c0 + w + nw i of the batch
+        const int64_t cell = c0 + w + (int64_t)nw * lane;
+        const bool mine = cell < b1;
+        const int cells = (int)max((int64_t)0, min((int64_t)32, (b1 - c0 - w + nw - 1) / nw));
+        long long beg = 0;
+        int len = 0;
+        uint32_t old = 0u;
+        if (mine) {
+            beg = a.csr.indptr[cell];
+            len = (int)(a.csr.indptr[cell + 1] - beg);
+            old = a.state[cell];
         }
-        o >>= 1;
-    }
-    return lane;
-}
-
-constexpr int kRowRegs = 8;   // row entries a lane keeps in registers (rows up to 256)
-
-// K <= 32: tables (and, when they fit, the statistics) in shared memory.
-// Per cell (one warp): the Philox words and the old state are fetched first;
-// the row's entries are read once into registers (rows longer than 256
-// entries re-read their tail); pass 1 forms per-lane partial sums against the
-// cluster table and a reduce-scatter gives every lane one cluster total;
-// Gumbel-max picks c; pass 2 gathers the two sub-cluster factors of c; lane 0
-// draws the eq. 8 sub-label; pass 3 adds the row into the block's statistics.
-template <int P>
-__device__ __forceinline__ void assign_cells_v2(const ChainArgs& a, const float* sLc, int Kp,
-                                                const float2* Ls2, int ldS, int K, uint32_t t,
-                                                const float* spi, const float* slw,
-                                                unsigned long long* wsq, uint32_t* wn,
-                                                uint32_t* sS) {
-    const int lane = threadIdx.x & 31;
-    const int wid = threadIdx.x >> 5;
-    const int64_t warp0 = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int col = lane_column<P>(lane);
-    // lanes whose column is unused draw the eq. 8 Gumbels: the lane of
-    // column K takes word 0, that of column K + 1 word 1 (when P >= K + 2)
-    const bool spare = P >= K + 2;
-    const int sub_word = col - K;                       // 0 or 1 on those lanes
-    const bool packed = a.csr.entries != nullptr;
-    constexpr int R = P <= 16 ? kRowRegs : kRowRegs / 2;   // register budget at 1024 threads
-    unsigned long long* my_sq = wsq + (size_t)wid * K;
-    uint32_t* my_n = wn + (size_t)wid * 2 * K;
-    for (int64_t cell = warp0; cell < a.N; cell += nwarps) {
-        const int64_t beg = a.csr.indptr[cell], end = a.csr.indptr[cell + 1];
-        const uint32_t old = lane == 0 ? a.state[cell] : 0u;
-        // one Philox call and one Gumbel per lane: label noise of the lane's
-        // column, or (spare lanes) the sub-label noise
-        // counters chosen per lane so that the whole warp runs one Philox call
-        const bool lab = col < K;
-        const uint4 w = a.st.words(lab ? TAG_LABEL : TAG_SUBLABEL, (uint32_t)cell, t,
-                                   lab ? (uint32_t)(col >> 2) : 0u);
-        const float g = gumbel(word_of(w, lab ? (col & 3) : (sub_word & 1)));
-        float h0, h1;
-        if (spare) {
-            h0 = __shfl_sync(0xFFFFFFFFu, g, lane_of_column<P>(K));
-            h1 = __shfl_sync(0xFFFFFFFFu, g, lane_of_column<P>(K + 1));
-        } else {
-            const uint4 ws = a.st.words(TAG_SUBLABEL, (uint32_t)cell, t, 0u);
-            h0 = gumbel(ws.x);
-            h1 = gumbel(ws.y);
-        }
-        const int len = (int)(end - beg);
-        const int slots = min(R, (len + 31) >> 5);
-        const uint32_t* row_ent = a.csr.entries + beg;
-        // pass 1: entries -> registers, partial sums against the cluster table
-        uint32_t ent[R];
-        float acc[P];
+        int c = -1;
+        float2 lik = make_float2(0.0f, 0.0f);
+        float n0 = 0.0f, n1 = 0.0f, n2 = 0.0f, n3 = 0.0f;   // noise of 4 ql .. 4 ql + 3
+        for (int i = 0; i < cells; ++i) {
+            if (i % E == 0) {
+                // lane (g, ql): cell i + g, clusters from 4 ql
+                const uint4 wd = a.st.words(TAG_LABEL,
+                                            (uint32_t)(c0 + w + (int64_t)nw * (i + g)), t,
+                                            (uint32_t)ql);
+                n0 = gumbel(wd.x);
+                n1 = gumbel(wd.y);
+                n2 = gumbel(wd.z);
+                n3 = gumbel(wd.w);
+            }
+            const long long rb = __shfl_sync(0xFFFFFFFFu, beg, i);
+            const int rl = __shfl_sync(0xFFFFFFFFu, len, i);
+            uint32_t ev[R], xv[R];
+            auto fetch = [&](int e0, int r) {
+                ev[r] = xv[r] = 0u;
+                const int e = e0 + 32 * r + lane;
+                if (e < rl) {
+                    if (packed) {
+                        ev[r] = __ldg(a.csr.entries + rb + e);
+                    } else {
+                        ev[r] = (uint32_t)__ldg(a.csr.cols + rb + e);
+                        xv[r] = (uint32_t)__ldg(a.csr.counts + rb + e);
+                    }
+                }
+            };
+            float4 acc[LPE];
 #pragma unroll
-        for (int j = 0; j < P; ++j) acc[j] = 0.0f;
-        auto add_row = [&](int32_t u, int32_t x) {
-            const float xf = (float)x;
-            const float4* row = reinterpret_cast<const float4*>(sLc + u * Kp);
+            for (int j = 0; j < LPE; ++j) acc[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            auto piece = [&](uint32_t e, uint32_t ex, auto whole, int n) {
 #pragma unroll
-            for (int q = 0; q < P / 4; ++q) {
-                if (4 * q < Kp) {
-                    const float4 l = row[q];
-                    acc[4 * q] = fmaf(xf, l.x, acc[4 * q]);
-                    acc[4 * q + 1] = fmaf(xf, l.y, acc[4 * q + 1]);
-                    acc[4 * q + 2] = fmaf(xf, l.z, acc[4 * q + 2]);
-                    acc[4 * q + 3] = fmaf(xf, l.w, acc[4 * q + 3]);
+                for (int j = 0; j < LPE; ++j) {
+                    const uint32_t v =
+                        LPE == 1 ? e : __shfl_sync(0xFFFFFFFFu, e, E * j + g);
+                    const uint32_t x = packed     ? v & 0xFFFFu
+                                       : LPE == 1 ? ex
+                                                  : __shfl_sync(0xFFFFFFFFu, ex, E * j + g);
+                    if (whole || E * j + g < n) {
+                        const float4 l = row4[(int)(packed ? v >> 16 : v) * ld4];
+                        const float xf = (float)(int32_t)x;
+                        acc[j].x = fmaf(xf, l.x, acc[j].x);
+                        acc[j].y = fmaf(xf, l.y, acc[j].y);
+                        acc[j].z = fmaf(xf, l.z, acc[j].z);
+                        acc[j].w = fmaf(xf, l.w, acc[j].w);
+                    }
+                }
+            };
+            for (int e0 = 0; e0 < rl; e0 += 32 * R) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) fetch(e0, r);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int n = rl - e0 - 32 * r;      // entries of this piece on
+                    if (n <= 0) break;
+                    // (no branch between the steps of a whole piece: their loads overlap)
+                    if (n >= 32) piece(ev[r], xv[r], std::true_type{}, n);
+                    else piece(ev[r], xv[r], std::false_type{}, n);
                 }
             }
-        };
-        if (packed) {
+            // slots E j + g: over j within the lane, then over g
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                ent[r] = 0u;
-                if (r < slots && lane + 32 * r < len) ent[r] = __ldg(row_ent + lane + 32 * r);
+            for (int h = LPE / 2; h >= 1; h >>= 1)
+#pragma unroll
+                for (int j = 0; j < h; ++j) {
+                    acc[j].x += acc[j + h].x;
+                    acc[j].y += acc[j + h].y;
+                    acc[j].z += acc[j + h].z;
+                    acc[j].w += acc[j + h].w;
+                }
+            float4 sc = acc[0];
+#pragma unroll
+            for (int o = 16; o >= LPE; o >>= 1) {
+                sc.x += __shfl_xor_sync(0xFFFFFFFFu, sc.x, o);
+                sc.y += __shfl_xor_sync(0xFFFFFFFFu, sc.y, o);
+                sc.z += __shfl_xor_sync(0xFFFFFFFFu, sc.z, o);
+                sc.w += __shfl_xor_sync(0xFFFFFFFFu, sc.w, o);
             }
+            // the LPE lanes that hold this cell's noise take its largest value
+            float bv = -CUDART_INF_F;
+            int bk = 0x7FFFFFFF;
+            if (g == i % E) {
+                auto take = [&](int k, float s, float noise) {
+                    if (k < K) {
+                        const float v = (spi[k] + s) + noise;
+                        if (v > bv || (v == bv && k < bk)) {
+                            bv = v;
+                            bk = k;
+                        }
+                    }
+                };
+                take(4 * ql, sc.x, n0);
+                take(4 * ql + 1, sc.y, n1);
+                take(4 * ql + 2, sc.z, n2);
+                take(4 * ql + 3, sc.w, n3);
+            }
+            // the warp's largest value, then the lowest cluster that has it
+            // (floats in the order of their sortable integers; no NaN here)
+            const uint32_t fb = __float_as_uint(bv + 0.0f);   // (-0 as 0)
+            const uint32_t key = fb & 0x80000000u ? ~fb : fb | 0x80000000u;
+            const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, key);
+            int ci = (int)__reduce_min_sync(0xFFFFFFFFu,
+                                            key == top ? (uint32_t)bk : 0x7FFFFFFFu);
+            if (ci >= K) ci = 0;       // every score a NaN: some cluster of the table
+            // eq. 8 likelihood factors of that cluster
+            float t[2] = {0.0f, 0.0f};
+            auto add = [&](int32_t u, int32_t x) {
+                const float2 l = Ls2[u * ldS + ci];
+                t[0] = fmaf((float)x, l.x, t[0]);
+                t[1] = fmaf((float)x, l.y, t[1]);
+            };
+            if (rl <= 32 * R) {
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-                if (r < slots && lane + 32 * r < len)
-                    add_row((int32_t)(ent[r] >> 16), (int32_t)(ent[r] & 0xFFFFu));
-        }
-        for (int64_t e = beg + lane + (packed ? 32 * R : 0); e < end; e += 32) {
-            int32_t u, x;
-            a.csr.get(e, u, x);
-            add_row(u, x);
-        }
-        int colr;
-        const float sc = warp_reduce_scatter<P>(acc, lane, &colr);
-        const float v = col < K ? (spi[col] + sc) + g : -CUDART_INF_F;
-        const int c = warp_argmax(v, col < K ? col : 0x7FFFFFFF);
-        // pass 2: eq. 8 likelihood factors of cluster c
-        float t0 = 0.0f, t1 = 0.0f;
-        if (packed) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (r < slots && lane + 32 * r < len) {
-                    const float2 l = Ls2[(int)(ent[r] >> 16) * ldS + c];
-                    const float xf = (float)(ent[r] & 0xFFFFu);
-                    t0 = fmaf(xf, l.x, t0);
-                    t1 = fmaf(xf, l.y, t1);
+                for (int r = 0; r < R; ++r) {
+                    if (32 * r >= rl) break;
+                    if (32 * r + lane < rl)
+                        add((int32_t)(packed ? ev[r] >> 16 : ev[r]),
+                            (int32_t)(packed ? ev[r] & 0xFFFFu : xv[r]));
+                }
+            } else {
+                for (int e = lane; e < rl; e += 32) {
+                    int32_t u, x;
+                    a.csr.get(rb + e, u, x);
+                    add(u, x);
                 }
             }
+            int side;
+            const float ts = warp_reduce_scatter<2>(t, lane, &side);
+            const float t0 = __shfl_sync(0xFFFFFFFFu, ts, 0);
+            const float t1 = __shfl_sync(0xFFFFFFFFu, ts, 16);
+            if (lane == i) {
+                c = ci;
+                lik = make_float2(t0, t1);
+            }
         }
-        for (int64_t e = beg + lane + (packed ? 32 * R : 0); e < end; e += 32) {
-            int32_t u, x;
-            a.csr.get(e, u, x);
-            const float2 l = Ls2[(size_t)u * ldS + c];
-            t0 = fmaf((float)x, l.x, t0);
-            t1 = fmaf((float)x, l.y, t1);
-        }
-        t0 = warp_sum(t0);
-        t1 = warp_sum(t1);
-        uint32_t s = 0;
-        if (lane == 0) {
+        uint32_t s = 0u;
+        unsigned long long q = 0ull;
+        if (mine) {
             // log weights of eq. 8: log n-bar, or log(n-bar - 1) for the cell's own old slot
             const bool stays = state_label(old) == (uint32_t)c;
             const uint32_t so = state_sub(old);
             const float lw0 = slw[4 * c + (stays && so == 0 ? 1 : 0)];
             const float lw1 = slw[4 * c + 2 + (stays && so == 1 ? 1 : 0)];
             const bool both_empty = lw0 == -CUDART_INF_F && lw1 == -CUDART_INF_F;
-            const float l0 = (both_empty ? 0.0f : lw0) + t0;
-            const float l1 = (both_empty ? 0.0f : lw1) + t1;
-            s = (l1 + h1 > l0 + h0) ? 1u : 0u;
+            const float l0 = (both_empty ? 0.0f : lw0) + lik.x;
+            const float l1 = (both_empty ? 0.0f : lw1) + lik.y;
+            const uint4 h = a.st.words(TAG_SUBLABEL, (uint32_t)cell, t, 0u);
+            s = (l1 + gumbel(h.y) > l0 + gumbel(h.x)) ? 1u : 0u;
             const float mx = fmaxf(l0, l1), mn = fminf(l0, l1);
-            const float logq = (s ? l1 : l0) - (mx + log1pf(expf(mn - mx)));
+            q = logq_fixed((s ? l1 : l0) - (mx + log1pf(expf(mn - mx))));
             a.state[cell] = pack_state((uint32_t)c, s);
-            my_sq[c] += logq_fixed(logq);
-            my_n[2 * c + s] += 1u;
         }
-        if (sS) {
-            // pass 3: the row into the block's statistics of (c, s)
-            s = __shfl_sync(0xFFFFFFFFu, s, 0);
-            uint32_t* dst = sS + (size_t)(2 * c + s) * a.D;
-            if (packed) {
+        warp_add_by_cluster(blk_logq, c, q);
+        if (!sS) continue;
+        // the rows once more, into the block's statistics of (c, s)
+        if (mine) atomicAdd(&bn[2 * c + s], 1u);
+        for (int i = 0; i < cells; ++i) {
+            const long long rb = __shfl_sync(0xFFFFFFFFu, beg, i);
+            const int rl = __shfl_sync(0xFFFFFFFFu, len, i);
+            uint32_t* dst = sS + (size_t)__shfl_sync(0xFFFFFFFFu, 2 * c + (int)s, i) * a.D;
+            for (int e0 = lane; e0 < rl; e0 += 32 * 4) {
+                uint32_t u[4], x[4];
 #pragma unroll
-                for (int r = 0; r < R; ++r)
-                    if (r < slots && lane + 32 * r < len && (ent[r] & 0xFFFFu))
-                        atomicAdd(dst + (ent[r] >> 16), ent[r] & 0xFFFFu);
-            }
-            for (int64_t e = beg + lane + (packed ? 32 * R : 0); e < end; e += 32) {
-                int32_t u, x;
-                a.csr.get(e, u, x);
-                if (x) atomicAdd(dst + u, (uint32_t)x);
+                for (int r = 0; r < 4; ++r) {
+                    u[r] = x[r] = 0u;
+                    if (e0 + 32 * r < rl) {
+                        if (packed) {
+                            u[r] = __ldg(a.csr.entries + rb + e0 + 32 * r);
+                        } else {
+                            u[r] = (uint32_t)__ldg(a.csr.cols + rb + e0 + 32 * r);
+                            x[r] = (uint32_t)__ldg(a.csr.counts + rb + e0 + 32 * r);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t n = packed ? u[r] & 0xFFFFu : x[r];
+                    if (n) atomicAdd(dst + (packed ? u[r] >> 16 : u[r]), n);
+                }
             }
         }
     }
 }
 
-// K > 32, or tables too long for assign_cells_v2: the cluster table passes
+// K > 32, or tables too long for assign_held: the cluster table passes
 // through shared memory in slabs of 4 LPE clusters (row stride 4 LPE floats).
 // LPE lanes hold one entry's slab row (a float4 each), so that a warp adds
 // 32 / LPE entries with one 16-byte shared-memory load per lane; LPE x 16 bytes
@@ -1633,14 +1694,10 @@ __device__ __forceinline__ void assign_chain(const ChainArgs& a, int64_t smem_by
     if (a.sc->tile_used) return;   // the dense-tile engine labelled this sweep
     const int K = a.sc->K;
     const uint32_t t = a.sc->t;
-    // per-warp accumulators exist only on the K <= 32 path
-    const int nw = K <= 32 ? (int)(blockDim.x >> 5) : 0;
-    // small per-block arrays first: per-warp sum log q and n-bar, block sum log q,
-    // log pi and the sweep-start n-bar
-    unsigned long long* wsq = reinterpret_cast<unsigned long long*>(smem_raw);   // [nw][K]
-    unsigned long long* blk_logq = wsq + (size_t)nw * K;                         // [K]
-    uint32_t* wn = reinterpret_cast<uint32_t*>(blk_logq + K);            // [nw][2K]
-    float* spi = reinterpret_cast<float*>(wn + (size_t)nw * 2 * K);      // [K]
+    // small per-block arrays first: sum log q, n-bar, log pi and the eq. 8 weights
+    unsigned long long* blk_logq = reinterpret_cast<unsigned long long*>(smem_raw);   // [K]
+    uint32_t* bn = reinterpret_cast<uint32_t*>(blk_logq + K);            // [2K]
+    float* spi = reinterpret_cast<float*>(bn + 2 * K);                   // [K]
     float* slw = spi + K;                                                // [K][2][2]
     const size_t head = ((size_t)(reinterpret_cast<unsigned char*>(slw + 4 * K) - smem_raw) + 15) &
                         ~(size_t)15;
@@ -1650,8 +1707,7 @@ __device__ __forceinline__ void assign_chain(const ChainArgs& a, int64_t smem_by
         blk_logq[k] = 0ull;
         spi[k] = a.logpi[k];
     }
-    for (int i = threadIdx.x; i < nw * K; i += blockDim.x) wsq[i] = 0ull;
-    for (int i = threadIdx.x; i < nw * 2 * K; i += blockDim.x) wn[i] = 0u;
+    for (int i = threadIdx.x; i < 2 * K; i += blockDim.x) bn[i] = 0u;
     // eq. 8 weights: log n-bar_{k,r} and log(n-bar_{k,r} - 1); log 0 = -inf
     for (int i = threadIdx.x; i < 2 * K; i += blockDim.x) {
         const float n = (float)a.nsub[i];
@@ -1665,46 +1721,47 @@ __device__ __forceinline__ void assign_chain(const ChainArgs& a, int64_t smem_by
     if (K <= 32 && bytes_c <= avail) {
         float* sLc = reinterpret_cast<float*>(rest);
         const bool sub_in = bytes_c + bytes_s <= avail;
-        float2* sLs = reinterpret_cast<float2*>(rest + bytes_c);
         // a chain with the blocked copy is counted by the tile statistics
         // kernel whichever engine labels it: no fused statistics then
         const bool fused = sub_in && !a.tile_enabled && bytes_c + bytes_s + bytes_st <= avail;
-        uint32_t* sS = fused ? reinterpret_cast<uint32_t*>(rest + bytes_c + bytes_s) : nullptr;
-        for (int64_t i = threadIdx.x; i < (int64_t)D * Kp; i += blockDim.x) {
-            const int64_t u = i / Kp, k = i - u * Kp;
-            sLc[i] = k < K ? __ldg(a.Lc + u * a.kmax + k) : 0.0f;
+        uint32_t* sS = fused ? reinterpret_cast<uint32_t*>(rest + bytes_c) : nullptr;
+        float2* sLs = reinterpret_cast<float2*>(rest + bytes_c + (fused ? bytes_st : 0));
+        // (32-bit indexes: the tables fit shared memory)
+        const int nthr = (int)blockDim.x;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < D * Kp; i += nthr) {
+            const int u = i / Kp, k = i - u * Kp;
+            sLc[i] = k < K ? __ldg(a.Lc + (size_t)u * a.kmax + k) : 0.0f;
         }
         if (sub_in)
-            for (int64_t i = threadIdx.x; i < (int64_t)D * K; i += blockDim.x) {
-                const int64_t u = i / K, k = i - u * K;
-                sLs[i] = __ldg(reinterpret_cast<const float2*>(a.Ls) + u * a.kmax + k);
+#pragma unroll 4
+            for (int i = threadIdx.x; i < D * K; i += nthr) {
+                const int u = i / K, k = i - u * K;
+                sLs[i] = __ldg(reinterpret_cast<const float2*>(a.Ls) + (size_t)u * a.kmax + k);
             }
         if (fused)
-            for (int64_t i = threadIdx.x; i < (int64_t)2 * K * D; i += blockDim.x) sS[i] = 0u;
+            for (int i = threadIdx.x; i < 2 * K * D; i += nthr) sS[i] = 0u;
         if (blockIdx.x == 0 && threadIdx.x == 0) a.sc->stats_fused = fused ? 1 : 0;
         __syncthreads();
         const float2* Ls2 = sub_in ? sLs : reinterpret_cast<const float2*>(a.Ls);
         const int ldS = sub_in ? K : a.kmax;
-        if (K <= 4) assign_cells_v2<4>(a, sLc, Kp, Ls2, ldS, K, t, spi, slw, wsq, wn, sS);
-        else if (K <= 8) assign_cells_v2<8>(a, sLc, Kp, Ls2, ldS, K, t, spi, slw, wsq, wn, sS);
-        else if (K <= 16) assign_cells_v2<16>(a, sLc, Kp, Ls2, ldS, K, t, spi, slw, wsq, wn, sS);
-        else assign_cells_v2<32>(a, sLc, Kp, Ls2, ldS, K, t, spi, slw, wsq, wn, sS);
+        const bool pk = a.csr.entries != nullptr;
+#define DPMM_HELD(L)                                                                         \
+    (pk ? assign_held<L, true>(a, sLc, Kp, Ls2, ldS, K, t, spi, slw, blk_logq, bn, sS)       \
+        : assign_held<L, false>(a, sLc, Kp, Ls2, ldS, K, t, spi, slw, blk_logq, bn, sS))
+        if (K <= 4) DPMM_HELD(1);
+        else if (K <= 8) DPMM_HELD(2);
+        else if (K <= 16) DPMM_HELD(4);
+        else DPMM_HELD(8);
+#undef DPMM_HELD
         __syncthreads();
         if (fused) {
-            for (int64_t i = threadIdx.x; i < (int64_t)2 * K * D; i += blockDim.x) {
+            for (int i = threadIdx.x; i < 2 * K * D; i += nthr) {
                 const uint32_t v = sS[i];
                 if (v) atomicAdd(&a.acc_Ssub[i], v);
             }
-            for (int i = threadIdx.x; i < 2 * K; i += blockDim.x) {
-                uint32_t v = 0;
-                for (int w = 0; w < nw; ++w) v += wn[w * 2 * K + i];
-                if (v) atomicAdd(&a.acc_nsub[i], v);
-            }
-        }
-        for (int k = threadIdx.x; k < K; k += blockDim.x) {
-            unsigned long long v = 0ull;
-            for (int w = 0; w < nw; ++w) v += wsq[w * K + k];
-            blk_logq[k] = v;
+            for (int i = threadIdx.x; i < 2 * K; i += nthr)
+                if (bn[i]) atomicAdd(&a.acc_nsub[i], bn[i]);
         }
     } else {
         float* slab = reinterpret_cast<float*>(rest);

@@ -1,8 +1,9 @@
-"""CSR label kernel with the cluster table in slabs (K > 32, or tables beyond
+"""CSR label kernel.  With the cluster table in slabs (K > 32, or tables beyond
 shared memory): slab widths from one to sixteen float4s, several slabs, odd
 kmax (no 16-byte table rows), unpacked counts, rows around the pieces a warp
-holds, fewer cells than blocks, tables that fit not even one slab; every label
-and sub-label against the FP64 decision."""
+holds, fewer cells than blocks, tables that fit not even one slab.  With the
+tables held (K <= 32): the edges of each number of lanes an entry, rows past the
+registers.  Every label and sub-label against the FP64 decision."""
 
 import numpy as np
 import pytest
@@ -31,6 +32,20 @@ def P():
     (700, 12000, 7, 16, 100, 0),      # K <= 32 with a table beyond shared memory
     (400, 16000, 40, 64, 100, 0),     # no slab fits: from global memory
     (900, 1000, 64, 64, 300, 70000),  # unpacked entries
+    # K <= 32 with the tables in shared memory: one to eight lanes an entry
+    (900, 333, 1, 1, 300, 0),
+    (900, 333, 4, 5, 257, 0),
+    (900, 333, 5, 7, 300, 0),
+    (900, 333, 8, 8, 256, 0),
+    (900, 333, 9, 33, 300, 0),
+    (120, 333, 16, 16, 300, 0),       # fewer cells than blocks
+    (900, 333, 17, 19, 300, 0),
+    (900, 1000, 32, 32, 300, 0),      # the sub-cluster table stays in global memory
+    (900, 333, 3, 4, 300, 70000),     # unpacked entries
+    (900, 333, 7, 8, 300, 70000),
+    (900, 333, 13, 16, 300, 70000),
+    (900, 333, 27, 32, 300, 70000),
+    (160000, 50, 6, 8, 33, 0),        # more than 1,024 cells a block
 ])
 def test_labels_match_fp64(P, N, D, K, kmax, longest, big):
     from scipy.sparse import csr_matrix

@@ -84,8 +84,9 @@ void dpmm_default_opts(dpmm_opts* opts);
  *   data    int32[nnz], counts >= 0
  * alpha > 0 (DP concentration), beta > 0 (eq. 28 lambda).  opts may be NULL.
  * stream: a cudaStream_t to run on, or NULL for a stream owned by the context.
- * The three arrays may be host or device memory: they are copied once on the
- * context's stream (device arrays must be complete before the call), then
+ * The three arrays may be host or device memory: host arrays are copied once on
+ * the context's stream, arrays of the context's own device are read in place
+ * (they must be complete before the call and are not needed after it).  They are
  * validated and turned into the packed and blocked copies on the device.
  * The chain starts with K = 1 (all cells in cluster 0) and fair-coin
  * sub-labels.  Errors: DPMM_EINVAL (malformed CSR, D < 1, N < 1, alpha or

@@ -193,7 +193,7 @@ struct Ctx {
     int32_t tile_Lmean = 0;         // mean padded segment, entries (rounded up)
     uint32_t* tile_ent = nullptr;   // row << 22 | gene-in-chunk << 16 | count (0: padding)
     int32_t* tile_ptr = nullptr;    // [4 T C + 1] quarter starts
-    unsigned char* tile_B = nullptr;  // per-sweep BF16 hi/lo table, [C][256 rows][64] swizzled
+    unsigned char* tile_B = nullptr;  // per-sweep FP16 or BF16 hi/lo table, [C][256 rows][64] swizzled
     float* noise = nullptr;         // [kTileMaxK + 2][N] the sweep's label noise (tile engine)
     int64_t tile_sumT = 0;          // tiles over the chains this context walks
     // launch tuning (dpmm_set_tuning; 0 = the built-in default).  None of these

@@ -1498,7 +1498,7 @@ __device__ __forceinline__ void assign_held(const ChainArgs& a, const float* sLc
 // traffic: 4 bytes an entry and cluster.  (Lanes that own clusters and take the
 // entries one by one read the same bytes but spend eight instructions an entry,
 // and with a table beyond shared memory read it from the L2, 256 bytes an entry
-// at K = 64: 30,011 x 1,000 cells 298 us, 113 us in slabs.)
+// at K = 64: 30,011 x 1,000 cells 298 us, 121 us in slabs.)
 //
 // The block's cells [N b / G, N (b + 1) / G) are taken in batches of at most
 // 1,024, 32 a warp: lane i keeps cell i's row bounds, running Gumbel-max and

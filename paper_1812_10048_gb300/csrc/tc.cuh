@@ -1,6 +1,6 @@
 // Blackwell (sm_103a) tensor-core primitives used by the dense-tile engine:
 // shared-memory matrix descriptors in the 128-byte-swizzled K-major layout,
-// tcgen05.mma (kind::f16, BF16 operands, FP32 accumulators in tensor memory),
+// tcgen05.mma (kind::f16, FP16 or BF16 operands, FP32 accumulators in tensor memory),
 // tensor-memory allocation and loads, bounded mbarrier waits and the 1-D bulk
 // copy engine.  Inline PTX only.
 #pragma once

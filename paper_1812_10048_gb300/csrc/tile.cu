@@ -744,6 +744,9 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                 // slot's first use the parity of the phase before the first)
                 bool ok = (uint32_t)lane >= n || tc::mbar_wait(&ent_free[es], eph ^ 1u, kWaitLimit);
                 ok = __all_sync(0xFFFFFFFFu, ok && *err == 0);
+                // a lane's copy may land where the item of another lane's slot lay: each
+                // lane takes over what the others have seen consumed
+                __syncwarp();
                 if (fixed) {
                     if (ok && (uint32_t)lane < n) issue((int32_t)(es * (uint32_t)e_max));
                 } else {
@@ -929,6 +932,10 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                         if (lane > 3) idx = st, ph = sph;
                     }
                     go = tc::mbar_wait_warp(ring + idx, ph, kWaitLimit);
+                    // each of lanes 0 - 3 has seen one of the round's barriers complete:
+                    // the lane that issues takes over what all four have seen
+                    __syncwarp();
+                    tc::fence_after_sync();
                     if (!go) break;
                     const int hq = planes && lane < 2
                                        ? reinterpret_cast<volatile int32_t*>(stage_hi)[idx]
@@ -970,6 +977,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                                 go = tc::mbar_wait_warp(&hi_full[hs],
                                                         ((uint32_t)(h - 1) / kHiStages) & 1u,
                                                         kWaitLimit);
+                                tc::fence_after_sync();
                                 if (go && tc::elect_one()) {
                                     four(ax, hlo + hs * (kStageBytes >> 4), blo + bx * bstep,
                                          idesc, 1u);

@@ -70,6 +70,31 @@ def test_fp16_scores(P, N, D, K):
     check_scores(P, X, K, logtheta, 2.0 ** -21)
 
 
+@pytest.mark.parametrize("N,D,K,deep", [(38989, 330, 10, 0), (38989, 330, 40, 0),
+                                        (38989, 330, 10, 300), (20001, 650, 40, 200)])
+def test_scores_repeat_bit_for_bit(P, N, D, K, deep):
+    """Every hand-over between the label kernel's roles is ordered (entries -> A stage
+    -> MMA -> epilogue, and each buffer back): a stage read before it is complete or
+    refilled while it is read shows as another score.  The same call ten times, with
+    segments in fixed slots and, where some cells are many times as deep as the
+    others, end to end in the ring."""
+    rng = np.random.default_rng([N, K, deep])
+    X = sparse(N, D, 40.0 / D, rng)
+    if deep:
+        from scipy.sparse import csr_matrix, vstack
+        full = csr_matrix(rng.integers(1, 200, size=(deep, D)).astype(np.float64))
+        X = vstack([X[:N - deep], full], format="csr")[rng.permutation(N)]
+    g = P.Sampler(X.indptr.astype(np.int32), X.indices.astype(np.int32), X.data.astype(np.int32),
+                  N, D, 1.0, 0.5, kmax=64, seed=3, engine=P.ENGINE_TILE_BF16)
+    g.set_state(np.arange(N) % K, np.zeros(N, np.uint8), K)
+    logtheta = np.log(rng.dirichlet(np.full(D, 0.3), size=3 * K) + 1e-30)
+    P.dpmm_set_params(g.ctx, np.full(K + 1, -np.log(K + 1.0)), logtheta)
+    first = P.dpmm_debug_tile_scores(g.ctx, N, K)
+    for _ in range(9):
+        np.testing.assert_array_equal(P.dpmm_debug_tile_scores(g.ctx, N, K), first)
+    g.close()
+
+
 @pytest.mark.parametrize("N,D,K,big", [(300, 200, 5, 40), (38989, 130, 10, 3000),
                                        (2000, 500, 40, 20000)])
 def test_second_planes(P, N, D, K, big):

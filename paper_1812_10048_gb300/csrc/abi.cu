@@ -183,10 +183,6 @@ ChainArgs dpmm::chain_args(const Ctx& c) {
     const double density = (c.N > 0 && c.D > 0) ? (double)c.nnz / ((double)c.N * c.D) : 0.0;
     a.tile_kmin = (c.opts.engine == DPMM_ENGINE_AUTO && density >= kTileDenseCut) ? kTileDenseKmin
                                                                                    : 1;
-    // The smallest log theta a draw can give: log G of a Gamma(a < 1) variate is
-    // above log(2^-24) / a - 51 (the boost and the cube of Marsaglia-Tsang at the
-    // smallest uniforms), less log of the total (below 32); FP16 ends at 65,504.
-    a.wide_beta = 16.64 / std::min(1.0, c.beta) + 100.0 > 60000.0;
     a.max_count = c.max_count;
     a.tile_ent = c.tile_ent;
     a.tile_ptr = c.tile_ptr;
@@ -1059,13 +1055,6 @@ int dpmm_set_params(dpmm_ctx* ctx, const float* logpi, const float* logtheta) {
     std::vector<float> lt, lp;
     if ((rc = fetch(lp, logpi, (size_t)K + 1))) return rc;
     if ((rc = fetch(lt, logtheta, 3 * (size_t)K * c.D))) return rc;
-    // values beyond +-30,000 (their centred differences could pass FP16's 65,504)
-    // and those that are not finite: BF16 operands in the dense-tile engine
-    int32_t wide = 0;
-    for (const float v : lt) wide |= !(std::fabs(v) <= 30000.0f);
-    c.sc_host->wide_params = wide;
-    CK(cudaMemcpy(&c.sc->wide_params, &c.sc_host->wide_params, sizeof(int32_t),
-                  cudaMemcpyHostToDevice));
     std::vector<float> lc((size_t)c.kmax * c.D, 0.0f), ls(2 * (size_t)c.kmax * c.D, 0.0f);
     for (int k = 0; k < K; ++k)
         for (int u = 0; u < c.D; ++u) {

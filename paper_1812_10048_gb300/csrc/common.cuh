@@ -84,9 +84,6 @@ struct DevScalars {
     uint32_t n_apply;     // plans applied so far (sweep compactions and moves)
     int32_t inst_fresh;   // the last plan was a sweep's compaction: the sweep's
                           // pi / theta draws (pre-compaction rows) serve eq. 18
-    int32_t wide_params;  // some log theta may lie beyond FP16's range (set by the draws
-                          // from beta, by dpmm_set_params from the values): the
-                          // dense-tile engine then takes BF16 operands
     int32_t open_slot;    // cluster K - 1 is the eq. 4 K+1 candidate appended for
                           // this sweep (no cells yet; cleared by every plan)
 };
@@ -99,13 +96,15 @@ constexpr int kTileMaxK = 40;
 // density; at K <= 2 and density >= kTileDenseCut the CSR engine is (up to 10%)
 // faster.  So the automatic choice takes the tile engine for K >= 3 always and
 // for K <= 2 only below that density.
-// Segment table of the blocked copy: bit 31 of a segment's quarter-1 pointer: it
-// has a count above 2,047 (a second plane in FP16); of its quarter-2 pointer: a
-// count above 255 (a second plane in BF16).
-constexpr int32_t kTilePtrMask = 0x7FFFFFFF;
-constexpr uint32_t kTileFlag = 0x80000000u;
 constexpr double kTileDenseCut = 0.12;
 constexpr int kTileDenseKmin = 3;
+
+// Segment table of the blocked copy: bit 31 of a segment's quarter-1 pointer: it
+// has a count above 255, which takes a second plane (two digits of BF16's eight
+// significant bits).
+constexpr int32_t kTilePtrMask = 0x7FFFFFFF;
+constexpr uint32_t kTileFlag = 0x80000000u;
+constexpr int32_t kTileLoMax = 255;
 
 // ---------------------------------------------------------------------------
 // The context (owned by the C ABI layer).
@@ -193,7 +192,7 @@ struct Ctx {
     int32_t tile_Lmean = 0;         // mean padded segment, entries (rounded up)
     uint32_t* tile_ent = nullptr;   // row << 22 | gene-in-chunk << 16 | count (0: padding)
     int32_t* tile_ptr = nullptr;    // [4 T C + 1] quarter starts
-    unsigned char* tile_B = nullptr;  // per-sweep FP16 or BF16 hi/lo table, [C][256 rows][64] swizzled
+    unsigned char* tile_B = nullptr;  // per-sweep BF16 hi/lo table, [C][256 rows][64] swizzled
     float* noise = nullptr;         // [kTileMaxK + 2][N] the sweep's label noise (tile engine)
     int64_t tile_sumT = 0;          // tiles over the chains this context walks
     // launch tuning (dpmm_set_tuning; 0 = the built-in default).  None of these
@@ -402,7 +401,6 @@ struct ChainArgs {
     int32_t tile_enabled, tile_C, tile_T, tile_Lslot, tile_Lmean;
     int32_t tile_kmin;    // smallest K the dense-tile engine labels (engine choice)
     int32_t max_count;    // largest count of the matrix
-    int32_t wide_beta;    // drawn log theta values may lie beyond FP16's range
     uint32_t* tile_ent;
     int32_t* tile_ptr;
     float* noise;

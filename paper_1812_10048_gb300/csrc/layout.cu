@@ -121,8 +121,8 @@ __global__ void k_check_colsum(const unsigned long long* __restrict__ colsum, in
 // Block (tile, quarter): its 32 rows, a warp each.  COUNT: bucket sizes into
 // qcount[4 (t C + chunk) + q].  Otherwise each entry is written to its
 // bucket's start + its stable rank in the bucket, the segment's padding is
-// cleared, and counts beyond the label kernel's lo digits set the segment's
-// flags in qptr.  (One warp for all 32 rows left a chain of dependent loads 32
+// cleared, and a count beyond the label kernel's lo digit sets the segment's
+// flag in qptr.  (One warp for all 32 rows left a chain of dependent loads 32
 // rows long: 68,000 x 1,000 88 + 101 us, 30 + 51 us with a warp a row.)
 constexpr int kBucketThreads = 1024;
 
@@ -186,8 +186,7 @@ k_tile_bucket(const int32_t* __restrict__ indptr, const uint32_t* __restrict__ e
             if (rank == 0) cnt[chunk] = at + __popc(peers);
             tent[at] = ((uint32_t)(32 * q + w) << 22) | (((e >> 16) & 63u) << 16) | (e & 0xFFFFu);
             uint32_t* flags = reinterpret_cast<uint32_t*>(qptr) + 4 * (t * C + chunk);
-            if ((e & 0xFFFFu) > 255u) atomicOr(flags + 2, kTileFlag);
-            if ((e & 0xFFFFu) > 2047u) atomicOr(flags + 1, kTileFlag);
+            if ((e & 0xFFFFu) > (uint32_t)kTileLoMax) atomicOr(flags + 1, kTileFlag);
         }
         __syncwarp();
     }

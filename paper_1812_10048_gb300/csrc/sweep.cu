@@ -283,10 +283,7 @@ k_draw_params(const __grid_constant__ Tab tab) {
     const int nblk = (int)gridDim.x / CS;
     auto first_row = [&](const ChainArgs& ch, int K) {
         if (rank) return;
-        if (threadIdx.x == 0) {
-            select_engine(ch.sc, K, ch);
-            ch.sc->wide_params = ch.wide_beta;
-        }
+        if (threadIdx.x == 0) select_engine(ch.sc, K, ch);
         clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
     };
     if (n > 1 && n <= kDrawTable) {

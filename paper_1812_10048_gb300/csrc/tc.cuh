@@ -1,6 +1,6 @@
 // Blackwell (sm_103a) tensor-core primitives used by the dense-tile engine:
 // shared-memory matrix descriptors in the 128-byte-swizzled K-major layout,
-// tcgen05.mma (kind::f16, FP16 or BF16 operands, FP32 accumulators in tensor memory),
+// tcgen05.mma (kind::f16, BF16 operands, FP32 accumulators in tensor memory),
 // tensor-memory allocation and loads, bounded mbarrier waits and the 1-D bulk
 // copy engine.  Inline PTX only.
 #pragma once
@@ -35,11 +35,6 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
 // N >> 3 in bits 17-22, M >> 4 in bits 24-28.
 __host__ __device__ __forceinline__ uint32_t idesc_bf16(uint32_t M, uint32_t N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
-}
-
-// The same with FP16 A and B (bits 7-9 = 0, 10-12 = 0).
-__host__ __device__ __forceinline__ uint32_t idesc_f16(uint32_t M, uint32_t N) {
-    return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
 // ---- mbarriers --------------------------------------------------------------
@@ -156,9 +151,8 @@ __device__ __forceinline__ void fence_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, one M x N x 16 step (FP16 or BF16 operands,
-// as the instruction descriptor says).
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+// D[tmem] (+)= A[smem] * B[smem]^T, one M x N x 16 step.
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                          uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"

@@ -4,7 +4,6 @@
 // layout, descriptors and tensor-memory path: C[128][N] = A[128][Kd] B[N][Kd]^T
 // for BF16 operands with FP32 accumulation, one CTA.
 #include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include <math_constants.h>
 
 #include "common.cuh"
@@ -57,7 +56,7 @@ k_debug_tc_gemm(const uint16_t* __restrict__ A, const uint16_t* __restrict__ B, 
                 const uint64_t ad = tc::desc_sw128(tc::smem_addr(sA + ch * 16384) + 32 * k);
                 const uint64_t bd =
                     tc::desc_sw128(tc::smem_addr(sB + (size_t)ch * N * 128) + 32 * k);
-                tc::mma_f16(taddr, ad, bd, idesc, (ch | k) != 0);
+                tc::mma_bf16(taddr, ad, bd, idesc, (ch | k) != 0);
             }
         tc::mma_commit(bar);
     }
@@ -97,13 +96,12 @@ cudaError_t launch_debug_tc_gemm(const uint16_t* A, const uint16_t* B, int Kd, i
 // Dense-tile label engine (eq. 4 third line and eq. 8 on the tensor cores).
 //
 // Tiles of 128 consecutive cells, 64-gene chunks.  Per (tile, chunk) item the
-// CTA zeroes a 128 x 64 16-bit operand in shared memory (128-byte swizzled
-// K-major layout) and scatters the counts into it; counts beyond the format's
-// exact integers (2,047 in FP16, 255 in BF16) are split into two exact digits,
-// the second of which goes through the same stage as another plane, only for
-// items that have such counts (flagged when the blocked copy is built).  The B
-// operand (bulk-copied per chunk) holds the centred log theta table split into
-// hi + lo parts of the same format, so that one M=128 MMA per 16 genes
+// CTA zeroes a 128 x 64 BF16 operand in shared memory (128-byte swizzled
+// K-major layout) and scatters the counts into it; counts above 255 are split
+// into two exact digits, the second of which goes through another stage as a
+// second plane, only for items that have such counts (flagged when the blocked
+// copy is built).  The B operand (bulk-copied per chunk) holds the centred log
+// theta table split into BF16 hi + lo parts, so that one M=128 MMA per 16 genes
 // accumulates, in FP32 tensor memory, every cluster and sub-cluster score of
 // the 128 cells:
 //   TMEM / B column 2k, 2k+1            cluster k, hi and lo part
@@ -128,17 +126,12 @@ __host__ __device__ __forceinline__ bool tile_usable(int K) {
 __host__ __device__ __forceinline__ int tile_s0(int K) { return (2 * K + 15) & ~15; }
 __host__ __device__ __forceinline__ int tile_ntot(int K) { return (tile_s0(K) + 4 * K + 15) & ~15; }
 
-// Operand format of a chain's contraction: FP16 (11 significant bits: log theta
-// as hi + lo to 2^-22, counts to 2,047 in one plane) unless a log theta may lie
-// beyond FP16's range, then BF16 (to 2^-16, counts to 255 in one plane).
-__device__ __forceinline__ bool chain_half(const ChainArgs& ch) { return !ch.sc->wide_params; }
-
-__device__ __forceinline__ uint16_t f16_bits_rn(float f) {
-    return __half_as_ushort(__float2half_rn(f));
-}
-__device__ __forceinline__ float f16_value(uint16_t b) {
-    return __half2float(__ushort_as_half(b));
-}
+// BF16 takes every log theta that a draw or a caller can give (FP16 ends at
+// 65,504, which drawn values pass from beta = 2.8e-4 down), and its coarse hi
+// part leaves the FP32 accumulator's additions nearly exact where few clusters
+// meet many counts: own-cluster scores of 4,000 cells x 3,000 genes, K = 3,
+// libraries of 3,000, differ from 64 bits by 3.8e-3 rms, with FP16 hi + lo by
+// 1.3e-2.
 __device__ __forceinline__ uint16_t bf16_bits_rn(float f) {
     const __nv_bfloat16 h = __float2bfloat16_rn(f);
     return *reinterpret_cast<const uint16_t*>(&h);
@@ -215,7 +208,6 @@ k_build_b(const __grid_constant__ Tab tab, int32_t force, int32_t rb) {
         __syncthreads();
     }
     unsigned char* dst = B + (size_t)c * kBChunkBytes;
-    const bool half = chain_half(ch);
     for (int i = blockIdx.y * rb * 64 + threadIdx.x; i < min(Ntot, (int)(blockIdx.y + 1) * rb) * 64;
          i += blockDim.x) {
         const int row = i >> 6, g = i & 63, u = c * 64 + g;
@@ -235,13 +227,8 @@ k_build_b(const __grid_constant__ Tab tab, int32_t force, int32_t rb) {
         uint16_t v = 0;
         if (live) {
             const float d = L - m[g];
-            if (half) {
-                const uint16_t hi = f16_bits_rn(d);
-                v = part ? f16_bits_rn(d - f16_value(hi)) : hi;
-            } else {
-                const uint16_t hi = bf16_bits_rn(d);
-                v = part ? bf16_bits_rn(d - bf16_value(hi)) : hi;
-            }
+            const uint16_t hi = bf16_bits_rn(d);
+            v = part ? bf16_bits_rn(d - bf16_value(hi)) : hi;
         }
         *reinterpret_cast<uint16_t*>(dst + tc::swz_offset((uint32_t)row, (uint32_t)g)) = v;
     }
@@ -314,16 +301,11 @@ constexpr int kEpiGroups = (kTileMaxK + 15) / 16;   // 8-cluster groups of a hal
 constexpr int kSmallBytes = 8192;
 constexpr int kScatterDefault = 12;  // entries per producer lane and batch (tunable: 8, 12, 16)
 
-// The digits of a count in the operand format: lo and hi with lo + hi = x, each
-// exact in 16 bits (FP16: 11 significant bits, x = (x & 2047) + (x & 0xF800);
-// BF16: 8, x = (x & 255) + (x & 0xFF00), whose FP32 patterns truncate exactly).
-template <bool kHalf>
+// A digit of a count, x & 255 or x & 0xFF00: at most eight significant bits, so
+// that its FP32 pattern truncates exactly to BF16.
 __device__ __forceinline__ uint16_t digit_bits(uint32_t v) {
-    if (kHalf) return __half_as_ushort(__ushort2half_rn((unsigned short)v));
     return (uint16_t)(__float_as_uint((float)v) >> 16);
 }
-template <bool kHalf>
-__device__ __forceinline__ constexpr uint32_t lo_mask() { return kHalf ? 0x7FFu : 0xFFu; }
 
 // One producer warp's share of a staged segment into its quarter q of the A stage
 // (kHi: the hi digits, else the lo ones): the 16-byte groups that hold entries
@@ -332,10 +314,10 @@ __device__ __forceinline__ constexpr uint32_t lo_mask() { return kHalf ? 0x7FFu 
 // segment's padding, whose counts are 0.  An entry row << 22 | gene << 16 | count
 // shifted right by 15 has its row and gene at the bytes row * 128 + gene * 2 of
 // the stage; the 128-byte swizzle exchanges bits 4-6 with the row's low bits.
-template <bool kHalf, bool kHi, int kScatter>
+template <bool kHi, int kScatter>
 __device__ __forceinline__ void scatter_entries(const uint32_t* ring, int i0, int i1, int q,
                                                 int lane, unsigned char* A) {
-    constexpr uint32_t mask = kHi ? 0xFFFFu & ~lo_mask<kHalf>() : lo_mask<kHalf>();
+    constexpr uint32_t mask = kHi ? 0xFF00u : 0xFFu;
     constexpr int U = kScatter / 4;
     const uint4* ring4 = reinterpret_cast<const uint4*>(ring);
     const int j1 = (i1 + 3) >> 2;
@@ -352,7 +334,7 @@ __device__ __forceinline__ void scatter_entries(const uint32_t* ring, int i0, in
                 const uint32_t x = e[k] & mask, t = e[k] >> 15;
                 if (x && (e[k] >> 27) == (uint32_t)q)
                     *reinterpret_cast<uint16_t*>(A + ((t & 0x3FFEu) ^ ((t >> 3) & 0x70u))) =
-                        digit_bits<kHalf>(x);
+                        digit_bits(x);
             }
         }
     }
@@ -369,10 +351,9 @@ __device__ __forceinline__ void clear_quarter(unsigned char* A, int q, int lane)
 // A chain's tiles for one CTA: first, first + gridDim.x, ... (cnt of them).
 struct TileJob {
     int32_t b, first, cnt;
-    uint32_t k;      // K | FP16 operands << 16 | second planes << 17
+    uint32_t k;      // K | second planes << 16
     __device__ __forceinline__ int K() const { return (int)(k & 0xFFFFu); }
-    __device__ __forceinline__ bool half() const { return (k >> 16) & 1u; }
-    __device__ __forceinline__ bool planes() const { return (k >> 17) & 1u; }
+    __device__ __forceinline__ bool planes() const { return (k >> 16) & 1u; }
 };
 
 // The jobs of this CTA in chain order (called by the whole block; jobs and
@@ -386,10 +367,9 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
                                           int32_t* scratch) {
     if (tab.n() == 1) {     // one chain: every thread by itself
         const ChainArgs& ch = tab[0];
-        const int K = ch.sc->K, used = ch.sc->tile_used, wide = ch.sc->wide_params;
+        const int K = ch.sc->K, used = ch.sc->tile_used;
         if (!ch.tile_enabled || !tile_usable(K) || !(dbg || used)) return;
-        TileJob job{0, 0, 0, (uint32_t)K | (wide ? 0u : 1u << 16) |
-                                 (ch.max_count > (wide ? 255 : 2047) ? 1u << 17 : 0u)};
+        TileJob job{0, 0, 0, (uint32_t)K | (ch.max_count > kTileLoMax ? 1u << 16 : 0u)};
         chain_tiles(0, ch.tile_T, job.first, job.cnt);
         if (!job.cnt) return;
         if (threadIdx.x == 0) jobs[0] = job;
@@ -413,13 +393,12 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
         if (b < tab.n()) {
             const ChainArgs& ch = tab[b];
             const bool enabled = ch.tile_enabled;
-            const int K = ch.sc->K, used = ch.sc->tile_used, wide = ch.sc->wide_params;
+            const int K = ch.sc->K, used = ch.sc->tile_used;
             if (enabled && tile_usable(K) && (dbg || used)) {
                 T = ch.tile_T;
                 lslot = ch.tile_Lslot;
                 lmean = ch.tile_Lmean;
-                k = (uint32_t)K | (wide ? 0u : 1u << 16) |
-                    (ch.max_count > (wide ? 255 : 2047) ? 1u << 17 : 0u);
+                k = (uint32_t)K | (ch.max_count > kTileLoMax ? 1u << 16 : 0u);
             }
         }
         int x = T;
@@ -451,7 +430,7 @@ __device__ __forceinline__ void list_jobs(const Tab& tab, bool dbg, TileJob* job
             atomicMax(&smax[1], tile_ntot((int)(k & 0xFFFFu)));
             atomicMax(&smax[2], lslot);
             atomicMax(&smax[4], lmean);
-            if (k >> 17) smax[3] = 1;
+            if (k >> 16) smax[3] = 1;
             smax[5] = tab[b].tile_C;     // (the chains share D)
         }
         __syncthreads();
@@ -615,15 +594,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         uint32_t st = (uint32_t)set % (uint32_t)nS, sph = 1u;   // parity of the stage's last use
         uint32_t es = (uint32_t)set % (uint32_t)nE, eph = 0u;
         uint32_t g = set < nsets ? (uint32_t)set : total;
-        uint32_t gend = 0;        // items before the end of the current chain
-        int jb = -1;
-        bool half = false;
         for (; g < total; g += (uint32_t)nsets) {
-            while (g >= gend) {   // the chain of item g: its operand format
-                const TileJob job = jobs[++jb];
-                gend += (uint32_t)job.cnt * (uint32_t)C;
-                half = job.half();
-            }
             unsigned char* A = A_base + st * kStageBytes;
             // (at a stage's first use the parity of the phase before the first)
             bool ok = tc::mbar_wait(&stage_free[st], sph, kWaitLimit);
@@ -640,8 +611,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             const int i1 = q == 0 ? mt.x : q == 1 ? mt.y : q == 2 ? mt.z : mt.w;
             const int hi = planes_any ? meta_hi[es] : 0;    // 0, or 1 + its number
             const uint32_t* ring = reinterpret_cast<const uint32_t*>(E_base + slot_off[es]);
-            if (half) scatter_entries<true, false, kScatter>(ring, i0, i1, q, lane, A);
-            else scatter_entries<false, false, kScatter>(ring, i0, i1, q, lane, A);
+            scatter_entries<false, kScatter>(ring, i0, i1, q, lane, A);
             tc::fence_async_smem();
             __syncwarp();
             if (lane == 0) {
@@ -665,8 +635,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                 }
                 unsigned char* H = H_base + hs * kStageBytes;
                 clear_quarter(H, q, lane);
-                if (half) scatter_entries<true, true, kScatter>(ring, i0, i1, q, lane, H);
-                else scatter_entries<false, true, kScatter>(ring, i0, i1, q, lane, H);
+                scatter_entries<true, kScatter>(ring, i0, i1, q, lane, H);
                 tc::fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
@@ -698,7 +667,6 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             const int first = job.first, cnt = job.cnt;
             const uint32_t Cu = (uint32_t)C;
             const uint32_t nitem = (uint32_t)cnt * Cu;
-            const bool half = job.half();
             // lane l < nsets takes the items l, l + nsets, ...: their five
             // quarter pointers, read one round ahead
             auto seg_ptrs = [&](uint32_t j, int32_t (&p)[6]) {
@@ -714,9 +682,8 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
 #pragma unroll
                     for (int k = 0; k < 5; ++k) p[k] = __ldg(ch.tile_ptr + 4 * sgm + k);
                     // the segment's second-plane flag, then the pointers
-                    p[5] = half ? p[1] < 0 : p[2] < 0;
+                    p[5] = p[1] < 0;
                     p[1] &= kTilePtrMask;
-                    p[2] &= kTilePtrMask;
                 }
             };
             int32_t cur[6], nxt[6];
@@ -874,17 +841,16 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         const uint32_t bstep = (uint32_t)(b_slot >> 4);
         auto four = [&](uint32_t acc, uint32_t a, uint32_t bb, uint32_t idesc, uint32_t accum) {
             const uint64_t ad = desc | a, bd = desc | bb;
-            tc::mma_f16(acc, ad, bd, idesc, accum);
+            tc::mma_bf16(acc, ad, bd, idesc, accum);
 #pragma unroll
-            for (int k = 1; k < 4; ++k) tc::mma_f16(acc, ad + 2 * k, bd + 2 * k, idesc, 1u);
+            for (int k = 1; k < 4; ++k) tc::mma_bf16(acc, ad + 2 * k, bd + 2 * k, idesc, 1u);
         };
         bool go = true;
         for (int jn = 0; jn < njobs && go; ++jn) {
             const TileJob job = jobs[jn];
             const int cnt = job.cnt;
             const uint32_t ntot = (uint32_t)tile_ntot(job.K());
-            const uint32_t idesc = job.half() ? tc::idesc_f16(128, ntot)
-                                              : tc::idesc_bf16(128, ntot);
+            const uint32_t idesc = tc::idesc_bf16(128, ntot);
             const bool planes = job.planes();
             for (int i = 0; i < cnt && go; i += kPair) {
                 const int m = min(kPair, cnt - i);

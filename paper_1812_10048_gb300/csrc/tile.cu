@@ -286,7 +286,6 @@ __device__ __forceinline__ void chain_tiles(int64_t off, int T, int& first, int&
 // it before the block exits.
 constexpr int kMaxStages = 8;        // A stages
 constexpr uint32_t kStageBytes = 16384;   // 128 cells x 64 genes x 2 bytes
-constexpr int kHiStages = 2;          // stages of the items' second planes
 constexpr int kMaxBStages = 4;
 constexpr int kMaxAcc = 4;
 constexpr int kPair = 2;             // tiles that share a chunk's B operand
@@ -480,8 +479,6 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     const int b_slot = (ntot_max * 128 + 1023) & ~1023;
     const int e_max = min(lslot_max, 1 << 20) * 4, e_mean = min(lmean_max, 1 << 20) * 4;
     const int avail = (int)(smem_bytes - (base - smem_raw)) - kSmallBytes;
-    // hi stages, only when some chain of the block has a second plane
-    const int h_bytes = planes_any ? kHiStages * (int)kStageBytes : 0;
     // Producer sets and A stages, the most that fit beside a segment ring for two
     // items of a set and the longest segment.  A set takes every nsets-th item
     // and always meets the same stages and slots, so nsets divides nS and nE:
@@ -489,7 +486,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // item g - nE, and a set's parity wait can never be two phases ahead.  Two
     // stages a set let it fill one while the MMAs read the other.
     auto ring_left = [&](int stages, int b_stages) {
-        return avail - stages * (int)kStageBytes - h_bytes - b_stages * b_slot;
+        return avail - stages * (int)kStageBytes - b_stages * b_slot;
     };
     auto fit = [&](int sets, int stages) {
         return ring_left(stages, 2) >= max(e_max, 2 * sets * e_mean);
@@ -520,8 +517,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     const uint32_t ldN = ((uint32_t)ntot_max + 31u) & ~31u;        // TMEM columns of a slot
     const uint32_t nAcc = min((uint32_t)kMaxAcc, 512u / ldN);      // >= 2
     unsigned char* A_base = base;
-    unsigned char* H_base = A_base + nS * kStageBytes;
-    unsigned char* B_base = H_base + h_bytes;
+    unsigned char* B_base = A_base + nS * kStageBytes;
     unsigned char* E_base = B_base + nB * b_slot;
     unsigned char* small = E_base + e_ring;
     small = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(small) + 15) & ~(uintptr_t)15);
@@ -530,9 +526,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     uint64_t* stage_free = a_full + kMaxStages;                     // [kMaxStages]
     uint64_t* b_full = stage_free + kMaxStages;                     // [kMaxBStages]
     uint64_t* b_free = b_full + kMaxBStages;                        // [kMaxBStages]
-    uint64_t* hi_full = b_free + kMaxBStages;                       // [kHiStages]
-    uint64_t* hi_used = hi_full + kHiStages;                        // [kHiStages]
-    uint64_t* ent_full = hi_used + kHiStages;                       // [kMaxESlots]
+    uint64_t* ent_full = b_free + kMaxBStages;                      // [kMaxESlots]
     uint64_t* ent_free = ent_full + kMaxESlots;                     // [kMaxESlots]
     uint64_t* acc_full = ent_free + kMaxESlots;                     // [kMaxAcc]
     uint64_t* acc_empty = acc_full + kMaxAcc;                       // [kMaxAcc]
@@ -543,8 +537,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     int32_t* stage_hi = stop + 2;                                   // [kMaxStages]
     int32_t* slot_off = stage_hi + kMaxStages;                      // [kMaxESlots] ring offsets
     int32_t* meta_hi = slot_off + kMaxESlots;                       // [kMaxESlots]
-    volatile int32_t* hi_done = meta_hi + kMaxESlots;               // second planes used up
-    float* spi = reinterpret_cast<float*>(meta_hi + kMaxESlots + 1);    // [K]
+    float* spi = reinterpret_cast<float*>(meta_hi + kMaxESlots);    // [K]
     float* slw = spi + kTileMaxK;                                   // [4K]
     float* xbest = slw + 4 * kTileMaxK;                             // [2][half][128]
     int* xc = reinterpret_cast<int*>(xbest + 512);                  // [2][half][128]
@@ -552,7 +545,6 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
 
     if (tid == 0) {
         *err = 0;
-        *hi_done = 0;
         stop[0] = stop[1] = 0;
         for (int i = 0; i < kMaxStages; ++i) {
             tc::mbar_init(&a_full[i], 4);   // four producer warps
@@ -561,10 +553,6 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         for (int i = 0; i < kMaxBStages; ++i) {
             tc::mbar_init(&b_full[i], 1);
             tc::mbar_init(&b_free[i], 1);
-        }
-        for (int i = 0; i < kHiStages; ++i) {
-            tc::mbar_init(&hi_full[i], 4);
-            tc::mbar_init(&hi_used[i], 1);
         }
         tc::mbar_init(drain, 1);
         for (int i = 0; i < kMaxESlots; ++i) {
@@ -594,58 +582,51 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         uint32_t st = (uint32_t)set % (uint32_t)nS, sph = 1u;   // parity of the stage's last use
         uint32_t es = (uint32_t)set % (uint32_t)nE, eph = 0u;
         uint32_t g = set < nsets ? (uint32_t)set : total;
-        for (; g < total; g += (uint32_t)nsets) {
-            unsigned char* A = A_base + st * kStageBytes;
-            // (at a stage's first use the parity of the phase before the first)
-            bool ok = tc::mbar_wait(&stage_free[st], sph, kWaitLimit);
-            if (__all_sync(0xFFFFFFFFu, ok)) {
-                clear_quarter(A, q, lane);      // while the segment is still on its way
-                ok = tc::mbar_wait(&ent_full[es], eph, kWaitLimit);
-            }
-            if (!__all_sync(0xFFFFFFFFu, ok && *err == 0)) {
-                if (lane == 0 && !ok) *err = DPMM_ETIMEOUT;
-                break;
-            }
-            const int4 mt = meta[es];
-            const int i0 = q == 0 ? 0 : q == 1 ? mt.x : q == 2 ? mt.y : mt.z;
-            const int i1 = q == 0 ? mt.x : q == 1 ? mt.y : q == 2 ? mt.z : mt.w;
-            const int hi = planes_any ? meta_hi[es] : 0;    // 0, or 1 + its number
-            const uint32_t* ring = reinterpret_cast<const uint32_t*>(E_base + slot_off[es]);
-            scatter_entries<false, kScatter>(ring, i0, i1, q, lane, A);
-            tc::fence_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-                if (planes_any && q == 0) stage_hi[st] = hi;
-                tc::mbar_arrive(&a_full[st]);
-                if (!hi) tc::mbar_arrive(&ent_free[es]);
-            }
-            if (hi) {
-                // its hi digits, in the block's order of second planes: the plane
-                // kHiStages before it has been used (a count, since this set may
-                // be more than one use of the stage ahead, which a phase's parity
-                // could not tell)
-                const uint32_t hs = (uint32_t)(hi - 1) % kHiStages;
-                ok = false;
-                for (uint32_t x = 0; x < kWaitLimit && !ok; ++x)
-                    ok = *hi_done + kHiStages >= hi;
-                __threadfence_block();
-                if (!__all_sync(0xFFFFFFFFu, ok)) {
-                    if (lane == 0) *err = DPMM_ETIMEOUT;
+        bool ok = true;
+        for (; g < total && ok; g += (uint32_t)nsets) {
+            int i0 = 0, i1 = 0, hi = 0;
+            const uint32_t* ring = nullptr;
+            // the item's plane of lo digits, then, if it has counts above 255, that of
+            // its hi digits in the set's next stage, a stage like any other: the MMA
+            // warp goes on to other items while it fills.  (Stages of its own that the
+            // MMA warp had to drain before they were used again: 68,000 x 1,000 step
+            // 96 -> 89 us, 1.3 M x 2,000 2,430 -> 2,260 us; both planes written in one
+            // pass over the entries 91 us.)
+            for (int pl = 0; pl <= hi; ++pl) {
+                unsigned char* A = A_base + st * kStageBytes;
+                // (at a stage's first use the parity of the phase before the first)
+                ok = tc::mbar_wait(&stage_free[st], sph, kWaitLimit);
+                if (__all_sync(0xFFFFFFFFu, ok)) {
+                    clear_quarter(A, q, lane);      // while the segment is still on its way
+                    if (!pl) ok = tc::mbar_wait(&ent_full[es], eph, kWaitLimit);
+                }
+                const bool mine = ok;
+                ok = __all_sync(0xFFFFFFFFu, ok && *err == 0);
+                if (!ok) {
+                    if (lane == 0 && !mine) *err = DPMM_ETIMEOUT;
                     break;
                 }
-                unsigned char* H = H_base + hs * kStageBytes;
-                clear_quarter(H, q, lane);
-                scatter_entries<true, kScatter>(ring, i0, i1, q, lane, H);
+                if (!pl) {
+                    const int4 mt = meta[es];
+                    i0 = q == 0 ? 0 : q == 1 ? mt.x : q == 2 ? mt.y : mt.z;
+                    i1 = q == 0 ? mt.x : q == 1 ? mt.y : q == 2 ? mt.z : mt.w;
+                    if (planes_any) hi = meta_hi[es];
+                    ring = reinterpret_cast<const uint32_t*>(E_base + slot_off[es]);
+                    scatter_entries<false, kScatter>(ring, i0, i1, q, lane, A);
+                } else {
+                    scatter_entries<true, kScatter>(ring, i0, i1, q, lane, A);
+                }
                 tc::fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tc::mbar_arrive(&hi_full[hs]);
-                    tc::mbar_arrive(&ent_free[es]);
+                    if (planes_any && q == 0 && !pl) stage_hi[st] = hi;
+                    tc::mbar_arrive(&a_full[st]);
+                    if (pl == hi) tc::mbar_arrive(&ent_free[es]);
                 }
-            }
-            if ((st += (uint32_t)nsets) >= (uint32_t)nS) {
-                st -= (uint32_t)nS;
-                sph ^= 1u;
+                if ((st += (uint32_t)nsets) >= (uint32_t)nS) {
+                    st -= (uint32_t)nS;
+                    sph ^= 1u;
+                }
             }
             if ((es += (uint32_t)nsets) >= (uint32_t)nE) {
                 es -= (uint32_t)nE;
@@ -655,11 +636,9 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     } else if (warp == kELoadWarp) {
         // ---------------- segment loader ----------------
         uint32_t g = 0;        // items started (slot sequence)
-        uint32_t hseq = 0;     // second planes started
         uint32_t es = (uint32_t)lane % (uint32_t)nE, eph = 0;   // this lane's slot, its use's parity
         uint32_t tail = 0;     // oldest item that may still be in the ring
         int32_t head = 0;      // the ring's next free byte (the items lie between)
-        const unsigned lanemask = (1u << lane) - 1u;
         bool stop_l = false;
         for (int jn = 0; jn < njobs && !stop_l; ++jn) {
             const TileJob job = jobs[jn];
@@ -691,14 +670,12 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             for (uint32_t jb = 0; jb < nitem; jb += (uint32_t)nsets) {
                 seg_ptrs(jb + (uint32_t)nsets + (uint32_t)lane, nxt);
                 const uint32_t n = min((uint32_t)nsets, nitem - jb);
-                const unsigned flagged = __ballot_sync(0xFFFFFFFFu, (uint32_t)lane < n && cur[5]);
                 const int32_t len = cur[4] - cur[0];
                 const int32_t room = (uint32_t)lane < n ? max(len, 4) * 4 : 0;   // ring bytes
                 auto issue = [&](int32_t at) {
                     slot_off[es] = at;
                     meta[es] = make_int4(cur[1] - cur[0], cur[2] - cur[0], cur[3] - cur[0], len);
-                    if (planes_any)
-                        meta_hi[es] = cur[5] ? 1 + (int)(hseq + __popc(flagged & lanemask)) : 0;
+                    if (planes_any) meta_hi[es] = cur[5];
                     if (len) {
                         tc::mbar_arrive_expect_tx(&ent_full[es], (uint32_t)len * 4u);
                         tc::bulk_g2s(E_base + at, ch.tile_ent + cur[0], (uint32_t)len * 4u,
@@ -776,7 +753,6 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                     eph ^= 1u;
                 }
                 g += n;
-                hseq += (uint32_t)__popc(flagged);
 #pragma unroll
                 for (int k = 0; k < 6; ++k) cur[k] = nxt[k];
             }
@@ -831,13 +807,21 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         // beside busy producers; the tensor core needs 257 at N = 128, 480 at
         // N = 240).  So the whole warp walks the items converged and an elected
         // lane issues (from a branch of one lane the same sequence took 282, its
-        // waits 270 - 500), and one wait serves two items: lanes 0 - 3 poll the
-        // barriers of two A stages and their B stages side by side.
-        uint32_t st = 0, sph = 0, bs = 0, bph = 0;   // next A stage and B stage, their parities
+        // waits 270 - 500), and one wait serves two items: lanes poll the barriers of
+        // two A stages and their B stages side by side.
+        // Lane l < nsets follows the stages of producer set l (index and parity of
+        // the next one); lane 5 polls a round's second B stage.
+        uint32_t s0 = 0, bs = 0, bph = 0;       // next item's set; next B stage, its parity
+        uint32_t idx = (uint32_t)lane % (uint32_t)nsets, ph = 0;
+        auto advance = [&]() {                  // a set's lane: one stage on
+            if ((idx += (uint32_t)nsets) >= (uint32_t)nS) {
+                idx -= (uint32_t)nS;
+                ph ^= 1u;
+            }
+        };
         uint32_t slot = 0, aph = 1;             // accumulator slot, its reads' parity
         const uint64_t desc = tc::desc_sw128(0);
         const uint32_t alo = tc::smem_addr(A_base) >> 4, blo = tc::smem_addr(B_base) >> 4;
-        const uint32_t hlo = tc::smem_addr(H_base) >> 4;
         const uint32_t bstep = (uint32_t)(b_slot >> 4);
         auto four = [&](uint32_t acc, uint32_t a, uint32_t bb, uint32_t idesc, uint32_t accum) {
             const uint64_t ad = desc | a, bd = desc | bb;
@@ -874,97 +858,76 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                 tc::fence_after_sync();
                 go = go && __all_sync(0xFFFFFFFFu, *err == 0);
                 // Rounds of two items: a chunk of both tiles, or two chunks of one
-                // (the last may be one chunk alone).  Lanes 0 and 1 follow the
-                // round's A stages, 2 and 3 its B stages (lanes above 3 as lane
-                // 0): index, parity, step, limit, so that a round costs few
-                // instructions.
+                // (the last may be one chunk alone).
                 const uint32_t nb = (uint32_t)(kPair / m);      // B stages of a round
                 const int rounds = (C + (int)nb - 1) / (int)nb;
-                const bool isb = lane == 2 || lane == 3;
-                const uint32_t lim = isb ? (uint32_t)nB : (uint32_t)nS;
-                const uint32_t step = isb ? nb : 2u;
-                uint64_t* ring = isb ? b_full : a_full;
-                uint32_t idx = isb ? bs : st, ph = isb ? bph : sph;
-                if (lane == 1 || (lane == 3 && nb == 2)) ++idx;
-                if (idx >= lim) {
-                    idx -= lim;
-                    ph ^= 1u;
-                }
                 for (int rd = 0; rd < rounds && go; ++rd) {
                     const bool two = m == kPair || 2 * rd + 1 < C;
-                    if (!two) {        // nothing comes for lanes 1 and 3
-                        idx = __shfl_sync(0xFFFFFFFFu, idx, lane & 2);
-                        ph = __shfl_sync(0xFFFFFFFFu, ph, lane & 2);
-                        if (lane > 3) idx = st, ph = sph;
+                    const uint32_t s1 = s0 + 1 == (uint32_t)nsets ? 0 : s0 + 1;
+                    const uint32_t bs1 = nb == 1 ? bs : bs + 1 == (uint32_t)nB ? 0 : bs + 1;
+                    const bool item = (uint32_t)lane == s0 || (two && (uint32_t)lane == s1);
+                    uint32_t a0 = __shfl_sync(0xFFFFFFFFu, idx, (int)s0);
+                    uint32_t a1 = __shfl_sync(0xFFFFFFFFu, idx, (int)s1);
+                    // (lanes without a barrier of their own poll the first B stage's)
+                    uint64_t* bar = item ? a_full + idx : b_full + bs;
+                    uint32_t par = item ? ph : bph;
+                    if (lane == 5 && two && nb == 2) {
+                        bar = b_full + bs1;
+                        par = bs1 ? bph : bph ^ 1u;
                     }
-                    go = tc::mbar_wait_warp(ring + idx, ph, kWaitLimit);
-                    // each of lanes 0 - 3 has seen one of the round's barriers complete:
-                    // the lane that issues takes over what all four have seen
+                    go = tc::mbar_wait_warp(bar, par, kWaitLimit);
+                    // each of the lanes has seen one of the round's barriers complete:
+                    // the lane that issues takes over what all of them have seen
                     __syncwarp();
                     tc::fence_after_sync();
                     if (!go) break;
-                    const int hq = planes && lane < 2
-                                       ? reinterpret_cast<volatile int32_t*>(stage_hi)[idx]
-                                       : 0;
-                    idx += step;
-                    if (idx >= lim) {
-                        idx -= lim;
-                        ph ^= 1u;
-                    }
-                    const uint32_t st1 = st + 1 == (uint32_t)nS ? 0 : st + 1;
-                    const uint32_t bs1 = nb == 1 ? bs : bs + 1 == (uint32_t)nB ? 0 : bs + 1;
+                    const int hq =
+                        planes && item ? reinterpret_cast<volatile int32_t*>(stage_hi)[idx] : 0;
+                    if (item) advance();
                     if (two && !(planes && __any_sync(0xFFFFFFFFu, hq != 0))) {
                         if (tc::elect_one()) {
-                            four(acc[0], alo + st * (kStageBytes >> 4), blo + bs * bstep, idesc,
+                            four(acc[0], alo + a0 * (kStageBytes >> 4), blo + bs * bstep, idesc,
                                  rd != 0);
-                            tc::mma_commit(&stage_free[st]);
+                            tc::mma_commit(&stage_free[a0]);
                             if (nb == 2) tc::mma_commit(&b_free[bs]);
-                            four(acc[1], alo + st1 * (kStageBytes >> 4), blo + bs1 * bstep, idesc,
+                            four(acc[1], alo + a1 * (kStageBytes >> 4), blo + bs1 * bstep, idesc,
                                  (rd != 0) | (nb - 1u));
-                            tc::mma_commit(&stage_free[st1]);
+                            tc::mma_commit(&stage_free[a1]);
                             tc::mma_commit(&b_free[bs1]);
                         }
                         __syncwarp();
                     } else {
-                        // one item, or one with a second plane
+                        // one item, or one with a second plane (its set's next stage)
 #pragma unroll 1
                         for (uint32_t x = 0; x < (two ? 2u : 1u) && go; ++x) {
-                            const uint32_t sx = x ? st1 : st, bx = x ? bs1 : bs;
+                            const uint32_t sx = x ? s1 : s0, bx = x ? bs1 : bs;
                             const uint32_t ax = x ? acc[1] : acc[0];
-                            const int h = __shfl_sync(0xFFFFFFFFu, hq, (int)x);
                             if (tc::elect_one()) {
-                                four(ax, alo + sx * (kStageBytes >> 4), blo + bx * bstep, idesc,
+                                const uint32_t a = x ? a1 : a0;
+                                four(ax, alo + a * (kStageBytes >> 4), blo + bx * bstep, idesc,
                                      (rd != 0) | (x & (nb - 1u)));
-                                tc::mma_commit(&stage_free[sx]);
+                                tc::mma_commit(&stage_free[a]);
                             }
                             __syncwarp();
-                            if (h) {
-                                const uint32_t hs = (uint32_t)(h - 1) % kHiStages;
-                                go = tc::mbar_wait_warp(&hi_full[hs],
-                                                        ((uint32_t)(h - 1) / kHiStages) & 1u,
+                            if (__shfl_sync(0xFFFFFFFFu, hq, (int)sx)) {
+                                const uint32_t a = __shfl_sync(0xFFFFFFFFu, idx, (int)sx);
+                                go = tc::mbar_wait_warp(a_full + a,
+                                                        __shfl_sync(0xFFFFFFFFu, ph, (int)sx),
                                                         kWaitLimit);
                                 tc::fence_after_sync();
                                 if (go && tc::elect_one()) {
-                                    four(ax, hlo + hs * (kStageBytes >> 4), blo + bx * bstep,
+                                    four(ax, alo + a * (kStageBytes >> 4), blo + bx * bstep,
                                          idesc, 1u);
-                                    tc::mma_commit(&hi_used[hs]);
+                                    tc::mma_commit(&stage_free[a]);
                                 }
                                 __syncwarp();
-                                go = go && tc::mbar_wait_warp(&hi_used[hs],
-                                                              ((uint32_t)(h - 1) / kHiStages) & 1u,
-                                                              kWaitLimit);
-                                __threadfence_block();
-                                if (lane == 0) *hi_done = h;
+                                if ((uint32_t)lane == sx) advance();
                             }
                             if ((nb == 2 || x == 1) && tc::elect_one()) tc::mma_commit(&b_free[bx]);
                             __syncwarp();
                         }
                     }
-                    const uint32_t na = two ? 2u : 1u;
-                    if ((st += na) >= (uint32_t)nS) {
-                        st -= (uint32_t)nS;
-                        sph ^= 1u;
-                    }
+                    if ((s0 += two ? 2u : 1u) >= (uint32_t)nsets) s0 -= (uint32_t)nsets;
                     if ((bs += two ? nb : 1u) >= (uint32_t)nB) {
                         bs -= (uint32_t)nB;
                         bph ^= 1u;

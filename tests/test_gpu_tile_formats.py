@@ -110,6 +110,18 @@ def test_second_planes(P, N, D, K, big):
     check_scores(P, X, K, logtheta, EPS)
 
 
+@pytest.mark.parametrize("N", [700, 38989])
+@pytest.mark.parametrize("density", [0.33, 0.5, 0.9])
+def test_second_planes_of_long_segments(P, N, density):
+    """Segments so long that a producer set has one stage (four sets, then two) or two sets
+    have two: the second plane takes the set's next stage, or the same one again."""
+    rng = np.random.default_rng([N, int(100 * density)])
+    D, K = 140, 40
+    X = sparse(N, D, density, rng, big=N)
+    logtheta = np.log(rng.dirichlet(np.full(D, 0.3), size=3 * K) + 1e-30)
+    check_scores(P, X, K, logtheta, EPS)
+
+
 @pytest.mark.parametrize("N,D,K", [(300, 200, 5), (20001, 130, 40)])
 def test_log_theta_of_any_size(P, N, D, K):
     """A log theta of -1e6 (a hopeless gene of one row) beside ordinary ones, counts

@@ -130,30 +130,57 @@ __global__ void k_open_slot(const __grid_constant__ Tab tab) {
 // candidate (open = 1) the alpha entry of pi is the candidate's weight and
 // there is no remainder entry (log pi_K = -inf).
 //
-// A row is drawn by a cluster of CS blocks, block r taking genes r Dc ..
-// (Dc = D / CS rounded up): the maximum and the sum of the logsumexp cross the
-// cluster through distributed shared memory, in rank order.  One block a row
+// A row is drawn by a cluster of CS blocks.  The sum of the logsumexp is 1,024
+// sums, of the genes u = j mod 1,024 in ascending order, added by warps of 32 and
+// then in order: those of one block of 1,024 threads, so that CS changes no bit of
+// a row.  Block r takes the genes of the sums j = r W .. r W + W - 1 (W = 1,024 /
+// CS): all its threads draw, W of them add, and the maximum and the warps' sums
+// cross the cluster through distributed shared memory.  One block a row
 // left most SMs idle where a chain has few clusters and many genes (19 rows of
-// 32,738 genes: 164 us with one block a row, 43 us with eight); CS comes
-// from D (draw_cluster), so a chain's values do not depend on what it is
-// batched with.
+// 32,738 genes: 164 us with one block a row, 42 us with eight); CS comes
+// from D (draw_cluster).
 constexpr int kDrawCache = 8192;
 // Row stride (in pairs) of the staged table: K rounded up to odd, so that
 // the pairs of one cluster for 32 random genes spread over 16 bank pairs.
 __host__ __device__ __forceinline__ int staged_ld(int K) { return K | 1; }
 
-// A value of every block of the cluster combined in rank order; slot: this
-// block's shared-memory word, rewritten only after another exchange's barrier.
-template <int CS, class Op>
-__device__ __forceinline__ float cluster_combine(float v, float* slot, Op op) {
+// What the blocks of a cluster read of one another.  Each member is rewritten only
+// after the barrier of the other's exchange, which a block passes once it has read.
+struct DrawExchange {
+    float mx;                       // the block's maximum
+    float sum[kDrawThreads / 32];   // its warps' sums
+};
+
+// The largest v of the cluster's blocks.
+template <int CS>
+__device__ __forceinline__ float cluster_max(float v, DrawExchange& ex) {
     if (CS == 1) return v;
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    if (threadIdx.x == 0) *slot = v;
+    if (threadIdx.x == 0) ex.mx = v;
     cl.sync();
-    float r = *cl.map_shared_rank(slot, 0);
+    float r = *cl.map_shared_rank(&ex.mx, 0);
 #pragma unroll
-    for (int i = 1; i < CS; ++i) r = op(r, *cl.map_shared_rank(slot, i));
+    for (int i = 1; i < CS; ++i) r = fmaxf(r, *cl.map_shared_rank(&ex.mx, i));
+    return r;
+}
+
+// The sum of v over the first kDrawThreads / CS threads of every block, in the
+// order of block_reduce_sum over one block that holds them all.
+template <int CS>
+__device__ __forceinline__ float cluster_sum(float v, float* red, DrawExchange& ex) {
+    if (CS == 1) return block_reduce_sum(v, red);
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    constexpr int warps = kDrawThreads / 32 / CS;
+    v = warp_sum(v);
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (l == 0 && w < warps) ex.sum[w] = v;
+    cl.sync();
+    if (w == 0) red[l] = *cl.map_shared_rank(&ex.sum[l % warps], l / warps);
+    __syncthreads();
+    float r = 0.0f;
+    for (int i = 0; i < kDrawThreads / 32; ++i) r += red[i];
     return r;
 }
 
@@ -161,41 +188,62 @@ __device__ __forceinline__ float cluster_combine(float v, float* slot, Op op) {
 // written to it as [D][K | 1] pairs, the local kernel's shared-memory layout.
 template <int CS>
 __device__ __forceinline__ void draw_row(const ChainArgs& ch, int K, int open, uint32_t theta_tag,
-                                         uint32_t t, int row, float* red, float* lgc, float* cx,
-                                         int rank, float* compact = nullptr) {
+                                         uint32_t t, int row, float* red, float* lgc,
+                                         DrawExchange& ex, int rank, float* compact = nullptr) {
     const int D = ch.D, kmax = ch.kmax;
     const float beta = (float)ch.beta, alpha = (float)ch.alpha;
     const Stream& st = ch.st;
     if (row < 3 * K) {
         const int k = row / 3, p = row % 3;
-        const int Dc = (D + CS - 1) / CS, u0 = min(D, rank * Dc), u1 = min(D, u0 + Dc);
+        // the block's i-th gene: gene_at(i) (from D on: none), of sum i mod W
+        constexpr int W = kDrawThreads / CS;
+        const int n = D > rank * W ? ((D - rank * W - 1) / kDrawThreads + 1) * W : 0;
+        auto gene_at = [&](int i) { return i / W * kDrawThreads + rank * W + i % W; };
         const uint32_t* S0 = ch.Ssub + (size_t)(2 * k) * D;
         const uint32_t* S1 = S0 + D;
         float* Lc = ch.Lc;
         float* Ls = ch.Ls;
-        const bool cached = Dc <= kDrawCache;
+        const bool cached = n <= kDrawCache;
         auto slot = [&](int u) -> float* {
             return p == 0 ? &Lc[(size_t)u * kmax + k] : &Ls[((size_t)u * kmax + k) * 2 + (p - 1)];
         };
         float mx = -CUDART_INF_F;
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
+        for (int i = threadIdx.x; i < n; i += kDrawThreads) {
+            const int u = gene_at(i);
+            if (u >= D) break;
             const uint32_t S = p == 0 ? S0[u] + S1[u] : (p == 1 ? S0[u] : S1[u]);
             const float lg = log_gamma_draw(st, theta_tag, beta + (float)S,
                                             (uint32_t)row * (uint32_t)D + (uint32_t)u, t);
-            if (cached) lgc[u - u0] = lg;
+            if (cached) lgc[i] = lg;
             else *slot(u) = lg;
             mx = fmaxf(mx, lg);
         }
         mx = block_reduce_max(mx, red);   // (its barrier also publishes lgc)
-        mx = cluster_combine<CS>(mx, cx, [](float a, float b) { return fmaxf(a, b); });
+        mx = cluster_max<CS>(mx, ex);
         float s = 0.0f;
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x)
-            s += expf((cached ? lgc[u - u0] : *slot(u)) - mx);
-        s = block_reduce_sum(s, red);
-        s = cluster_combine<CS>(s, cx + 1, [](float a, float b) { return a + b; });
+        if (CS > 1 && 2 * n <= kDrawCache) {
+            // the exponentials by all threads, where the cache has room for them as well
+            // (D <= 32,768; 32,738 genes: 46.4 us without, 42.4 with)
+            for (int i = threadIdx.x; i < n; i += kDrawThreads)
+                lgc[n + i] = gene_at(i) < D ? expf(lgc[i] - mx) : 0.0f;
+            __syncthreads();
+            if (threadIdx.x < W) {
+#pragma unroll 8
+                for (int i = threadIdx.x; i < n; i += W) s += lgc[n + i];
+            }
+        } else if (threadIdx.x < W) {
+#pragma unroll 4
+            for (int i = threadIdx.x; i < n; i += W) {
+                const int u = gene_at(i);
+                if (u < D) s += expf((cached ? lgc[i] : *slot(u)) - mx);
+            }
+        }
+        s = cluster_sum<CS>(s, red, ex);
         const float lse = mx + logf(s);
-        for (int u = u0 + threadIdx.x; u < u1; u += blockDim.x) {
-            const float v = (cached ? lgc[u - u0] : *slot(u)) - lse;
+        for (int i = threadIdx.x; i < n; i += kDrawThreads) {
+            const int u = gene_at(i);
+            if (u >= D) break;
+            const float v = (cached ? lgc[i] : *slot(u)) - lse;
             *slot(u) = v;
             if (compact && p != 0) compact[((size_t)u * staged_ld(K) + k) * 2 + (p - 1)] = v;
         }
@@ -273,7 +321,7 @@ template <class Tab, int CS>
 __global__ void __launch_bounds__(kDrawThreads)
 k_draw_params(const __grid_constant__ Tab tab) {
     __shared__ float red[32];
-    __shared__ float cx[2];
+    __shared__ DrawExchange ex;
     __shared__ __align__(16) float lgc[kDrawCache];   // also the noise split's scratch
     __shared__ int32_t srow[kDrawTable + 1];           // rows before chain b
     __shared__ int32_t sK[kDrawTable], sopen[kDrawTable];
@@ -322,7 +370,7 @@ k_draw_params(const __grid_constant__ Tab tab) {
             const ChainArgs& ch = tab[c];
             const int row = id - srow[c], K = sK[c];
             if (row == 0) first_row(ch, K);
-            draw_row<CS>(ch, K, sopen[c], TAG_THETA, st_[c], row, red, lgc, cx, rank);
+            draw_row<CS>(ch, K, sopen[c], TAG_THETA, st_[c], row, red, lgc, ex, rank);
             __syncthreads();
         }
         const int64_t free0 = total < nblk ? (int64_t)total * CS : 0;
@@ -343,7 +391,7 @@ k_draw_params(const __grid_constant__ Tab tab) {
         for (int64_t id = first; id < base + rows; id += nblk) {
             const int row = (int)(id - base);
             if (row == 0) first_row(ch, K);
-            draw_row<CS>(ch, K, open, TAG_THETA, t, row, red, lgc, cx, rank);
+            draw_row<CS>(ch, K, open, TAG_THETA, t, row, red, lgc, ex, rank);
             __syncthreads();
         }
         base += rows;
@@ -372,7 +420,7 @@ template <class Tab, int CS>
 __global__ void __launch_bounds__(kDrawThreads)
 k_draw_local(const __grid_constant__ Tab tab, int32_t j) {
     __shared__ float red[32];
-    __shared__ float cx[2];
+    __shared__ DrawExchange ex;
     __shared__ float lgc[kDrawCache];
     const uint32_t tag = kLocalTag0 + 2u * (uint32_t)(j - 1);
     const int rank = (int)blockIdx.x % CS, blk = (int)blockIdx.x / CS;
@@ -387,7 +435,7 @@ k_draw_local(const __grid_constant__ Tab tab, int32_t j) {
         for (int64_t id = first; id < base + rows; id += nblk) {
             const int i = (int)(id - base);
             if (i == 0 && rank == 0) clear_accumulators(K, ch.acc_nsub, ch.acc_logq);
-            draw_row<CS>(ch, K, 0, tag, t, 3 * (i >> 1) + 1 + (i & 1), red, lgc, cx, rank,
+            draw_row<CS>(ch, K, 0, tag, t, 3 * (i >> 1) + 1 + (i & 1), red, lgc, ex, rank,
                          ch.local_tab);
             __syncthreads();
         }

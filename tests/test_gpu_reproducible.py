@@ -19,7 +19,11 @@ CASES = {
     "assign_40_large_counts": ("assign", 2501, 700, 40, 50, 3000),
     "assign_3_deep": ("assign", 1300, 3000, 3, 700, 300),
     "draw_2048": ("draw", 900, 2048, 5, 40, 9),
+    "draw_2049": ("draw", 900, 2049, 5, 40, 9),
+    "draw_5003": ("draw", 900, 5003, 5, 40, 9),
+    "draw_9001": ("draw", 900, 9001, 3, 40, 9),
     "draw_32738": ("draw", 900, 32738, 3, 40, 9),
+    "draw_70001": ("draw", 300, 70001, 2, 40, 9),
     "local_5003": ("local", 900, 5003, 5, 40, 9),
     "chain_400": ("chain", 1500, 400, 6, 50, 40),
     "chain_5003": ("chain", 900, 5003, 4, 200, 40),

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "tile_runs.h"
 #include "logml.cuh"
 
 using namespace dpmm;
@@ -708,7 +709,12 @@ int dpmm_init_batch(dpmm_ctx** out, int32_t B, const int32_t* const* indptr,
         c.max_Lslot = std::max(c.max_Lslot, m->c.tile_Lslot);
         tab.push_back(*m->c.h_chain0);
     }
-    for (const ChainArgs& a : tab) c.tile_sumT += a.tile_enabled ? a.tile_T : 0;
+    std::vector<int32_t> tiles;
+    for (const ChainArgs& a : tab) {
+        tiles.push_back(a.tile_enabled ? a.tile_T : 0);
+        c.tile_sumT += tiles.back();
+    }
+    c.label_runs = tile_runs(tiles, c.num_sms, kMaxTileJobs);
     cudaError_t e;
     if ((e = dalloc(&c.gbar_own, 1)) || (e = dalloc(&c.chains_own, (size_t)B)) ||
         (e = cudaMemsetAsync(c.gbar_own, 0, sizeof(GridBar), c.stream)) ||

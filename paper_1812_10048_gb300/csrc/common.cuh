@@ -209,6 +209,7 @@ struct Ctx {
     // batch, its members (each a full context sharing this stream)
     struct ChainArgs* d_chains = nullptr;
     int32_t nchains = 0;
+    std::vector<int32_t> label_runs;        // chains of each label launch (tile_runs.h)
     struct ChainArgs* h_chain0 = nullptr;   // host copy of the single chain (nchains == 1)
     bool tile_any = false;           // some chain of the table has the blocked copy
     int32_t max_Lslot = 0;           // longest segment slot over the chains

@@ -355,8 +355,9 @@ struct TileJob {
     __device__ __forceinline__ bool planes() const { return (k >> 16) & 1u; }
 };
 
-// The jobs of this CTA in chain order (called by the whole block; jobs and
-// scratch, 70 words: shared memory).  A batch's chains are read side by side, one thread each: the roles
+// The jobs of this CTA in chain order (called by the whole block; jobs, at most
+// kMaxTileJobs by the host's choice of runs, and scratch, 70 words: shared memory).
+// A batch's chains are read side by side, one thread each: the roles
 // used to walk the table themselves, three dependent loads a chain for each of
 // them.
 template <class Tab>
@@ -1320,7 +1321,7 @@ int32_t tile_label_stages(const Ctx& c) {
 cudaError_t launch_tile_label(Ctx& c, float* dbg) {
     const int scatter = c.tune_tile_scatter ? c.tune_tile_scatter : kScatterDefault;
     const int32_t stages = tile_label_stages(c);
-    return with_table(c, [&](auto tab) {
+    auto launch = [&](auto tab) {
         using T = decltype(tab);
         const int64_t sm = (int64_t)c.smem_optin;
         if (scatter == 8)
@@ -1333,7 +1334,12 @@ cudaError_t launch_tile_label(Ctx& c, float* dbg) {
             k_assign_tc<T, 12><<<c.num_sms, kTileThreadsP, c.smem_optin, c.stream>>>(
                 tab, dbg, sm, stages);
         return cudaGetLastError();
-    });
+    };
+    if (c.label_runs.size() <= 2) return with_table(c, launch);
+    cudaError_t e = cudaSuccess;
+    for (size_t i = 0; i + 1 < c.label_runs.size() && e == cudaSuccess; ++i)
+        e = launch(TabP{c.d_chains + c.label_runs[i], c.label_runs[i + 1] - c.label_runs[i]});
+    return e;
 }
 
 cudaError_t launch_tile_stats(Ctx& c) {

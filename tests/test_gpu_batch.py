@@ -122,6 +122,29 @@ def test_large_batch_of_small_chains(P):
     batch.close()
 
 
+def test_batch_of_more_chains_than_a_block_lists(P):
+    """600 chains with a tile for every block each, so that one label launch of all would
+    list 600 jobs a block: two launches, the chains on both sides of the cut evolving as
+    alone."""
+    N, D, B = 128 * 152 + 1, 64, 600
+    rng = np.random.default_rng(3)
+    indptr = np.arange(0, 3 * N + 1, 3, dtype=np.int32)
+    col = np.sort(rng.integers(0, 20, size=(N, 3)) + [0, 20, 40], axis=1).astype(np.int32).ravel()
+    ds = [(indptr, col, rng.integers(1, 5, size=3 * N).astype(np.int32), N) for _ in range(B)]
+    batch = P.BatchSampler(ds, D, 1.0, 0.5, kmax=8, seed=5, engine=P.ENGINE_TILE_BF16)
+    batch.step(3)
+    for b in (0, 511, 512, 599):
+        s = P.Sampler(*ds[b][:3], N, D, 1.0, 0.5, kmax=8, seed=5, chain_id=b,
+                      engine=P.ENGINE_TILE_BF16)
+        s.step(3)
+        for x, y in zip(s.get_state(), batch.chain(b).get_state()):
+            np.testing.assert_array_equal(x, y)
+        for x, y in zip(s.stats(), batch.chain(b).stats()):
+            np.testing.assert_array_equal(x, y)
+        s.close()
+    batch.close()
+
+
 @pytest.mark.parametrize("engine", ["auto", "tile"])
 def test_batch_of_degenerate_and_tile_boundary_chains(P, engine):
     """A batch holding a one-cell chain, chains of 127, 128 and 129 cells (the

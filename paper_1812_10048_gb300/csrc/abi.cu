@@ -82,8 +82,10 @@ bool is_host_ptr(const void* p) {
     return a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeUnregistered;
 }
 
-// Device memory of device `dev`.
+// Device memory of device `dev` that its kernels can read as 32-bit words (an
+// address off their boundary can be copied from, not loaded from).
 bool on_this_device(const void* p, int dev) {
+    if (reinterpret_cast<uintptr_t>(p) & 3) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
@@ -409,8 +411,8 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
     // each, a pinned allocation 270 us; thirty of them were 1 ms of a 2 ms start)
     int32_t ends[2] = {0, 0};
     if (is_host_ptr(indptr)) {
-        ends[0] = indptr[0];
-        ends[1] = indptr[N];
+        std::memcpy(&ends[0], indptr, sizeof(int32_t));
+        std::memcpy(&ends[1], indptr + N, sizeof(int32_t));
     } else {
         CKI(cudaMemcpyAsync(&ends[0], indptr, sizeof(int32_t), cudaMemcpyDefault, c.stream));
         CKI(cudaMemcpyAsync(&ends[1], indptr + N, sizeof(int32_t), cudaMemcpyDefault, c.stream));

@@ -207,13 +207,16 @@ extern "C" int dpmm_logml_grad_noalloc(const int32_t* indptr, const int32_t* ind
     p.part = reinterpret_cast<double*>(base + kOffPart);
     p.ticket = reinterpret_cast<int32_t*>(base + kOffTicket);
     // log_beta and grad_log_beta on this device are used where they are, unless
-    // they overlap
+    // they overlap or lie off their words' boundary (which a copy can cross)
+    auto in_place = [&](const float* q) {
+        return (reinterpret_cast<uintptr_t>(q) & 3) == 0 && on_device(q, dev);
+    };
     const float* lb = p.beta_stage;
     float* grad = p.grad;
     if (!e) {
-        if (on_device(grad_log_beta, dev)) grad = grad_log_beta;
+        if (in_place(grad_log_beta)) grad = grad_log_beta;
         const bool apart = log_beta + D <= grad_log_beta || grad_log_beta + D <= log_beta;
-        if (apart && on_device(log_beta, dev)) lb = log_beta;
+        if (apart && in_place(log_beta)) lb = log_beta;
         else
             e = cudaMemcpyAsync(p.beta_stage, log_beta, sizeof(float) * D, cudaMemcpyDefault,
                                 p.stream);

@@ -589,6 +589,66 @@ def test_init_from_device_and_pinned_arrays(P, tiny):
         P.Sampler(dev[0], dev[1], badv, *args, **kw)
 
 
+class OffBoundary:
+    """A host array's values in device memory, one byte past a word's boundary."""
+
+    def __init__(self, a):
+        import torch
+        a = np.ascontiguousarray(a)
+        self.raw = torch.zeros(a.nbytes + 16, dtype=torch.uint8, device="cuda")
+        self.raw[1:1 + a.nbytes] = torch.from_numpy(a.view(np.uint8).reshape(-1)).cuda()
+        self.dtype, self.n = a.dtype, a.nbytes
+
+    def data_ptr(self):
+        return self.raw.data_ptr() + 1
+
+    def is_contiguous(self):
+        return True
+
+    def contiguous(self):
+        return self
+
+    def numpy(self):
+        return self.raw[1:1 + self.n].cpu().numpy().view(self.dtype)
+
+
+def test_init_from_device_arrays_off_their_boundary(P, tiny):
+    """Device arrays at odd addresses are copied, not read where they are: the same chain
+    (each array alone and all of them)."""
+    import torch
+    csr = [tiny.indptr, tiny.indices, tiny.data]
+
+    def states(arrays):
+        torch.cuda.synchronize()
+        s = P.Sampler(*arrays, tiny.N, tiny.D, 1.0, 0.5, seed=5)
+        s.step(3)
+        out = s.get_state(), s.stats()
+        s.close()
+        return out
+    ref = states(csr)
+    for off in ((0,), (1,), (2,), (0, 1, 2)):
+        got = states([OffBoundary(a) if i in off else torch.from_numpy(np.ascontiguousarray(a)).cuda()
+                      for i, a in enumerate(csr)])
+        for r, g in zip(ref, got):
+            for x, y in zip(r, g):
+                np.testing.assert_array_equal(x, y)
+
+
+def test_noalloc_gradient_arrays_off_their_boundary(P, tiny):
+    import torch
+    dev = [torch.from_numpy(np.ascontiguousarray(a.astype(np.int32))).cuda()
+           for a in (tiny.indptr, tiny.indices, tiny.data, tiny.labels)]
+    K = int(tiny.labels.max()) + 1
+    lb = np.linspace(-1.0, 0.5, tiny.D).astype(np.float32)
+    grad = torch.empty(tiny.D, device="cuda")
+    args = (dev[0], dev[1], dev[2], tiny.N, tiny.D, dev[3], K, 0.3)
+    ref = P.dpmm_logml_grad_noalloc(*args, torch.from_numpy(lb).cuda(), grad)
+    odd_lb, odd_grad = OffBoundary(lb), OffBoundary(np.zeros(tiny.D, np.float32))
+    torch.cuda.synchronize()
+    assert P.dpmm_logml_grad_noalloc(*args, odd_lb, odd_grad) == ref
+    np.testing.assert_array_equal(odd_grad.numpy(), grad.cpu().numpy())
+
+
 @pytest.mark.parametrize("engine", ["tile", "csr", "csr_large_k"])
 def test_sum_log_q_is_bit_identical_between_runs(P, tiny, engine):
     """The per-cluster sums of log q are exact integer sums of 2^-32 units, so

@@ -725,6 +725,11 @@ int dpmm_init_batch(dpmm_ctx** out, int32_t B, const int32_t* const* indptr,
         (e = cudaStreamSynchronize(c.stream)))
         return bail(fail(e == cudaErrorMemoryAllocation ? DPMM_ENOMEM : DPMM_ECUDA,
                          "batch table: %s", cudaGetErrorString(e)));
+    if (B == 1) {
+        // (launches over one chain take its table by value)
+        c.h_chain0 = new (std::nothrow) ChainArgs(tab[0]);
+        if (!c.h_chain0) return bail(fail(DPMM_ENOMEM, "host allocation failed"));
+    }
     c.gbar = c.gbar_own;
     c.d_chains = c.chains_own;
     c.nchains = B;

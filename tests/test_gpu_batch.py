@@ -122,6 +122,23 @@ def test_large_batch_of_small_chains(P):
     batch.close()
 
 
+@pytest.mark.parametrize("local_iters", [1, 2])
+def test_batch_of_one(P, local_iters):
+    """One dataset in a batch evolves as alone, through every call on the batch."""
+    ds = datasets()[:1]
+    batch = P.BatchSampler(ds, 300, 1.0, 0.5, kmax=32, seed=9, local_iters=local_iters)
+    single = P.Sampler(*ds[0], 300, 1.0, 0.5, kmax=32, seed=9, chain_id=0,
+                       local_iters=local_iters)
+    for s in (batch, single):
+        s.sweep(2)
+        s.split_merge(1)
+        s.step(4)
+    compare(P, batch, [single], 300)
+    assert batch.plans_applied() == single.plans_applied()
+    single.close()
+    batch.close()
+
+
 def test_batch_of_more_chains_than_a_block_lists(P):
     """600 chains with a tile for every block each, so that one label launch of all would
     list 600 jobs a block: two launches, the chains on both sides of the cut evolving as

@@ -392,9 +392,11 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
 #define CKI(expr)                                                                            \
     do {                                                                                     \
         cudaError_t _e = (expr);                                                             \
-        if (_e != cudaSuccess)                                                               \
+        if (_e != cudaSuccess) {                                                             \
+            cudaGetLastError();   /* (not the next call's) */                                \
             return bail(fail(_e == cudaErrorMemoryAllocation ? DPMM_ENOMEM : DPMM_ECUDA,     \
                              "%s: %s", #expr, cudaGetErrorString(_e)));                      \
+        }                                                                                    \
     } while (0)
 
     CKI(cudaGetDevice(&c.device));
@@ -430,9 +432,11 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
     CsrCheck* d_chk = nullptr;
     int32_t* d_qcount = nullptr;
     long long* d_scan = nullptr;
-    // packed: with the packed entries and, unless the engine is the CSR one, the
-    // blocked copy's arrays (but its entries, whose number is found by counting)
-    auto carve = [&](char* base, bool packed) {
+    // kPacked: with the packed entries and, unless the engine is the CSR one, the
+    // blocked copy's arrays (but its entries, whose number is found by counting);
+    // kCheck: what the checks of the matrix need alone
+    enum Arrays { kCheck, kUnpacked, kPacked };
+    auto carve = [&](char* base, Arrays which) {
         size_t off = 0;
         auto take = [&](auto** p, size_t n) {
             *p = base ? reinterpret_cast<std::remove_reference_t<decltype(*p)>>(base + off)
@@ -440,6 +444,12 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
             off += (std::max<size_t>(1, n) * sizeof(**p) + 255) & ~(size_t)255;
         };
         take(&c.indptr, (size_t)N + 1);
+        take(&d_chk, 1);
+        c.entries = nullptr;
+        c.tile_ptr = nullptr;
+        c.tile_B = nullptr;
+        c.noise = nullptr;
+        if (which == kCheck) return off;
         take(&c.state, (size_t)N);
         take(&c.sc, 1);
         take(&c.nsub, K2);
@@ -463,12 +473,7 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         take(&c.move_ticket, (size_t)c.kmax);
         take(&c.gbar, 1);
         take(&c.d_chains, 1);
-        take(&d_chk, 1);
-        c.entries = nullptr;
-        c.tile_ptr = nullptr;
-        c.tile_B = nullptr;
-        c.noise = nullptr;
-        if (packed) {
+        if (which == kPacked) {
             // padded to a multiple of four entries (zeros) so that 16-byte aligned
             // bulk copies of rows stay inside the allocation
             take(&c.entries, std::max<size_t>(4, ((size_t)nnz + 3) & ~(size_t)3));
@@ -484,17 +489,28 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         }
         return off;
     };
-    auto allocate = [&](bool packed) {
-        cudaError_t e = cudaMalloc((void**)&c.arena, carve(nullptr, packed));
+    auto allocate = [&](Arrays which) {
+        cudaError_t e = cudaMalloc((void**)&c.arena, carve(nullptr, which));
         if (e != cudaSuccess) {
             c.arena = nullptr;
             return e;
         }
-        carve(c.arena, packed);
+        carve(c.arena, which);
         return cudaMemcpyAsync(c.indptr, indptr, sizeof(int32_t) * (N + 1), cudaMemcpyDefault,
                                c.stream);
     };
-    CKI(allocate(D <= 65536));
+    // (a matrix that is malformed, or that cannot be packed after all, is told from one
+    // that does not fit: the arrays then follow the checks)
+    bool arrays = true;
+    {
+        cudaError_t e = allocate(D <= 65536 ? kPacked : kUnpacked);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            arrays = false;
+            e = allocate(kCheck);
+        }
+        CKI(e);
+    }
     // the entries: a caller's arrays on this device are read where they are,
     // others are staged
     const int32_t *s_idx = indices, *s_val = data;
@@ -550,12 +566,13 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
     if (c.packed) {
         if (c.csr_mem) CKI(cudaFree(c.csr_mem));
         c.csr_mem = nullptr;
+        if (!arrays) return bail(fail(DPMM_ENOMEM, "the chain's arrays do not fit device memory"));
     } else {
         // two int32 arrays instead of the packed entries
-        if (c.entries) {
+        if (c.entries || !arrays) {
             CKI(cudaFree(c.arena));
             c.arena = nullptr;
-            CKI(allocate(false));
+            CKI(allocate(kUnpacked));
         }
         if (!c.csr_mem && nnz > 0) CKI(stage());
         c.cols = const_cast<int32_t*>(s_idx);

@@ -589,6 +589,24 @@ def test_init_from_device_and_pinned_arrays(P, tiny):
         P.Sampler(dev[0], dev[1], badv, *args, **kw)
 
 
+def test_malformed_matrix_too_large_for_the_arrays(P):
+    """What is malformed is told even where the chain's arrays (8.8 TB here) would not fit;
+    a sound matrix is then out of memory, and the next call works."""
+    D = 1 << 30
+    indptr, val = np.array([0, 1], np.int32), np.ones(1, np.int32)
+    for idx, x, match in ((D, 1, "column index"), (0, -3, "negative count")):
+        with pytest.raises(P.DpmmError, match=match) as e:
+            P.Sampler(indptr, np.array([idx], np.int32), np.array([x], np.int32), 1, D, 1.0, 0.5,
+                      kmax=1024)
+        assert e.value.code == -1
+    with pytest.raises(P.DpmmError, match="DPMM_ENOMEM"):
+        P.Sampler(indptr, np.zeros(1, np.int32), val, 1, D, 1.0, 0.5, kmax=1024)
+    s = P.Sampler(indptr, np.zeros(1, np.int32), val, 1, 8, 1.0, 0.5)
+    s.step(2)
+    assert s.labels()[1] == 1
+    s.close()
+
+
 class OffBoundary:
     """A host array's values in device memory, one byte past a word's boundary."""
 

@@ -1,12 +1,14 @@
 // C ABI of the library (include/dpmm.h): argument checking, device memory,
 // the sweep / move pipelines and the CUDA graph of dpmm_step.
 #include <curand_kernel.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <type_traits>
@@ -118,7 +120,28 @@ int check_csr(const std::vector<int32_t>& indptr, const std::vector<int32_t>& id
     return DPMM_OK;
 }
 
+// The scalars' mirror in a page of its own that the GPU copies into directly: a
+// read takes 9.1 us instead of 9.8.  Registering and giving back the page take
+// 27 us (a pinned allocation 270), so it comes with the kPinReads-th read, for the
+// programs that go on reading; without one the mirror stays where it is.
+constexpr int32_t kPinReads = 32;
+
+void pin_mirror(Ctx& c) {
+    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    void* p = std::aligned_alloc(page, page);
+    if (p && cudaHostRegister(p, page, cudaHostRegisterDefault) == cudaSuccess) {
+        std::memcpy(p, c.sc_host, sizeof(DevScalars));
+        delete c.sc_host;
+        c.sc_host = static_cast<DevScalars*>(p);
+        c.sc_pinned = true;
+    } else {
+        cudaGetLastError();
+        std::free(p);
+    }
+}
+
 int sync_scalars(Ctx& c) {
+    if (++c.sc_reads == kPinReads) pin_mirror(c);
     CK(cudaMemcpyAsync(c.sc_host, c.sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c.stream));
     CK(cudaStreamSynchronize(c.stream));
     return DPMM_OK;
@@ -132,7 +155,12 @@ void free_ctx(Ctx& c) {
     void* ptrs[] = {c.arena, c.csr_mem, c.tile_ent, c.gbar_own, c.chains_own};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    delete c.sc_host;
+    if (c.sc_pinned) {
+        cudaHostUnregister(c.sc_host);
+        std::free(c.sc_host);
+    } else {
+        delete c.sc_host;
+    }
     delete c.h_chain0;
     c.h_chain0 = nullptr;
     if (c.lml) {

@@ -150,6 +150,8 @@ struct Ctx {
     uint32_t* state = nullptr;    // [N]
     DevScalars* sc = nullptr;     // device scalars
     DevScalars* sc_host = nullptr;  // host mirror for reads
+    bool sc_pinned = false;         // in a registered page (pin_mirror)
+    uint32_t sc_reads = 0;
 
     // statistics: main (current state) and accumulators (being built)
     uint32_t* nsub = nullptr;     // [kmax][2]

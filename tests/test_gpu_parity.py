@@ -607,6 +607,21 @@ def test_malformed_matrix_too_large_for_the_arrays(P):
     s.close()
 
 
+def test_many_reads_between_writes(P, tiny):
+    """The scalars' mirror moves to a registered page on the way (32 reads): K, t and m
+    are the same before and after, and a state set later is the one read."""
+    s = P.Sampler(tiny.indptr, tiny.indices, tiny.data, tiny.N, tiny.D, 1.0, 0.5, seed=5)
+    s.step(3)
+    first = s.get_state()
+    for _ in range(70):
+        assert s.get_state()[2:] == first[2:]
+    s.set_state(np.arange(tiny.N) % 3, np.zeros(tiny.N, np.uint8), 3, 17, 5)
+    assert s.get_state()[2:] == (3, 17, 5)
+    s.step(2)
+    assert s.get_state()[3:] == (19, 7)
+    s.close()
+
+
 class OffBoundary:
     """A host array's values in device memory, one byte past a word's boundary."""
 

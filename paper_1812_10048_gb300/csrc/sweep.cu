@@ -1216,7 +1216,8 @@ __device__ __forceinline__ void assign_cells(const ChainArgs& a, const float* L,
                 }
             }
         }
-        const int c = warp_argmax(best, bestk);
+        int c = warp_argmax(best, bestk);
+        if (c >= K) c = 0;             // every score -inf or a NaN: some cluster of the table
         // eq. 8 with the sweep-start counts minus this cell's own old membership
         const float2 lik = sub_scores(a.csr, beg, end, reinterpret_cast<const float2*>(a.Ls), a.kmax, c, lane);
         if (lane == 0) {

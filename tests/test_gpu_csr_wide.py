@@ -86,3 +86,26 @@ def test_labels_match_fp64(P, N, D, K, kmax, longest, big):
     rows = np.repeat(got_lab, length)
     np.add.at(tot, (rows, idx), val)
     np.testing.assert_array_equal(S2.astype(np.int64).sum(1), tot)
+
+
+@pytest.mark.parametrize("engine", ["csr", "tile"])
+@pytest.mark.parametrize("D,K", [(300, 5), (300, 40), (300, 70), (20001, 5), (20001, 40)])
+@pytest.mark.parametrize("value", [np.nan, -np.inf])
+def test_scores_without_an_order(P, engine, D, K, value):
+    """Parameters that leave a cell no finite score (every form of the label step): it
+    takes cluster 0 of the table, and the statistics follow."""
+    rng = np.random.default_rng(D + K)
+    N = 300
+    idx = np.sort(rng.integers(0, D // 8, size=(N, 8)) + np.arange(8) * (D // 8), axis=1)
+    csr = (np.arange(0, 8 * N + 1, 8, dtype=np.int32), idx.astype(np.int32).ravel(),
+           np.ones(8 * N, np.int32))
+    s = P.Sampler(*csr, N, D, 1.0, 0.5, kmax=80, seed=3,
+                  engine=P.ENGINE_CSR_FP32 if engine == "csr" else P.ENGINE_TILE_BF16)
+    s.set_state(np.arange(N) % K, np.zeros(N, np.uint8), K, 1)
+    P.dpmm_set_params(s.ctx, np.zeros(K + 1, np.float32),
+                      np.full((3 * K, D), value, np.float32))
+    P.dpmm_assign(s.ctx)
+    labels, sub, Kn, _, _ = s.get_state()
+    assert Kn == 1 and not labels.any()
+    assert s.stats()[0].sum() == N and s.stats()[1].sum() == 8 * N
+    s.close()

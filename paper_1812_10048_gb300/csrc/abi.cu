@@ -656,7 +656,6 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         CKI(cudaMemcpyAsync(c.d_chains, c.h_chain0, sizeof(ChainArgs), cudaMemcpyHostToDevice,
                             c.stream));
         c.nchains = 1;
-        c.max_Lslot = c.tile_Lslot;
         c.tile_sumT = c.tile_enabled ? c.tile_T : 0;
     }
     if (c.tile_enabled) CKI(configure_tile(c));
@@ -753,7 +752,6 @@ int dpmm_init_batch(dpmm_ctx** out, int32_t B, const int32_t* const* indptr,
         c.tile_enabled = c.tile_enabled && m->c.tile_enabled;
         c.tile_any = c.tile_any || m->c.tile_enabled;
         if (m->c.tile_enabled) c.tile_C = m->c.tile_C;
-        c.max_Lslot = std::max(c.max_Lslot, m->c.tile_Lslot);
         tab.push_back(*m->c.h_chain0);
     }
     std::vector<int32_t> tiles;

@@ -170,8 +170,6 @@ struct Ctx {
     // move plan
     uint32_t* lmap = nullptr;     // [2 kmax] old (k, r) -> new label | sub mode
     int32_t* desc = nullptr;      // [2 kmax] destination (k, r) <- source descriptor
-    uint32_t* plan_nsub = nullptr;   // [2 kmax]
-    double* plan_sumlogq = nullptr;  // [kmax]
     uint8_t* reinit = nullptr;    // [kmax] new cluster needs fair-coin sub-labels
     int32_t* decide = nullptr;    // [kmax] split decisions / merge pair decisions
     double* log_h = nullptr;      // [kmax]
@@ -214,7 +212,6 @@ struct Ctx {
     std::vector<int32_t> label_runs;        // chains of each label launch (tile_runs.h)
     struct ChainArgs* h_chain0 = nullptr;   // host copy of the single chain (nchains == 1)
     bool tile_any = false;           // some chain of the table has the blocked copy
-    int32_t max_Lslot = 0;           // longest segment slot over the chains
 
     // plan + application kernel (cooperative, one block per SM)
     GridBar* gbar = nullptr;

@@ -1254,54 +1254,6 @@ __device__ __forceinline__ float warp_reduce_scatter(float (&v)[P], int lane, in
     return r;
 }
 
-// Per-lane partial sums of the contraction for P >= K columns: lane takes the
-// row's entries lane, lane + 32, ...; table row u holds the K log theta values
-// (row stride ld, a multiple of 4 when VEC loads float4 from shared memory).
-template <int P, bool VEC>
-__device__ __forceinline__ void lane_partials(const Csr& csr, int64_t beg, int64_t end,
-                                              const float* __restrict__ L, int ld, int K,
-                                              int lane, float (&acc)[P]) {
-#pragma unroll
-    for (int j = 0; j < P; ++j) acc[j] = 0.0f;
-    for (int64_t e = beg + lane; e < end; e += 32) {
-        int32_t u, x;
-        csr.get(e, u, x);
-        const float xf = (float)x;
-        const float* row = L + (size_t)u * ld;
-        if (VEC) {
-#pragma unroll
-            for (int q = 0; q < P / 4; ++q) {
-                if (4 * q < K) {
-                    const float4 l = reinterpret_cast<const float4*>(row)[q];
-                    acc[4 * q] = fmaf(xf, l.x, acc[4 * q]);
-                    acc[4 * q + 1] = fmaf(xf, l.y, acc[4 * q + 1]);
-                    acc[4 * q + 2] = fmaf(xf, l.z, acc[4 * q + 2]);
-                    acc[4 * q + 3] = fmaf(xf, l.w, acc[4 * q + 3]);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < P; ++j)
-                if (j < K) acc[j] = fmaf(xf, row[j], acc[j]);
-        }
-    }
-}
-
-// Sub-cluster likelihood factors of cluster c from a table of float2 rows.
-__device__ __forceinline__ float2 sub_pair(const Csr& csr, int64_t beg, int64_t end,
-                                           const float2* __restrict__ Ls2, int ld, int c,
-                                           int lane) {
-    float t0 = 0.0f, t1 = 0.0f;
-    for (int64_t e = beg + lane; e < end; e += 32) {
-        int32_t u, x;
-        csr.get(e, u, x);
-        const float2 l = Ls2[(size_t)u * ld + c];
-        t0 = fmaf((float)x, l.x, t0);
-        t1 = fmaf((float)x, l.y, t1);
-    }
-    return make_float2(warp_sum(t0), warp_sum(t1));
-}
-
 // K <= 32 with the tables (and, when they fit, the statistics) in shared memory.
 // LPE lanes hold one entry's cluster row (a float4 each), so that a warp takes
 // 32 / LPE entries at a time with one 16-byte load per lane, and entry i of a row
@@ -1920,14 +1872,49 @@ __global__ void k_init_state(uint32_t* __restrict__ state, int64_t N, Stream st)
     }
 }
 
-// Scores of selected cells with the label kernel's own contraction routines
-// (same per-lane order of products and the same reductions).
+// Per-lane partial sums of the contraction for P >= K columns: lane takes the
+// row's entries lane, lane + 32, ...; table row u (stride ld) holds the K log theta
+// values.
+template <int P>
+__device__ __forceinline__ void lane_partials(const Csr& csr, int64_t beg, int64_t end,
+                                              const float* __restrict__ L, int ld, int K,
+                                              int lane, float (&acc)[P]) {
+#pragma unroll
+    for (int j = 0; j < P; ++j) acc[j] = 0.0f;
+    for (int64_t e = beg + lane; e < end; e += 32) {
+        int32_t u, x;
+        csr.get(e, u, x);
+        const float xf = (float)x;
+        const float* row = L + (size_t)u * ld;
+#pragma unroll
+        for (int j = 0; j < P; ++j)
+            if (j < K) acc[j] = fmaf(xf, row[j], acc[j]);
+    }
+}
+
+// Sub-cluster likelihood factors of cluster c from a table of float2 rows.
+__device__ __forceinline__ float2 sub_pair(const Csr& csr, int64_t beg, int64_t end,
+                                           const float2* __restrict__ Ls2, int ld, int c,
+                                           int lane) {
+    float t0 = 0.0f, t1 = 0.0f;
+    for (int64_t e = beg + lane; e < end; e += 32) {
+        int32_t u, x;
+        csr.get(e, u, x);
+        const float2 l = Ls2[(size_t)u * ld + c];
+        t0 = fmaf((float)x, l.x, t0);
+        t1 = fmaf((float)x, l.y, t1);
+    }
+    return make_float2(warp_sum(t0), warp_sum(t1));
+}
+
+// Scores of selected cells: K <= 32 with the CSR label kernel's sums (32 slots in row
+// order, combined in the same order), K > 32 entry after entry.
 template <int P>
 __device__ __forceinline__ void debug_cell_v2(const Csr& csr, int64_t beg, int64_t end,
                                               const float* Lc, int kmax, int K, int lane,
                                               const float* logpi, float* o) {
     float acc[P];
-    lane_partials<P, false>(csr, beg, end, Lc, kmax, K, lane, acc);
+    lane_partials<P>(csr, beg, end, Lc, kmax, K, lane, acc);
     int col;
     const float sc = warp_reduce_scatter<P>(acc, lane, &col);
     if (col < K && (lane & ((32 / P) - 1)) == 0) o[col] = __ldg(logpi + col) + sc;

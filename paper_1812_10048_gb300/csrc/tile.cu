@@ -263,7 +263,7 @@ __device__ __forceinline__ void chain_tiles(int64_t off, int T, int& first, int&
 //               ahead.  The items lie end to end in the ring: a few deep cells
 //               make one segment several times the mean, and slots of that
 //               size left room for fewer A stages (1.3 M x 2,000 with 2% deep
-//               cells: 1,557 us with slots, 1,246 us)
+//               cells: 1,714 us with slots, 1,611 us)
 //   warp 16     lane 0 bulk-copies the B operand of each chunk into its ring
 // The roles that feed the tensor core are alone on their scheduler (w % 4 = 0)
 // but for two epilogue warps: each item costs them the latency of a chain of
@@ -492,8 +492,9 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     auto fit = [&](int sets, int stages) {
         return ring_left(stages, 2) >= max(e_max, 2 * sets * e_mean);
     };
-    // 1.3 M x 2,000, K = 40: four sets of one stage 1,364 us, three of two
-    // 1,288 us; 68,000 x 1,000, K = 10: four sets of two stages 37 us, three 41.
+    // Four sets of two stages against three: 68,000 x 1,000, K = 10 44 and 48 us,
+    // 1.3 M x 2,000, K = 40 1,611 and 1,711; three of two against four of one:
+    // 24 datasets 81 and 95.
     int nsets = 2, nS = 2;
     if (fit(4, 8)) nsets = 4, nS = 8;
     else if (fit(3, 6)) nsets = 3, nS = 6;
@@ -506,8 +507,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     // items in the ring at most: as many as it nearly always has room for, so
     // that a round seldom waits for more than its own slots
     // (fixed slots for the longest segment where two a set fit: a round of the
-    // loader is shorter then; 68,000 x 1,000 39 -> 35 us, 8,000 x 32,738
-    // 191 -> 172 us, while the ring gives 89 -> 76 us for 24 datasets)
+    // loader is shorter then; 68,000 x 1,000 44.3 us, 45.7 in the ring)
     const bool fixed = e_ring >= 2 * nsets * e_max;
     const int e_item = fixed ? e_max : e_mean + e_mean / 4;
     const int nE = min(kMaxESlots / nsets, max(2, e_ring / (e_item * nsets))) * nsets;

@@ -1,7 +1,7 @@
 """Cluster statistics of the log ML counted in shared memory: sizes around the
 kernel's edges (one or several cluster groups, rows longer than a warp's batch,
 ragged flush tails, empty rows and clusters), totals of 2^32 and more, and the
-short lgamma forms over the range of beta, against the FP64 oracle."""
+range of beta, against the FP64 oracle."""
 
 import numpy as np
 import pytest
@@ -89,7 +89,7 @@ def test_total_of_2_to_32_without_a_wrapped_gene(P):
 
 @pytest.mark.parametrize("log_beta", [-60.0, -20.0, -2.0, 0.0, 2.7, 9.0, 30.0])
 def test_lgamma_forms_over_beta(P, log_beta):
-    """Counts on both sides of the product / Stirling line at every beta."""
+    """Small and large counts at beta from 1e-26 to 1e13."""
     rng = np.random.default_rng(3)
     D, K = 24, 2
     val = np.concatenate([np.arange(1, D + 1), 2 ** np.arange(D) % 65521 + 1]).astype(np.int32)

@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -307,16 +309,16 @@ __device__ __forceinline__ uint16_t digit_bits(uint32_t v) {
 }
 
 // One producer warp's share of a staged segment into its quarter q of the A stage
-// (kHi: the hi digits, else the lo ones): the 16-byte groups that hold entries
+// (kPlanes 1: the lo digits into A, 2: the hi ones into H, 3: both): the 16-byte groups that hold entries
 // [i0, i1), kScatter entries per lane in flight.  A group at either end may hold
 // entries of a neighbouring quarter, which their rows tell apart, and the
 // segment's padding, whose counts are 0.  An entry row << 22 | gene << 16 | count
 // shifted right by 15 has its row and gene at the bytes row * 128 + gene * 2 of
 // the stage; the 128-byte swizzle exchanges bits 4-6 with the row's low bits.
-template <bool kHi, int kScatter>
+template <int kPlanes, int kScatter>
 __device__ __forceinline__ void scatter_entries(const uint32_t* ring, int i0, int i1, int q,
-                                                int lane, unsigned char* A) {
-    constexpr uint32_t mask = kHi ? 0xFF00u : 0xFFu;
+                                                int lane, unsigned char* A, unsigned char* H) {
+    constexpr uint32_t mask = kPlanes == 1 ? 0xFFu : kPlanes == 2 ? 0xFF00u : 0xFFFFu;
     constexpr int U = kScatter / 4;
     const uint4* ring4 = reinterpret_cast<const uint4*>(ring);
     const int j1 = (i1 + 3) >> 2;
@@ -331,9 +333,13 @@ __device__ __forceinline__ void scatter_entries(const uint32_t* ring, int i0, in
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const uint32_t x = e[k] & mask, t = e[k] >> 15;
-                if (x && (e[k] >> 27) == (uint32_t)q)
-                    *reinterpret_cast<uint16_t*>(A + ((t & 0x3FFEu) ^ ((t >> 3) & 0x70u))) =
-                        digit_bits(x);
+                if (x && (e[k] >> 27) == (uint32_t)q) {
+                    const uint32_t at = (t & 0x3FFEu) ^ ((t >> 3) & 0x70u);
+                    if (kPlanes & 1)
+                        *reinterpret_cast<uint16_t*>(A + at) = digit_bits(x & 0xFFu);
+                    if (kPlanes == 2 || (kPlanes == 3 && x > 0xFFu))
+                        *reinterpret_cast<uint16_t*>(H + at) = digit_bits(x & 0xFF00u);
+                }
             }
         }
     }
@@ -504,6 +510,13 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
     int nB = 2;
     while (nB < kMaxBStages && ring_left(nS, nB + 1) >= max(e_max, 12 * e_mean)) ++nB;
     const int e_ring = ring_left(nS, nB) & ~15;
+    // An item's two planes filled and multiplied together, where every set of four has
+    // two stages and an item's MMAs are short (N <= 128 columns: the MMA warp's waits
+    // are what an item costs); else the second plane follows the first.  68,000 x 1,000,
+    // libraries of 8,000: K = 5 67 -> 55 us, K = 20 (N = 128) 70 -> 60; K = 40 (N = 240)
+    // 87 us one after the other, 90 together, 1.3 M x 2,000 1,611 and 1,743.  For a
+    // batch one after the other: 24 datasets 80 us, 85 together.
+    const bool both = std::is_same<Tab, TabV>::value && nsets == 4 && nS == 8 && ntot_max <= 128;
     // items in the ring at most: as many as it nearly always has room for, so
     // that a round seldom waits for more than its own slots
     // (fixed slots for the longest segment where two a set fit: a round of the
@@ -583,6 +596,12 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         uint32_t st = (uint32_t)set % (uint32_t)nS, sph = 1u;   // parity of the stage's last use
         uint32_t es = (uint32_t)set % (uint32_t)nE, eph = 0u;
         uint32_t g = set < nsets ? (uint32_t)set : total;
+        auto next_stage = [&]() {
+            if ((st += (uint32_t)nsets) >= (uint32_t)nS) {
+                st -= (uint32_t)nS;
+                sph ^= 1u;
+            }
+        };
         bool ok = true;
         for (; g < total && ok; g += (uint32_t)nsets) {
             int i0 = 0, i1 = 0, hi = 0;
@@ -591,8 +610,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
             // its hi digits in the set's next stage, a stage like any other: the MMA
             // warp goes on to other items while it fills.  (Stages of its own that the
             // MMA warp had to drain before they were used again: 68,000 x 1,000 step
-            // 96 -> 89 us, 1.3 M x 2,000 2,430 -> 2,260 us; both planes written in one
-            // pass over the entries: label kernel 46.5 us, 44.2 so.)
+            // 96 -> 89 us, 1.3 M x 2,000 2,430 -> 2,260 us.)
             for (int pl = 0; pl <= hi; ++pl) {
                 unsigned char* A = A_base + st * kStageBytes;
                 // (at a stage's first use the parity of the phase before the first)
@@ -613,9 +631,34 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                     i1 = q == 0 ? mt.x : q == 1 ? mt.y : q == 2 ? mt.z : mt.w;
                     if (planes_any) hi = meta_hi[es];
                     ring = reinterpret_cast<const uint32_t*>(E_base + slot_off[es]);
-                    scatter_entries<false, kScatter>(ring, i0, i1, q, lane, A);
+                    if (both && hi) {
+                        // both planes at once; the second stage is full when the first is
+                        const uint32_t st1 = st;
+                        next_stage();
+                        ok = tc::mbar_wait(&stage_free[st], sph, kWaitLimit);
+                        const bool mine2 = ok;
+                        ok = __all_sync(0xFFFFFFFFu, ok && *err == 0);
+                        if (!ok) {
+                            if (lane == 0 && !mine2) *err = DPMM_ETIMEOUT;
+                            break;
+                        }
+                        unsigned char* H = A_base + st * kStageBytes;
+                        clear_quarter(H, q, lane);
+                        scatter_entries<3, kScatter>(ring, i0, i1, q, lane, A, H);
+                        tc::fence_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (q == 0) stage_hi[st1] = hi;
+                            tc::mbar_arrive(&a_full[st]);
+                            tc::mbar_arrive(&a_full[st1]);
+                            tc::mbar_arrive(&ent_free[es]);
+                        }
+                        next_stage();
+                        break;
+                    }
+                    scatter_entries<1, kScatter>(ring, i0, i1, q, lane, A, nullptr);
                 } else {
-                    scatter_entries<true, kScatter>(ring, i0, i1, q, lane, A);
+                    scatter_entries<2, kScatter>(ring, i0, i1, q, lane, nullptr, A);
                 }
                 tc::fence_async_smem();
                 __syncwarp();
@@ -624,10 +667,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                     tc::mbar_arrive(&a_full[st]);
                     if (pl == hi) tc::mbar_arrive(&ent_free[es]);
                 }
-                if ((st += (uint32_t)nsets) >= (uint32_t)nS) {
-                    st -= (uint32_t)nS;
-                    sph ^= 1u;
-                }
+                next_stage();
             }
             if ((es += (uint32_t)nsets) >= (uint32_t)nE) {
                 es -= (uint32_t)nE;
@@ -882,10 +922,13 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                     __syncwarp();
                     tc::fence_after_sync();
                     if (!go) break;
-                    const int hq =
-                        planes && item ? reinterpret_cast<volatile int32_t*>(stage_hi)[idx] : 0;
+                    const unsigned hq =
+                        planes ? __ballot_sync(0xFFFFFFFFu,
+                                               item && reinterpret_cast<volatile int32_t*>(
+                                                           stage_hi)[idx])
+                               : 0u;
                     if (item) advance();
-                    if (two && !(planes && __any_sync(0xFFFFFFFFu, hq != 0))) {
+                    if (two && !hq) {
                         if (tc::elect_one()) {
                             four(acc[0], alo + a0 * (kStageBytes >> 4), blo + bs * bstep, idesc,
                                  rd != 0);
@@ -898,32 +941,39 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                         }
                         __syncwarp();
                     } else {
-                        // one item, or one with a second plane (its set's next stage)
+                        // one item, or some with a second plane: its set's next stage (both:
+                        // full when the first is)
 #pragma unroll 1
                         for (uint32_t x = 0; x < (two ? 2u : 1u) && go; ++x) {
                             const uint32_t sx = x ? s1 : s0, bx = x ? bs1 : bs;
                             const uint32_t ax = x ? acc[1] : acc[0];
+                            const uint32_t a = x ? a1 : a0;
+                            const bool h = (hq >> sx) & 1u;
+                            const uint32_t e = __shfl_sync(0xFFFFFFFFu, idx, (int)sx);
                             if (tc::elect_one()) {
-                                const uint32_t a = x ? a1 : a0;
                                 four(ax, alo + a * (kStageBytes >> 4), blo + bx * bstep, idesc,
                                      (rd != 0) | (x & (nb - 1u)));
                                 tc::mma_commit(&stage_free[a]);
+                                if (h && both) {
+                                    four(ax, alo + e * (kStageBytes >> 4), blo + bx * bstep,
+                                         idesc, 1u);
+                                    tc::mma_commit(&stage_free[e]);
+                                }
                             }
                             __syncwarp();
-                            if (__shfl_sync(0xFFFFFFFFu, hq, (int)sx)) {
-                                const uint32_t a = __shfl_sync(0xFFFFFFFFu, idx, (int)sx);
-                                go = tc::mbar_wait_warp(a_full + a,
+                            if (h && !both) {
+                                go = tc::mbar_wait_warp(a_full + e,
                                                         __shfl_sync(0xFFFFFFFFu, ph, (int)sx),
                                                         kWaitLimit);
                                 tc::fence_after_sync();
                                 if (go && tc::elect_one()) {
-                                    four(ax, alo + a * (kStageBytes >> 4), blo + bx * bstep,
+                                    four(ax, alo + e * (kStageBytes >> 4), blo + bx * bstep,
                                          idesc, 1u);
-                                    tc::mma_commit(&stage_free[a]);
+                                    tc::mma_commit(&stage_free[e]);
                                 }
                                 __syncwarp();
-                                if ((uint32_t)lane == sx) advance();
                             }
+                            if (h && (uint32_t)lane == sx) advance();
                             if ((nb == 2 || x == 1) && tc::elect_one()) tc::mma_commit(&b_free[bx]);
                             __syncwarp();
                         }

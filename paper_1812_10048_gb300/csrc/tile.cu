@@ -309,8 +309,9 @@ __device__ __forceinline__ uint16_t digit_bits(uint32_t v) {
 }
 
 // One producer warp's share of a staged segment into its quarter q of the A stage
-// (kPlanes 1: the lo digits into A, 2: the hi ones into H, 3: both): the 16-byte groups that hold entries
-// [i0, i1), kScatter entries per lane in flight.  A group at either end may hold
+// (kPlanes 1: the lo digits into A, 2: the hi ones into H, 3: both): the 16-byte
+// groups that hold entries [i0, i1), kScatter entries per lane in flight.  A group at
+// either end may hold
 // entries of a neighbouring quarter, which their rows tell apart, and the
 // segment's padding, whose counts are 0.  An entry row << 22 | gene << 16 | count
 // shifted right by 15 has its row and gene at the bytes row * 128 + gene * 2 of
@@ -676,65 +677,121 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
         }
     } else if (warp == kELoadWarp) {
         // ---------------- segment loader ----------------
-        uint32_t g = 0;        // items started (slot sequence)
-        uint32_t es = (uint32_t)lane % (uint32_t)nE, eph = 0;   // this lane's slot, its use's parity
-        uint32_t tail = 0;     // oldest item that may still be in the ring
-        int32_t head = 0;      // the ring's next free byte (the items lie between)
-        bool stop_l = false;
-        for (int jn = 0; jn < njobs && !stop_l; ++jn) {
-            const TileJob job = jobs[jn];
-            const ChainArgs& ch = tab[job.b];
-            const int first = job.first, cnt = job.cnt;
+        // the five quarter pointers of a job's item j and (last) its second-plane flag
+        auto seg_ptrs = [&](const TileJob& job, uint32_t j, int32_t (&p)[6]) {
             const uint32_t Cu = (uint32_t)C;
-            const uint32_t nitem = (uint32_t)cnt * Cu;
-            // lane l < nsets takes the items l, l + nsets, ...: their five
-            // quarter pointers, read one round ahead
-            auto seg_ptrs = [&](uint32_t j, int32_t (&p)[6]) {
+            const uint32_t pr = j / (kPair * Cu);          // pair, then chunk, then tile
+            const uint32_t m = min((uint32_t)kPair, (uint32_t)job.cnt - kPair * pr);
+            const uint32_t r = j - pr * kPair * Cu, ci = r / m;
+            const int64_t sgm =
+                ((int64_t)job.first + (int64_t)(kPair * pr + (r - ci * m)) * gridDim.x) *
+                    (int64_t)Cu + ci;
+            const int32_t* ptr = tab[job.b].tile_ptr + 4 * sgm;
 #pragma unroll
-                for (int k = 0; k < 6; ++k) p[k] = 0;
-                if (lane < nsets && j < nitem) {
-                    const uint32_t pr = j / (kPair * Cu);          // pair, then chunk, then tile
-                    const uint32_t m = min((uint32_t)kPair, (uint32_t)cnt - kPair * pr);
-                    const uint32_t r = j - pr * kPair * Cu, ci = r / m;
-                    const int64_t sgm =
-                        ((int64_t)first + (int64_t)(kPair * pr + (r - ci * m)) * gridDim.x) *
-                            (int64_t)Cu + ci;
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) p[k] = __ldg(ch.tile_ptr + 4 * sgm + k);
-                    // the segment's second-plane flag, then the pointers
-                    p[5] = p[1] < 0;
-                    p[1] &= kTilePtrMask;
-                }
-            };
+            for (int k = 0; k < 5; ++k) p[k] = __ldg(ptr + k);
+            p[5] = p[1] < 0;
+            p[1] &= kTilePtrMask;
+        };
+        // an item's segment into slot es, at byte `at` of the ring
+        auto issue = [&](const uint32_t* ent, const int32_t (&p)[6], uint32_t es, int32_t at) {
+            const int32_t len = p[4] - p[0];
+            slot_off[es] = at;
+            meta[es] = make_int4(p[1] - p[0], p[2] - p[0], p[3] - p[0], len);
+            if (planes_any) meta_hi[es] = p[5];
+            if (len) {
+                tc::mbar_arrive_expect_tx(&ent_full[es], (uint32_t)len * 4u);
+                tc::bulk_g2s(E_base + at, ent + p[0], (uint32_t)len * 4u, &ent_full[es]);
+            } else {
+                tc::mbar_arrive(&ent_full[es]);
+            }
+        };
+        if (fixed) {
+            // Lane l < nsets loads for set l by itself, so that a set that is late
+            // (second planes) keeps no other's entries back: the next item's pointers
+            // are read one item ahead, its slot is polled.  (In rounds of all sets
+            // 68,000 x 1,000, K = 10 44.1 us, 42.7 so; libraries of 1,500, K = 16, a
+            // step 111 and 109.)
+            uint32_t g = lane < nsets ? (uint32_t)lane : total;     // next item
+            uint32_t es = (uint32_t)lane, eph = 0, n = 0;           // its slot; items started
+            int jn = -1;                                            // its job, whose items are
+            uint32_t j0 = 0, jend = 0;                              // j0 .. jend - 1
             int32_t cur[6], nxt[6];
-            seg_ptrs((uint32_t)lane, cur);
-            for (uint32_t jb = 0; jb < nitem; jb += (uint32_t)nsets) {
-                seg_ptrs(jb + (uint32_t)nsets + (uint32_t)lane, nxt);
-                const uint32_t n = min((uint32_t)nsets, nitem - jb);
-                const int32_t len = cur[4] - cur[0];
-                const int32_t room = (uint32_t)lane < n ? max(len, 4) * 4 : 0;   // ring bytes
-                auto issue = [&](int32_t at) {
-                    slot_off[es] = at;
-                    meta[es] = make_int4(cur[1] - cur[0], cur[2] - cur[0], cur[3] - cur[0], len);
-                    if (planes_any) meta_hi[es] = cur[5];
-                    if (len) {
-                        tc::mbar_arrive_expect_tx(&ent_full[es], (uint32_t)len * 4u);
-                        tc::bulk_g2s(E_base + at, ch.tile_ent + cur[0], (uint32_t)len * 4u,
-                                     &ent_full[es]);
-                    } else {
-                        tc::mbar_arrive(&ent_full[es]);
+            auto fetch = [&](uint32_t item, int32_t (&p)[6]) {
+                while (item >= jend && jn + 1 < njobs) {
+                    j0 = jend;
+                    jend += (uint32_t)jobs[++jn].cnt * (uint32_t)C;
+                }
+                if (item < total) seg_ptrs(jobs[jn], item - j0, p);
+            };
+            int jcur = 0;
+            if (g < total) {
+                fetch(g, cur);
+                jcur = jn;
+                fetch(g + (uint32_t)nsets, nxt);
+            }
+            const uint32_t* ent = tab[jobs[jcur].b].tile_ent;
+            uint32_t polls = 0;
+            while (__any_sync(0xFFFFFFFFu, g < total)) {
+                const bool ready = g < total && tc::mbar_test(&ent_free[es], eph ^ 1u);
+                if (ready) {
+                    issue(ent, cur, es, (int32_t)(es * (uint32_t)e_max));
+                    ++n;
+                    g += (uint32_t)nsets;
+                    if ((es += (uint32_t)nsets) >= (uint32_t)nE) {
+                        es -= (uint32_t)nE;
+                        eph ^= 1u;
                     }
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) cur[k] = nxt[k];
+                    if (jn != jcur) {
+                        jcur = jn;
+                        ent = tab[jobs[jn].b].tile_ent;
+                    }
+                    fetch(g + (uint32_t)nsets, nxt);
+                }
+                polls = __any_sync(0xFFFFFFFFu, ready) ? 0u : polls + 1u;
+                if (polls >= kWaitLimit || __any_sync(0xFFFFFFFFu, *err != 0)) {
+                    if (lane == 0 && *err == 0) *err = DPMM_ETIMEOUT;
+                    break;
+                }
+            }
+            // every started copy has landed before the block can exit
+            const uint32_t per = (uint32_t)(nE / nsets);
+            for (uint32_t q = n > per ? n - per : 0u; q < n; ++q)
+                tc::mbar_wait(&ent_full[(uint32_t)lane + (uint32_t)nsets * (q % per)],
+                              (q / per) & 1u, kWaitLimit);
+            __syncwarp();
+        } else {
+            uint32_t g = 0;        // items started (slot sequence)
+            uint32_t es = (uint32_t)lane % (uint32_t)nE, eph = 0;   // this lane's slot, its use's parity
+            uint32_t tail = 0;     // oldest item that may still be in the ring
+            int32_t head = 0;      // the ring's next free byte (the items lie between)
+            bool stop_l = false;
+            for (int jn = 0; jn < njobs && !stop_l; ++jn) {
+                const TileJob job = jobs[jn];
+                const uint32_t* ent = tab[job.b].tile_ent;
+                const uint32_t nitem = (uint32_t)job.cnt * (uint32_t)C;
+                // lane l < nsets takes the items l, l + nsets, ...: their pointers, read
+                // one round ahead
+                auto ptrs = [&](uint32_t j, int32_t (&p)[6]) {
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) p[k] = 0;
+                    if (lane < nsets && j < nitem) seg_ptrs(job, j, p);
                 };
-                // the slots' previous items have been consumed (a lane each; at a
-                // slot's first use the parity of the phase before the first)
-                bool ok = (uint32_t)lane >= n || tc::mbar_wait(&ent_free[es], eph ^ 1u, kWaitLimit);
-                ok = __all_sync(0xFFFFFFFFu, ok && *err == 0);
-                // a lane's copy may land where the item of another lane's slot lay: each
-                // lane takes over what the others have seen consumed
-                __syncwarp();
-                if (fixed) {
-                    if (ok && (uint32_t)lane < n) issue((int32_t)(es * (uint32_t)e_max));
-                } else {
+                int32_t cur[6], nxt[6];
+                ptrs((uint32_t)lane, cur);
+                for (uint32_t jb = 0; jb < nitem; jb += (uint32_t)nsets) {
+                    ptrs(jb + (uint32_t)nsets + (uint32_t)lane, nxt);
+                    const uint32_t n = min((uint32_t)nsets, nitem - jb);
+                    const int32_t len = cur[4] - cur[0];
+                    const int32_t room = (uint32_t)lane < n ? max(len, 4) * 4 : 0;   // ring bytes
+                    // the slots' previous items have been consumed (a lane each; at a
+                    // slot's first use the parity of the phase before the first)
+                    bool ok = (uint32_t)lane >= n || tc::mbar_wait(&ent_free[es], eph ^ 1u, kWaitLimit);
+                    ok = __all_sync(0xFFFFFFFFu, ok && *err == 0);
+                    // a lane's copy may land where the item of another lane's slot lay: each
+                    // lane takes over what the others have seen consumed
+                    __syncwarp();
                     if (g + n > tail + (uint32_t)nE) tail = g + n - (uint32_t)nE;
                     // the round's items side by side when the ring has room for all
                     int32_t off = room;
@@ -748,7 +805,7 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                     if (tail == g) head = 0;
                     int32_t toff = tail == g ? -1 : slot_off[tail % (uint32_t)nE];
                     if (ok && (head > toff ? (int32_t)e_ring - head : toff - head) >= all) {
-                        if ((uint32_t)lane < n) issue(head + off);
+                        if ((uint32_t)lane < n) issue(ent, cur, es, head + off);
                         head += all;
                     } else {
                         // one after the other, wrapping, and waiting for the oldest
@@ -777,34 +834,34 @@ k_assign_tc(const __grid_constant__ Tab tab, float* dbg_out, int64_t smem_bytes,
                                     }
                                 }
                             }
-                            if (ok && (uint32_t)lane == j) issue(at);
+                            if (ok && (uint32_t)lane == j) issue(ent, cur, es, at);
                             head = at + need;
                             __syncwarp();
                         }
                     }
-                }
-                if (!ok) {
-                    if (lane == 0) *err = DPMM_ETIMEOUT;
-                    stop_l = true;
-                    break;
-                }
-                __syncwarp();
-                if ((es += n) >= (uint32_t)nE) {
-                    es -= (uint32_t)nE;
-                    eph ^= 1u;
-                }
-                g += n;
+                    if (!ok) {
+                        if (lane == 0) *err = DPMM_ETIMEOUT;
+                        stop_l = true;
+                        break;
+                    }
+                    __syncwarp();
+                    if ((es += n) >= (uint32_t)nE) {
+                        es -= (uint32_t)nE;
+                        eph ^= 1u;
+                    }
+                    g += n;
 #pragma unroll
-                for (int k = 0; k < 6; ++k) cur[k] = nxt[k];
+                    for (int k = 0; k < 6; ++k) cur[k] = nxt[k];
+                }
             }
+            // every started copy has landed before the block can exit (after a
+            // timeout perhaps some of the round that was cut short)
+            const uint32_t issued = g + (stop_l ? (uint32_t)nsets : 0u);
+            if (lane == 0)
+                for (uint32_t q = issued > (uint32_t)nE ? issued - (uint32_t)nE : 0u; q < issued; ++q)
+                    tc::mbar_wait(&ent_full[q % (uint32_t)nE], (q / (uint32_t)nE) & 1u,
+                                  stop_l ? kWaitLimit >> 8 : kWaitLimit);
         }
-        // every started copy has landed before the block can exit (after a
-        // timeout perhaps some of the round that was cut short)
-        const uint32_t issued = g + (stop_l ? (uint32_t)nsets : 0u);
-        if (lane == 0)
-            for (uint32_t q = issued > (uint32_t)nE ? issued - (uint32_t)nE : 0u; q < issued; ++q)
-                tc::mbar_wait(&ent_full[q % (uint32_t)nE], (q / (uint32_t)nE) & 1u,
-                              stop_l ? kWaitLimit >> 8 : kWaitLimit);
     } else if (warp == kBLoadWarp) {
         // ---------------- B loader ----------------
         if (lane == 0) {

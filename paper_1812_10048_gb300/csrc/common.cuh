@@ -90,12 +90,13 @@ struct DevScalars {
 
 // The dense-tile engine serves 1 <= K <= kTileMaxK.
 constexpr int kTileMaxK = 40;
-// Engine choice measured on one GB300 (68,000 x 1,000, one sweep from a fixed
-// K-cluster state, densities 5.7% - 22.8%, K = 2 .. 40): the dense-tile engine
-// is faster for every K >= 5 at every density and for K <= 2 below ~12%
-// density; at K <= 2 and density >= kTileDenseCut the CSR engine is (up to 10%)
-// faster.  So the automatic choice takes the tile engine for K >= 3 always and
-// for K <= 2 only below that density.
+// Engine choice of the automatic engine: the dense-tile engine for K >= 3, and for
+// K <= 2 below kTileDenseCut.  Measured on one GB300 (68,000 x 1,000, one sweep from
+// a fixed K-cluster state, densities 5.7% - 22.8%, K = 2 .. 40): the dense-tile
+// engine is faster from K = 10 up at every density (K = 40 at 14%: 0.18 against
+// 0.45 ms), the CSR engine for K = 2 everywhere (by 5 to 16%) and for K = 5 from 14%
+// up (by 1 to 9%).  The line stays where it was drawn with an earlier CSR kernel: the
+// engine is part of what fixes a chain's bits.
 constexpr double kTileDenseCut = 0.12;
 constexpr int kTileDenseKmin = 3;
 

@@ -123,25 +123,29 @@ int check_csr(const std::vector<int32_t>& indptr, const std::vector<int32_t>& id
 // The scalars' mirror in a page of its own that the GPU copies into directly: a
 // read takes 9.1 us instead of 9.8.  Registering and giving back the page take
 // 27 us (a pinned allocation 270), so it comes with the kPinReads-th read, for the
-// programs that go on reading; without one the mirror stays where it is.
-constexpr int32_t kPinReads = 32;
+// programs that go on reading; without one the mirror stays where it is.  The first
+// mirror is kept until the context goes: another thread may be reading it.
+constexpr uint32_t kPinReads = 32;
 
 void pin_mirror(Ctx& c) {
     const size_t page = (size_t)sysconf(_SC_PAGESIZE);
     void* p = std::aligned_alloc(page, page);
+    // (no capture that another thread has under way is broken by the registration)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (p && cudaHostRegister(p, page, cudaHostRegisterDefault) == cudaSuccess) {
         std::memcpy(p, c.sc_host, sizeof(DevScalars));
-        delete c.sc_host;
-        c.sc_host = static_cast<DevScalars*>(p);
-        c.sc_pinned = true;
+        c.sc_pinned = static_cast<DevScalars*>(p);
+        c.sc_host = c.sc_pinned;
     } else {
         cudaGetLastError();
         std::free(p);
     }
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 int sync_scalars(Ctx& c) {
-    if (++c.sc_reads == kPinReads) pin_mirror(c);
+    if (__atomic_add_fetch(&c.sc_reads, 1u, __ATOMIC_RELAXED) == kPinReads) pin_mirror(c);
     CK(cudaMemcpyAsync(c.sc_host, c.sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, c.stream));
     CK(cudaStreamSynchronize(c.stream));
     return DPMM_OK;
@@ -156,11 +160,10 @@ void free_ctx(Ctx& c) {
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c.sc_pinned) {
-        cudaHostUnregister(c.sc_host);
-        std::free(c.sc_host);
-    } else {
-        delete c.sc_host;
+        cudaHostUnregister(c.sc_pinned);
+        std::free(c.sc_pinned);
     }
+    delete c.sc_first;
     delete c.h_chain0;
     c.h_chain0 = nullptr;
     if (c.lml) {
@@ -606,7 +609,7 @@ int dpmm_init(dpmm_ctx** out, const int32_t* indptr, const int32_t* indices, con
         c.cols = const_cast<int32_t*>(s_idx);
         c.counts = const_cast<int32_t*>(s_val);
     }
-    c.sc_host = new (std::nothrow) DevScalars();
+    c.sc_host = c.sc_first = new (std::nothrow) DevScalars();
     if (!c.sc_host) return bail(fail(DPMM_ENOMEM, "host allocation failed"));
     CKI(cudaMemsetAsync(c.move_ticket, 0, sizeof(int32_t) * c.kmax, c.stream));
 

@@ -150,8 +150,9 @@ struct Ctx {
     // chain state
     uint32_t* state = nullptr;    // [N]
     DevScalars* sc = nullptr;     // device scalars
-    DevScalars* sc_host = nullptr;  // host mirror for reads
-    bool sc_pinned = false;         // in a registered page (pin_mirror)
+    DevScalars* sc_host = nullptr;  // host mirror for reads: sc_first, then sc_pinned
+    DevScalars* sc_first = nullptr;
+    DevScalars* sc_pinned = nullptr;   // in a registered page (pin_mirror)
     uint32_t sc_reads = 0;
 
     // statistics: main (current state) and accumulators (being built)
